@@ -52,21 +52,22 @@ constexpr int NWORK = 16;
 // 2k+1 are contiguous and form a full-lattice vector (even then odd).
 int get_work(qcd_ctx *c, int prec, int slot, HVec *out)
 {
-    if (slot < 0 || slot >= NWORK) {
+    const int nwork = prec == QCD_FX ? (int)NWORK_FX : NWORK;
+    if (slot < 0 || slot >= nwork) {
         set_error_message("workspace slot %d out of range", slot);
         return QCD_EINVAL;
     }
     if (!c->work[prec][0].p) {
         const size_t hb = hvec_bytes(c->g, prec);
-        const size_t nb = prec == QCD_F16 ? (size_t)c->g.Vh_pad * sizeof(float) : 0;
+        const size_t nb = prec == QCD_F16 || prec == QCD_FX ? (size_t)c->g.Vh_pad * sizeof(float) : 0;
         void *base = nullptr, *nbase = nullptr;
-        int rc = dev_alloc(c, &base, hb * NWORK);
+        int rc = dev_alloc(c, &base, hb * nwork);
         if (rc) return rc;
         if (nb) {
-            rc = dev_alloc(c, &nbase, nb * NWORK);
+            rc = dev_alloc(c, &nbase, nb * nwork);
             if (rc) return rc;
         }
-        for (int k = 0; k < NWORK; ++k) {
+        for (int k = 0; k < nwork; ++k) {
             c->work[prec][k].p = (char *)base + k * hb;
             c->work[prec][k].norm = nb ? (float *)((char *)nbase + k * nb) : nullptr;
             c->work[prec][k].prec = prec;
@@ -204,7 +205,9 @@ extern "C" int qcd_create(qcd_ctx **out, const int dims[4], int t_bc, void *stre
         if ((rc = dev_alloc(c, &c->U32[p], vp * 12 * 16))) return fail(rc);
         if ((rc = dev_alloc(c, &c->U16a[p], vp * 4 * 16))) return fail(rc);
         if ((rc = dev_alloc(c, &c->U16b[p], vp * 4 * 8))) return fail(rc);
-        if ((rc = dev_alloc(c, &c->UDF[p], vp * 36 * 16))) return fail(rc);
+        if ((rc = dev_alloc(c, &c->UX[p], vp * 36 * 16))) return fail(rc);
+        if ((rc = dev_alloc(c, (void **)&c->Cx[p], vp * 2 * sizeof(int)))) return fail(rc);
+        if ((rc = dev_alloc(c, (void **)&c->Cix[p], vp * 2 * sizeof(int)))) return fail(rc);
         const size_t cl[4] = {vp * 36 * 16, vp * 18 * 16, vp * 9 * 16, vp * 36 * 16};
         for (int q = 0; q < 4; ++q) {
             if ((rc = dev_alloc(c, &c->C[q][p], cl[q]))) return fail(rc);
@@ -327,7 +330,7 @@ struct ApiBufs {
 int api_bufs(qcd_ctx *c, int prec, int nrhs, ApiBufs *b)
 {
     const size_t hb = hvec_bytes(c->g, prec);
-    const size_t nb = prec == QCD_F16 ? (size_t)c->g.Vh_pad * sizeof(float) : 0;
+    const size_t nb = prec == QCD_F32 ? 0 : (size_t)c->g.Vh_pad * sizeof(float);  // norms, or fixed-point exponents
     // three regions of nrhs vectors each, plus norms
     const size_t need = 3 * nrhs * (hb + nb);
     int rc = ensure_staging(c, need > (size_t)c->g.V * 12 * 16 * 2 ? need : (size_t)c->g.V * 12 * 16 * 2);
@@ -378,7 +381,12 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
         if (rc) return rc;
         const char *src = (const char *)in + r0 * cbytes;
         char *dst = (char *)out + r0 * cbytes;
-        rc = canon_to_half(c, prec, f32io, src, -1, B.in, nr, B.stride);
+        // FP64 and DF64 operators read fixed-point fields (fx.cuh)
+        if (c->fx_links && (prec == QCD_F64 || prec == QCD_DF64) && kind != 3) {
+            B.in.prec = B.tmp.prec = QCD_FX;
+            if (kind <= 1) B.out.prec = QCD_FX;
+        }
+        rc = canon_to_half(c, B.in.prec, f32io, src, -1, B.in, nr, B.stride);
         if (rc) return rc;
         if (kind == 3) {
             rc = clover_apply_half(c, prec, out_par, inverse, B.in, B.out, nr, B.stride);
@@ -412,7 +420,7 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
             rc = launch_stencil(c, s);
         }
         if (rc) return rc;
-        rc = half_to_canon(c, prec, f32io, B.out, dst, -1, nr, B.stride);
+        rc = half_to_canon(c, B.out.prec, f32io, B.out, dst, -1, nr, B.stride);
         if (rc) return rc;
     }
     return QCD_OK;
@@ -785,13 +793,14 @@ int bench_buffers(qcd_ctx *c, int prec, int nrhs, StencilCall &s)
     }
     char *base = (char *)c->bench_buf;
     HVec in, out;
-    in.prec = out.prec = prec;
+    // FP64 and DF64 as the solvers run them: fixed point in and out
+    in.prec = out.prec = c->fx_links && (prec == QCD_F64 || prec == QCD_DF64) ? QCD_FX : prec;
     in.p = base;
     out.p = base + nrhs * hb;
     in.norm = (float *)(base + 2 * nrhs * hb);
     out.norm = (float *)(base + 2 * nrhs * hb + nrhs * nb);
     const size_t stride = hvec_elems(c->g, prec);
-    if ((rc = fill_pattern(c, prec, in, nrhs, stride, 7))) return rc;
+    if ((rc = fill_pattern(c, in.prec, in, nrhs, stride, 7))) return rc;
     s.prec = prec;
     s.mode = M_MULT;
     s.out_par = 0;

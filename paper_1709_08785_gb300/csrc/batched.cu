@@ -49,10 +49,12 @@ struct BProb {
     Geom g;
     double k2;  // kappa^2
     float k2f;  // kappa^2 rounded to FP32 on the host, for the FP32 phases
+    int fx;  // the outer level's links and clover in fixed point (fx.cuh)
     GaugePtr U32, UO;
     CloverPtr Ci32, CiO;                       // UO, CiO: in the outer level's precision
     SpinorPtr x, r, rt, p, q, t, tmp;          // FP32 inner (tmp: odd parity)
     SpinorPtr X, R, RT, P, Q, T, Vv, TMP;      // outer level: DF64 (default) or FP64; X in PX
+    SpinorPtr VX, TX;                          // fixed point: Vv again, and TMP's place
     SolverState *in, *out;                     // inner, outer scalars
     double *partials;                          // [ntiles][4]
     int tile0, ntiles;
@@ -140,7 +142,8 @@ enum Phase {
     PH_LIFT, PH_OMULT, PH_ODHAT, PH_OUPD, PH_OP
 };
 
-// the outer level's hopping term: the rolled loops for DF64 (instruction cache)
+// the outer level's hopping term and F^-1 in its own arithmetic (links out of
+// the fixed-point range): the rolled loops for DF64 (instruction cache)
 template <int PO>
 __device__ __forceinline__ void hop_outer(const BProb &pr, const SpinorPtr &in, int out_par, int cb,
                                           Spinor<typename Prec<PO>::T> &a)
@@ -248,21 +251,33 @@ __device__ void run_phase(const BatchArgs &A, int ph)
                 OpHalf<C32>{pr.x, pr.p, &s_in}(cb, acc);
                 const double *n2 = A.half == 0 ? &s_out.norm2[1] : &s_out.rr;
                 OpLift<C32, PO>{pr.x, pr.Vv, n2}(cb, acc);
+                if (pr.fx) {
+                    Spinor<TO> v;
+                    Spinor<fx2> o;
+                    Prec<PO>::load(pr.Vv, cb, v);  // this thread's own store
+                    const int e = fx_from_spinor(v, o);
+                    fx_store(pr.VX, cb, o, e);
+                }
             }
             break;
         case PH_OMULT:
             if constexpr (!OUTER) break;
             if (site) {
-                Spinor<TO> a;
-                hop_outer<PO>(pr, pr.Vv, 1, cb, a);
-                Prec<PO>::store(pr.TMP, cb, a);
+                if (pr.fx) {
+                    fx_hop_store<false, true, true>(pr.g, pr.UO, pr.CiO, pr.VX, 1, cb, pr.TX);
+                } else {
+                    Spinor<TO> a;
+                    hop_outer<PO>(pr, pr.Vv, 1, cb, a);
+                    Prec<PO>::store(pr.TMP, cb, a);
+                }
             }
             break;
         case PH_ODHAT:
             if constexpr (!OUTER) break;
             if (site) {
                 Spinor<TO> a, v;
-                hop_outer<PO>(pr, pr.TMP, 0, cb, a);
+                if (pr.fx) fx_hop<false, true, true>(pr.g, pr.UO, pr.CiO, pr.TX, 0, cb, a);
+                else hop_outer<PO>(pr, pr.TMP, 0, cb, a);
                 Prec<PO>::load(pr.Vv, cb, v);
                 axpby_sp(a, TO(-pr.k2), a, TO(1.0), v);
                 Prec<PO>::store(A.half == 0 ? pr.Q : pr.T, cb, a);
@@ -487,8 +502,11 @@ int batched_solve(qcd_ctx **ctxs, int n, const void *const *b, void *const *x, c
         for (int k = 0; k < 8; ++k)
             if ((rc = get_work(c, PO, S64_LEVEL + k, &LO[k])) || (rc = get_work(c, QCD_F32, S32_LEVEL + k, &L32[k])))
                 return rc;
+        HVec vx, tx;
+        if (c->fx_links && ((rc = get_work(c, QCD_FX, FX_IN, &vx)) || (rc = get_work(c, QCD_FX, FX_TMP, &tx)))) return rc;
         tmpX = LO[7];
         if (PX != PO && (rc = get_work(c, QCD_F64, S64_RE, &tmpX))) return rc;
+        if (c->fx_links) tmpX = tx;
         SolverState *outer = c->states + ST_OUTER, *inner = c->states + ST_MID, *aux = c->states + ST_AUX;
         const int nn = c->g.Vh_pad;
         cudaStream_t keep = c->stream;
@@ -521,21 +539,26 @@ int batched_solve(qcd_ctx **ctxs, int n, const void *const *b, void *const *x, c
         c->stream = keep;
         if (rc) return rc;
         BProb &pr = host[i];
+        const bool fx = c->fx_links;
+        pr.fx = fx;
         pr.g = c->g;
         pr.k2 = c->kappa * c->kappa;
         pr.k2f = (float)pr.k2;
         for (int par = 0; par < 2; ++par) {
             pr.U32.a[par] = c->U32[par];
             pr.U32.b[par] = nullptr;
-            pr.UO.a[par] = PO == QCD_DF64 ? (const void *)c->UDF[par] : (const void *)c->U64[par];
+            pr.UO.a[par] = (fx || PO == QCD_DF64) ? (const void *)c->UX[par] : (const void *)c->U64[par];
             pr.UO.b[par] = nullptr;
             pr.Ci32.p[par] = c->Ci[QCD_F32][par];
-            pr.CiO.p[par] = c->Ci[PO][par];
+            pr.CiO.p[par] = c->Ci[fx ? QCD_DF64 : PO][par];
+            pr.CiO.e[par] = c->Cix[par];
         }
         pr.x = sp(L32[0]); pr.r = sp(L32[1]); pr.rt = sp(L32[2]); pr.p = sp(L32[3]);
         pr.q = sp(L32[4]); pr.t = sp(L32[5]); pr.tmp = sp(L32[7]);
         pr.X = sp(XX); pr.R = sp(LO[1]); pr.RT = sp(LO[2]); pr.P = sp(LO[3]);
         pr.Q = sp(LO[4]); pr.T = sp(LO[5]); pr.Vv = sp(LO[6]); pr.TMP = sp(LO[7]);
+        pr.VX = sp(vx);
+        pr.TX = sp(tx);
         pr.in = inner;
         pr.out = outer;
         pr.partials = c->partials;

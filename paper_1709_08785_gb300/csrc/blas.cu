@@ -11,6 +11,7 @@
 
 #include "blas.cuh"
 #include "blas_ops.cuh"
+#include "stencil.cuh"
 
 namespace qcd {
 
@@ -112,6 +113,14 @@ __global__ void k_set_tol2(SolverState *dst, const SolverState *src, int slot, d
     case QCD_DF64: { constexpr int P = QCD_DF64; __VA_ARGS__; } \
     default: { constexpr int P = QCD_F16; __VA_ARGS__; }      \
     }
+
+// the same over the fixed-point fields as well
+#define PREC_SWITCH_FX(p, ...)                               \
+    if ((p) == QCD_FX) {                                     \
+        constexpr int P = QCD_FX;                            \
+        for (int once = 0; once < 1; ++once) { __VA_ARGS__; } \
+    } else                                                   \
+        PREC_SWITCH(p, __VA_ARGS__)
 
 int state_init(qcd_ctx *c, SolverState *st, double tol2, double tol2_rel, int maxit, double bd_eps, int unit)
 {
@@ -332,11 +341,11 @@ int canon_to_half(qcd_ctx *c, int prec, int src_is_f32, const void *src, int ful
     const size_t ns = (size_t)c->g.Vh_pad;
     ProfScope prof(c, QCD_K_OTHER, 0.0);
     if (src_is_f32) {
-        PREC_SWITCH(prec, k_canon_to_half<P, float><<<grid, 128, 0, c->stream>>>(c->g, (const float *)src, dst.sp(), full,
+        PREC_SWITCH_FX(prec, k_canon_to_half<P, float><<<grid, 128, 0, c->stream>>>(c->g, (const float *)src, dst.sp(), full,
                                                                                in_stride, rhs_stride, ns);
                     break);
     } else {
-        PREC_SWITCH(prec, k_canon_to_half<P, double><<<grid, 128, 0, c->stream>>>(c->g, (const double *)src, dst.sp(),
+        PREC_SWITCH_FX(prec, k_canon_to_half<P, double><<<grid, 128, 0, c->stream>>>(c->g, (const double *)src, dst.sp(),
                                                                                 full, in_stride, rhs_stride, ns);
                     break);
     }
@@ -351,11 +360,11 @@ int half_to_canon(qcd_ctx *c, int prec, int dst_is_f32, HVec src, void *dst, int
     const size_t ns = (size_t)c->g.Vh_pad;
     ProfScope prof(c, QCD_K_OTHER, 0.0);
     if (dst_is_f32) {
-        PREC_SWITCH(prec, k_half_to_canon<P, float><<<grid, 128, 0, c->stream>>>(c->g, src.sp(), (float *)dst, full,
+        PREC_SWITCH_FX(prec, k_half_to_canon<P, float><<<grid, 128, 0, c->stream>>>(c->g, src.sp(), (float *)dst, full,
                                                                                out_stride, rhs_stride, ns);
                     break);
     } else {
-        PREC_SWITCH(prec, k_half_to_canon<P, double><<<grid, 128, 0, c->stream>>>(c->g, src.sp(), (double *)dst, full,
+        PREC_SWITCH_FX(prec, k_half_to_canon<P, double><<<grid, 128, 0, c->stream>>>(c->g, src.sp(), (double *)dst, full,
                                                                                 out_stride, rhs_stride, ns);
                     break);
     }
@@ -388,7 +397,7 @@ int fill_pattern(qcd_ctx *c, int prec, HVec v, int nrhs, size_t rhs_stride, int 
 {
     dim3 grid(nblocks(c->g.Vh_pad, 128), nrhs);
     ProfScope prof(c, QCD_K_OTHER, 0.0);
-    PREC_SWITCH(prec, k_fill<P><<<grid, 128, 0, c->stream>>>(c->g, v.sp(), rhs_stride, (size_t)c->g.Vh_pad, seed);
+    PREC_SWITCH_FX(prec, k_fill<P><<<grid, 128, 0, c->stream>>>(c->g, v.sp(), rhs_stride, (size_t)c->g.Vh_pad, seed);
                 break);
     QCD_CUDA_CHECK(cudaGetLastError());
     return QCD_OK;
@@ -408,22 +417,40 @@ struct OpConvert {
     }
 };
 
-int convert_half(qcd_ctx *c, HVec src, HVec dst)
+// one half vector to fixed point
+template <int P>
+struct OpToFx {
+    SpinorPtr src, dst;
+    __device__ void operator()(int cb, double *) const
+    {
+        Spinor<typename Prec<P>::T> S;
+        Prec<P>::load(src, cb, S);
+        Spinor<fx2> o;
+        const int e = fx_from_spinor(S, o);
+        fx_store(dst, cb, o, e);
+    }
+};
+
+int convert_half(qcd_ctx *c, HVec src, HVec dst, const int *done)
 {
     const int n = c->g.Vh_pad;
     const double by = (sp_bytes(src.prec) + sp_bytes(dst.prec)) * n;
     if (src.prec == QCD_F64 && dst.prec == QCD_DF64)
-        return run<0>(c, n, OpConvert<QCD_F64, QCD_DF64>{src.sp(), dst.sp()}, FIN_NONE, nullptr, nullptr, QCD_K_BLAS, by);
+        return run<0>(c, n, OpConvert<QCD_F64, QCD_DF64>{src.sp(), dst.sp()}, FIN_NONE, nullptr, done, QCD_K_BLAS, by);
     if (src.prec == QCD_DF64 && dst.prec == QCD_F64)
-        return run<0>(c, n, OpConvert<QCD_DF64, QCD_F64>{src.sp(), dst.sp()}, FIN_NONE, nullptr, nullptr, QCD_K_BLAS, by);
+        return run<0>(c, n, OpConvert<QCD_DF64, QCD_F64>{src.sp(), dst.sp()}, FIN_NONE, nullptr, done, QCD_K_BLAS, by);
+    if (src.prec == QCD_F64 && dst.prec == QCD_FX)
+        return run<0>(c, n, OpToFx<QCD_F64>{src.sp(), dst.sp()}, FIN_NONE, nullptr, done, QCD_K_BLAS, by);
+    if (src.prec == QCD_DF64 && dst.prec == QCD_FX)
+        return run<0>(c, n, OpToFx<QCD_DF64>{src.sp(), dst.sp()}, FIN_NONE, nullptr, done, QCD_K_BLAS, by);
     set_error_message("unsupported conversion %d -> %d", src.prec, dst.prec);
     return QCD_EINVAL;
 }
 
 // ---------------------------------------------------------------- clover apply
-template <int P>
+template <int P, bool FX>
 __global__ void k_clover_apply(Geom g, CloverPtr C, int par, SpinorPtr in, SpinorPtr out, size_t rhs_stride,
-                               size_t norm_stride)
+                               size_t norm_stride, int out_fx)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = blockIdx.y;
@@ -436,20 +463,46 @@ __global__ void k_clover_apply(Geom g, CloverPtr C, int par, SpinorPtr in, Spino
     o.norm = out.norm ? out.norm + r * norm_stride : nullptr;
     Spinor<T> S;
     Prec<P>::load(i, cb, S);
-    apply_clover<P>(C, par, cb, S);
+    if constexpr (FX) {
+        Spinor<fx2> x;
+        Spinor<long long> y;
+        int e = fx_from_spinor(S, x);
+        fx_clover(C, par, cb, x, e, y);
+        if (out_fx) {
+            fx_normalise(y, e, x);
+            fx_store(o, cb, x, e);
+            return;
+        }
+        fx_to_spinor(y, e, S);
+    } else {
+        apply_clover<P>(C, par, cb, S);
+    }
     Prec<P>::store(o, cb, S);
 }
 
 int clover_apply_half(qcd_ctx *c, int prec, int parity, int inverse, HVec in, HVec out, int nrhs, size_t rhs_stride)
 {
+    const bool fx = c->fx_links && (prec == QCD_F64 || prec == QCD_DF64);
     CloverPtr C;
-    for (int p = 0; p < 2; ++p) C.p[p] = inverse ? c->Ci[prec][p] : c->C[prec][p];
+    for (int p = 0; p < 2; ++p) {
+        const int pf = fx ? QCD_DF64 : prec;
+        C.p[p] = inverse ? c->Ci[pf][p] : c->C[pf][p];
+        C.e[p] = inverse ? c->Cix[p] : c->Cx[p];
+    }
     dim3 grid(nblocks(c->g.Vh, 128), nrhs);
     const double cl = prec == QCD_F32 ? 288 : prec == QCD_F16 ? 144 : 576;
     ProfScope prof(c, QCD_K_OTHER, (cl + 2 * nrhs * sp_bytes(prec)) * c->g.Vh);
-    PREC_SWITCH(prec, k_clover_apply<P><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride,
-                                                                    (size_t)c->g.Vh_pad);
-                break);
+    const size_t ns = (size_t)c->g.Vh_pad;
+    if (fx && prec == QCD_F64)
+        k_clover_apply<QCD_F64, true><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns,
+                                                                  out.prec == QCD_FX);
+    else if (fx)
+        k_clover_apply<QCD_DF64, true><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns,
+                                                                   out.prec == QCD_FX);
+    else
+        PREC_SWITCH(prec, k_clover_apply<P, false><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(),
+                                                                               rhs_stride, ns, 0);
+                    break);
     QCD_CUDA_CHECK(cudaGetLastError());
     return QCD_OK;
 }

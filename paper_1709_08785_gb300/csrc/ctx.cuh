@@ -99,12 +99,19 @@ struct qcd_ctx {
     void *U32[2] = {nullptr, nullptr};
     void *U16a[2] = {nullptr, nullptr};
     void *U16b[2] = {nullptr, nullptr};
-    void *UDF[2] = {nullptr, nullptr};  // DF64: 18 reals as float pairs
+    // 18 reals per link for the FP64 and DF64 operators: fixed point (fx.cuh),
+    // or float pairs if some link is out of its range (fx_links false; the
+    // FP64 operators then read U64)
+    void *UX[2] = {nullptr, nullptr};
+    bool fx_links = false;
     bool have_gauge = false;
 
-    // clover term F and inverse, [precision][parity]
+    // clover term F and inverse, [precision][parity]; QCD_DF64: fixed point
+    // with two unit exponents per site, or float pairs (as UX)
     void *C[4][2] = {};
     void *Ci[4][2] = {};
+    int *Cx[2] = {nullptr, nullptr};
+    int *Cix[2] = {nullptr, nullptr};
     bool have_clover = false;
     double kappa = 0.0, csw = 0.0;
 
@@ -118,7 +125,7 @@ struct qcd_ctx {
 
     // workspace vectors, allocated on first use
     std::vector<void *> pool;
-    qcd::HVec work[4][16];  // [precision][slot]
+    qcd::HVec work[5][16];  // [precision][slot]; QCD_FX has NWORK_FX of them
     void *staging = nullptr;        // canonical full-lattice complex128 staging
     size_t staging_bytes = 0;
 
@@ -183,6 +190,10 @@ struct qcd_ctx {
 namespace qcd {
 
 constexpr int NSTATES = 8;
+// fixed-point work vectors: the converted input of an FP64 / DF64 operator
+// whose caller holds it in that precision, and the odd-parity vector between
+// the halves of D^
+enum FxSlot { FX_IN = 0, FX_TMP = 1, NWORK_FX = 2 };
 constexpr int PROF_CAP = 1 << 16;  // profiled launches between two collections
 enum StateSlot { ST_OUTER = 0, ST_MID = 1, ST_INNER = 2, ST_AUX = 3, ST_TUNE = 4 };
 
@@ -242,7 +253,8 @@ int fill_pattern(qcd_ctx *c, int prec, HVec v, int nrhs, size_t rhs_stride, int 
 
 // blas.cu -- conversions between canonical and internal layouts
 int canon_to_half(qcd_ctx *c, int prec, int src_is_f32, const void *src, int parity_full, HVec dst, int nrhs, size_t rhs_stride);
-int convert_half(qcd_ctx *c, HVec src, HVec dst);  // between precisions, one half vector
+// between precisions, one half vector (skipped on the device once *done)
+int convert_half(qcd_ctx *c, HVec src, HVec dst, const int *done = nullptr);
 int half_to_canon(qcd_ctx *c, int prec, int dst_is_f32, HVec src, void *dst, int parity_full, int nrhs, size_t rhs_stride);
 int clover_apply_half(qcd_ctx *c, int prec, int parity, int inverse, HVec in, HVec out, int nrhs, size_t rhs_stride);
 

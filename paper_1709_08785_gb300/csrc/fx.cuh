@@ -1,0 +1,313 @@
+// Block fixed-point arithmetic ("FX"): FP64-accurate sums of products on the
+// integer multiply-add pipe.
+//
+// GB300 issues an FP64 FMA on 2 lanes per clock and SM, an IMAD.WIDE
+// (32 x 32 + 64 -> 64 bits) on 64 (measured: 2.0 and 63.8), so a product
+// built from three IMAD.WIDE is ten times cheaper than one FP64 FMA.  A
+// number is a signed integer t times a power of two shared by a whole site
+// (spinors, |t| < 2^57; clover blocks, 2^55) or by the field (links, whose
+// entries are at most 1 = 2^55), kept as two limbs, t = h 2^28 + l.  A sum of products keeps two 64-bit
+// accumulators:
+//     sum a b = 2^56 sum ah bh + 2^28 sum (ah bl + al bh) + (sum al bl),
+// the last term (below 1/4 unit of the result per product) is dropped, and
+// the result is sum ah bh + (mid >> 28) in units of 2^56.  Every step is
+// exact integer arithmetic but for that term and the final rounding, about
+// 2^-57 of the largest component of the site: several times less than the FP64
+// forms lose in their chains of roundings (2^-53 of the running sum per FMA).
+#pragma once
+
+#include "qcd_internal.cuh"
+
+namespace qcd {
+
+constexpr int FX_BITS = 55;  // links and clover blocks: |t| <= 2^FX_BITS
+constexpr int FX_VBITS = 57; // spinors: |t| < 2^FX_VBITS
+constexpr int FX_LIMB = 28;
+// Links of a larger squared Frobenius norm (SU(3): 3) keep the FP64 forms.
+// With it every product of links below stays in range: |A B| <= 3, |A B C| <=
+// 5.2 entry by entry, so that limbs stay below 2^31 and sums below 2^63.
+constexpr float FX_LINK_FRO2 = 3.001f;
+
+// a += x y as one instruction (written in C the sums are reassociated into
+// products and 64-bit additions, three instructions each)
+__device__ __forceinline__ void fx_mac(long long &a, int x, int y)
+{
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(x), "r"(y));
+}
+__device__ __forceinline__ long long fx_mul(int x, int y) { return (long long)x * y; }
+
+// the limbs of t
+__device__ __forceinline__ int fx_lo(long long t) { return ((int)(unsigned)t << 4) >> 4; }
+__device__ __forceinline__ int fx_hi(long long t) { return (int)((t + (1ll << (FX_LIMB - 1))) >> FX_LIMB); }
+
+// One complex number as limbs
+struct fxc {
+    int rh, rl, ih, il;
+};
+__device__ __forceinline__ fxc fx_unpack(int4 v) { return fxc{v.x, v.y, v.z, v.w}; }
+__device__ __forceinline__ int4 fx_pack(long long r, long long i) { return make_int4(fx_hi(r), fx_lo(r), fx_hi(i), fx_lo(i)); }
+
+// rint-free conversion of a double with |d| <= 1: t = d 2^55 (bits below one
+// unit cut off: 2^-55 absolute, an eighth of a unit in the last place of 1).
+// Larger, infinite or NaN values set *bad (links of SU(3) have none).
+__device__ __forceinline__ long long fx_from_unit(double d, int &bad)
+{
+    const long long b = __double_as_longlong(d);
+    const int hi = (int)(b >> 32);
+    const int ex = (hi >> 20) & 0x7ff;
+    bad |= !(fabs(d) <= 1.0 + 1e-9);
+    if (ex == 0) return 0;  // zero and denormals
+    long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;  // 2^52 <= m < 2^53
+    const int sh = 1023 - ex;                                    // |d| = m 2^(-52 - sh)
+    m = sh >= 0 ? (m << 3) >> (sh > 63 ? 63 : sh) : m << 3;
+    return b < 0 ? -m : m;
+}
+
+// ---------------------------------------------------------------- 3x3 matrices
+// A link product in FX: entries at most 1 (field scale 2^-55)
+struct M3x {
+    fxc m[3][3];
+};
+
+// C = op(A) op(B), op = dagger where DA / DB is set, times sgn (+-1); in the
+// operands' scale: t_C = t_A t_B 2^-55.  For entries up to 1 every
+// accumulator stays below 2^62 (three complex products, limbs up to 2^29.6
+// after one product of three terms).
+template <bool DA, bool DB>
+__device__ __forceinline__ void fx_mul_elem(const M3x &A, const M3x &B, int i, int j, long long &tr, long long &ti)
+{
+    // mid sums start at half a unit of their final shift
+    long long mr = 1ll << 26, mi = 1ll << 26, hr = 0, hi = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const fxc a = DA ? A.m[k][i] : A.m[i][k];
+        const fxc b = DB ? B.m[j][k] : B.m[k][j];
+        // (ar + i sa ai)(br + i sb bi)
+        const int aih = DA ? -a.ih : a.ih, ail = DA ? -a.il : a.il;
+        const int bih = DB ? -b.ih : b.ih, bil = DB ? -b.il : b.il;
+        fx_mac(mr, a.rh, b.rl);
+        fx_mac(mr, a.rl, b.rh);
+        fx_mac(mr, -aih, bil);
+        fx_mac(mr, -ail, bih);
+        fx_mac(mi, a.rh, bil);
+        fx_mac(mi, a.rl, bih);
+        fx_mac(mi, aih, b.rl);
+        fx_mac(mi, ail, b.rh);
+        fx_mac(hr, a.rh, b.rh);
+        fx_mac(hr, -aih, bih);
+        fx_mac(hi, a.rh, bih);
+        fx_mac(hi, aih, b.rh);
+    }
+    tr = (hr << 1) + (mr >> 27);
+    ti = (hi << 1) + (mi >> 27);
+}
+
+// ---------------------------------------------------------------- spinors
+// A real as limbs, with the additions the spin projection needs (limb by limb:
+// the sum of two numbers below 2^55 has limbs below 2^28 and 2^29)
+struct fx2 {
+    int h, l;
+};
+__device__ __forceinline__ fx2 operator+(fx2 a, fx2 b) { return {a.h + b.h, a.l + b.l}; }
+__device__ __forceinline__ fx2 operator-(fx2 a, fx2 b) { return {a.h - b.h, a.l - b.l}; }
+__device__ __forceinline__ fx2 operator-(fx2 a) { return {-a.h, -a.l}; }
+
+// Unit exponents: the value of t is t 2^e.  A zero site has FX_ZERO; a site
+// with an infinite or NaN component has FX_NAN, and so has every result that
+// reads it.
+constexpr int FX_ZERO = -100000, FX_NAN = 100000;
+
+// the limbs of a signed t, the low one unsigned (the partner's low limb is
+// balanced wherever two low limbs would meet)
+__device__ __forceinline__ fx2 fx_split(long long t) { return {(int)(t >> FX_LIMB), (int)t & ((1 << FX_LIMB) - 1)}; }
+
+__device__ __forceinline__ int fx_clamp63(int s) { return s > 63 ? 63 : s; }
+
+// a double's exponent field, and its t in units of 2^(E - 1023 - 56) for a site
+// whose largest exponent field is E (bits below one unit cut off)
+__device__ __forceinline__ int fx_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
+__device__ __forceinline__ fx2 fx_limbs(double d, int E)
+{
+    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+    unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << (FX_VBITS - 53);
+    m >>= fx_clamp63(ex ? E - ex : 63);
+    const int sg = (hi >> 31) | 1;
+    const fx2 v = fx_split((long long)m);
+    return {v.h * sg, v.l * sg};
+}
+// the same as one signed integer in units of 2^(E - 1023 - 54), |t| < 2^55 (for
+// operands stored with balanced limbs)
+__device__ __forceinline__ long long fx_int(double d, int E)
+{
+    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+    unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 2;
+    m >>= fx_clamp63(ex ? E - ex : 63);
+    return hi < 0 ? -(long long)m : (long long)m;
+}
+// the same for a float pair: field of the leading float, widened
+__device__ __forceinline__ int fx_field(df d)
+{
+    const int ex = (__float_as_int(d.hi) >> 23) & 0xff;
+    return ex == 0xff ? 0x7ff : ex ? ex + 896 : 0;
+}
+__device__ __forceinline__ long long fx_float(float f, int E)
+{
+    const int b = __float_as_int(f), ex = (b >> 23) & 0xff;
+    const long long m = (long long)((b & 0x7fffff) | 0x800000) << (FX_VBITS - 24);
+    const long long t = m >> fx_clamp63(ex ? E - (ex + 896) : 63);
+    return b < 0 ? -t : t;
+}
+__device__ __forceinline__ fx2 fx_limbs(df d, int E) { return fx_split(fx_float(d.hi, E) + fx_float(d.lo, E)); }
+
+// a spinor in FP64 or DF64 arithmetic as limbs; returns its unit exponent
+template <class T>
+__device__ __forceinline__ int fx_from_spinor(const Spinor<T> &p, Spinor<fx2> &o)
+{
+    int E = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) E = max(E, max(fx_field(p.s[a][i].r), fx_field(p.s[a][i].i)));
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) o.s[a][i] = cx<fx2>{fx_limbs(p.s[a][i].r, E), fx_limbs(p.s[a][i].i, E)};
+    return E == 0 ? FX_ZERO : E == 0x7ff ? FX_NAN : E - (1023 + FX_VBITS - 1);
+}
+
+// t 2^e in the arithmetic type T
+__device__ __forceinline__ double fx_pow2(int e)  // 2^e; the caller keeps e in the normal range
+{
+    return __longlong_as_double((long long)(1023 + e) << 52);
+}
+__device__ __forceinline__ void fx_normalise(const Spinor<long long> &v, int &e, Spinor<long long> &o);
+template <class T>
+__device__ __forceinline__ void fx_to_spinor(const Spinor<long long> &v, int e, Spinor<T> &o)
+{
+    if constexpr (std::is_same<T, df>::value) {
+        // float pairs without the FP64 pipe: the site scaled to 57 bits, the top
+        // 24 exactly and the next 31 rounded to a float
+        Spinor<long long> t;
+        int en = e;
+        fx_normalise(v, en, t);
+        const int es = en + FX_VBITS - 24;
+        if (es > -100 && es < 100) {
+            const float s = __int_as_float((127 + es) << 23), s31 = 4.656612873077392578125e-10f * s;  // 2^-31 s
+            auto conv = [&](long long x) {
+                const float hi = (float)(int)(x >> (FX_VBITS - 24)) * s;
+                const float lo = (float)((int)(x >> (FX_VBITS - 55)) & 0x7fffffff) * s31;
+                return fast_two_sum(hi, lo);
+            };
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) o.s[a][i] = mk(conv(t.s[a][i].r), conv(t.s[a][i].i));
+            return;
+        }
+    }
+    if (e >= FX_NAN / 2) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) o.s[a][i] = mk(T(__longlong_as_double(0x7ff8000000000000ll)), T(__longlong_as_double(0x7ff8000000000000ll)));
+        return;
+    }
+    // below the normal range (sites under 2^-900) in two steps
+    const double s1 = fx_pow2(e < -1000 ? -1000 : e);
+    const double s2 = e >= -1000 ? 1.0 : e < -2000 ? 0.0 : fx_pow2(e + 1000);
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            double r = (double)v.s[a][i].r * s1, m = (double)v.s[a][i].i * s1;
+            if (e < -1000) {
+                r *= s2;
+                m *= s2;
+            }
+            o.s[a][i] = mk(T(r), T(m));
+        }
+}
+
+// v scaled below 2^57; e follows
+__device__ __forceinline__ void fx_normalise(const Spinor<long long> &v, int &e, Spinor<long long> &o)
+{
+    unsigned mh = 0, ml = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const long long c[2] = {v.s[a][i].r, v.s[a][i].i};
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const unsigned h = (unsigned)((unsigned long long)c[k] >> 32), s = (unsigned)((int)h >> 31);
+                mh |= h ^ s;
+                ml |= (unsigned)c[k] ^ s;
+            }
+        }
+    // lz >= 1 leading zeros of the largest magnitude (up to 63 for all zero)
+    const int lz = mh ? __clz(mh) : 32 + min(__clz(ml), 31);
+    const int up = lz - 1;  // the largest to 2^62 or more, then six bits down: below 2^57
+    constexpr int DN = 63 - FX_VBITS;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            o.s[a][i].r = (v.s[a][i].r << up) >> DN;
+            o.s[a][i].i = (v.s[a][i].i << up) >> DN;
+        }
+    if (e > FX_ZERO / 2 && e < FX_NAN / 2) e += DN - up;
+}
+
+// the same, split into limbs
+__device__ __forceinline__ void fx_normalise(const Spinor<long long> &v, int &e, Spinor<fx2> &o)
+{
+    Spinor<long long> t;
+    fx_normalise(v, e, t);
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) o.s[a][i] = cx<fx2>{fx_split(t.s[a][i].r), fx_split(t.s[a][i].i)};
+}
+
+// ---------------------------------------------------------------- fields
+// A fixed-point spinor field, the operators' input: 12 int4 (re h, re l, im h,
+// im l) per site in the site-blocked order, and one unit exponent per site in
+// the place of the FP16 norms.
+
+__device__ __forceinline__ void fx_store(const SpinorPtr &v, int cb, const Spinor<fx2> &s, int e)
+{
+    int4 *p = (int4 *)v.p;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const cx<fx2> z = s.s[k / 3][k % 3];
+        p[soa(cb, 12, k)] = make_int4(z.r.h, z.r.l, z.i.h, z.i.l);
+    }
+    ((int *)v.norm)[cb] = e;
+}
+
+template <>
+struct Prec<QCD_FX> {
+    using T = double;
+    static constexpr int SP_NC = 12;
+    static __device__ __forceinline__ void load(const SpinorPtr &v, int cb, Spinor<T> &s)
+    {
+        const int4 *p = (const int4 *)v.p;
+        Spinor<long long> t;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const int4 q = __ldg(p + soa(cb, 12, k));
+            t.s[k / 3][k % 3] = mk(((long long)q.x << FX_LIMB) + q.y, ((long long)q.z << FX_LIMB) + q.w);
+        }
+        fx_to_spinor(t, __ldg((const int *)v.norm + cb), s);
+    }
+    static __device__ __forceinline__ void store(const SpinorPtr &v, int cb, const Spinor<T> &s)
+    {
+        Spinor<fx2> o;
+        const int e = fx_from_spinor(s, o);
+        fx_store(v, cb, o, e);
+    }
+};
+
+}  // namespace qcd

@@ -12,6 +12,7 @@
 //   B_1 = F_yz, B_2 = F_zx, B_3 = F_xy, E_k = F_kt,
 // each a 6x6 Hermitian matrix indexed 3*spin + colour.
 #include "ctx.cuh"
+#include "fx.cuh"
 
 namespace qcd {
 
@@ -22,9 +23,12 @@ __device__ __forceinline__ float4 df_pair(double2 z)
     return make_float4(r.hi, r.lo, i.hi, i.lo);
 }
 
+// FX: the third copy of a link is its fixed-point form (fx.cuh); otherwise, for
+// fields with links beyond that form's range, float pairs.
+template <bool FX>
 __global__ void k_gauge_convert(Geom g, const double2 *__restrict__ U, double2 *U64e, double2 *U64o, float4 *U32e,
-                                float4 *U32o, uint4 *U16ae, uint4 *U16ao, uint2 *U16be, uint2 *U16bo, float4 *UDFe,
-                                float4 *UDFo)
+                                float4 *U32o, uint4 *U16ae, uint4 *U16ao, uint2 *U16be, uint2 *U16bo, void *UXe,
+                                void *UXo, int *wide)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.V) return;
@@ -39,12 +43,22 @@ __global__ void k_gauge_convert(Geom g, const double2 *__restrict__ U, double2 *
     float4 *u32 = par ? U32o : U32e;
     uint4 *u16a = par ? U16ao : U16ae;
     uint2 *u16b = par ? U16bo : U16be;
+    void *ux = par ? UXo : UXe;
     for (int mu = 0; mu < 4; ++mu) {
         double2 m[9];
         for (int k = 0; k < 9; ++k) m[k] = U[((size_t)s * 4 + mu) * 9 + k];
         for (int k = 0; k < 9; ++k) u64[soa(cb, 36, mu * 9 + k)] = m[k];
-        float4 *udf = par ? UDFo : UDFe;
-        for (int k = 0; k < 9; ++k) udf[soa(cb, 36, mu * 9 + k)] = df_pair(m[k]);
+        if constexpr (FX) {
+            float fro = 0.f;
+            int bad = 0;
+            for (int k = 0; k < 9; ++k) {
+                ((int4 *)ux)[soa(cb, 36, mu * 9 + k)] = fx_pack(fx_from_unit(m[k].x, bad), fx_from_unit(m[k].y, bad));
+                fro += (float)m[k].x * (float)m[k].x + (float)m[k].y * (float)m[k].y;
+            }
+            if (bad || !(fro <= FX_LINK_FRO2)) *wide = 1;
+        } else {
+            for (int k = 0; k < 9; ++k) ((float4 *)ux)[soa(cb, 36, mu * 9 + k)] = df_pair(m[k]);
+        }
         // first two columns: a = (m00, m10, m20), b = (m01, m11, m21)
         const double2 a0 = m[0], a1 = m[3], a2 = m[6], b0 = m[1], b1 = m[4], b2 = m[7];
         u32[soa(cb, 12, mu * 3 + 0)] = make_float4(a0.x, a0.y, a1.x, a1.y);
@@ -58,259 +72,436 @@ __global__ void k_gauge_convert(Geom g, const double2 *__restrict__ U, double2 *
 
 int gauge_convert(qcd_ctx *c, const void *U_dev)
 {
-    k_gauge_convert<<<nblocks(c->g.V, 256), 256, 0, c->stream>>>(
-        c->g, (const double2 *)U_dev, (double2 *)c->U64[0], (double2 *)c->U64[1], (float4 *)c->U32[0],
-        (float4 *)c->U32[1], (uint4 *)c->U16a[0], (uint4 *)c->U16a[1], (uint2 *)c->U16b[0], (uint2 *)c->U16b[1],
-        (float4 *)c->UDF[0], (float4 *)c->UDF[1]);
-    QCD_CUDA_CHECK(cudaGetLastError());
-    return QCD_OK;
+    auto go = [&](auto kernel) -> int {
+        kernel<<<nblocks(c->g.V, 256), 256, 0, c->stream>>>(
+            c->g, (const double2 *)U_dev, (double2 *)c->U64[0], (double2 *)c->U64[1], (float4 *)c->U32[0],
+            (float4 *)c->U32[1], (uint4 *)c->U16a[0], (uint4 *)c->U16a[1], (uint2 *)c->U16b[0], (uint2 *)c->U16b[1],
+            c->UX[0], c->UX[1], c->flag_dev);
+        QCD_CUDA_CHECK(cudaGetLastError());
+        return QCD_OK;
+    };
+    QCD_CUDA_CHECK(cudaMemsetAsync(c->flag_dev, 0, sizeof(int), c->stream));
+    int rc = go(k_gauge_convert<true>);
+    if (rc) return rc;
+    int wide = 0;
+    QCD_CUDA_CHECK(cudaMemcpyAsync(&wide, c->flag_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    QCD_CUDA_CHECK(cudaStreamSynchronize(c->stream));
+    c->fx_links = !wide;
+    return wide ? go(k_gauge_convert<false>) : QCD_OK;
 }
 
 // ---------------------------------------------------------------- clover
+// F_munu from ten 3x3 products per plane: with K = (L1 - L4^dag) + (L3 - L2^dag)
+// the leaves' sum Q obeys Q - Q^dag = K - K^dag, and the four leaves of K pair
+// by their first and last links,
+//   K = [U_mu(n) P1 - U_mu(n-mu)^dag P1'] U_nu(n)^dag
+//     - [U_mu(n) P2 - U_mu(n-mu)^dag P2'] U_nu(n-nu),
+//   P1  = U_nu(n+mu) U_mu(n+nu)^dag,          P1' = U_nu(n-mu) U_mu(n-mu+nu),
+//   P2  = U_nu(n+mu-nu)^dag U_mu(n-nu)^dag,   P2' = U_nu(n-mu-nu)^dag U_mu(n-mu-nu)
+// (twelve products leaf by leaf).  The products run in an algebra: AlgX, the
+// fixed-point form of fx.cuh on the integer pipe, whose accumulators hold
+// every product of links with a Frobenius norm up to sqrt(3) (each of SU(3)
+// has exactly that); AlgD, FP64, for fields with larger links.
 struct M3 {
     cx<double> m[3][3];
 };
 
-__device__ __forceinline__ M3 mul(const M3 &a, const M3 &b)
-{
-    M3 c;
+struct AlgX {
+    using M = M3x;
+    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu)
+    {
+        const int4 *p = (const int4 *)U.a[par];
+        M r;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<double> s = mk(0.0, 0.0);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) fma_(s, a.m[i][k], b.m[k][j]);
-            c.m[i][j] = s;
-        }
-    return c;
-}
-
-__device__ __forceinline__ M3 dag(const M3 &a)
-{
-    M3 c;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) c.m[i][j] = conj(a.m[j][i]);
-    return c;
-}
-
-// link U_mu at lexicographic site s
-__device__ __forceinline__ M3 link_at(const Geom &g, const GaugePtr &U, int s, int mu)
-{
-    int c[4], t = s;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        c[k] = t % g.L[k];
-        t /= g.L[k];
+        for (int k = 0; k < 9; ++k) r.m[k / 3][k % 3] = fx_unpack(__ldg(p + soa(cb, 36, mu * 9 + k)));
+        return r;
     }
-    const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
-    Link<double> L;
-    Prec<QCD_F64>::load_link(U, par, s >> 1, mu, L);
-    M3 m;
+    template <bool DA, bool DB>
+    static __device__ __forceinline__ M mul(const M &A, const M &B)
+    {
+        M C;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) m.m[i][j] = L.u[i][j];
-    return m;
-}
-
-// lexicographic site s + dm*mu + dn*nu
-__device__ __forceinline__ int shift2(const Geom &g, const int c[4], int mu, int dm, int nu, int dn)
-{
-    int d[4] = {c[0], c[1], c[2], c[3]};
-    d[mu] = (d[mu] + dm + g.L[mu]) % g.L[mu];
-    d[nu] = (d[nu] + dn + g.L[nu]) % g.L[nu];
-    return lex_of(g, d);
-}
-
-// F_munu(n) = (Q - Q^dag)/(8i), Q = sum of the four counter-clockwise leaves
-// at n in the (mu, nu) plane.
-__device__ M3 field_strength(const Geom &g, const GaugePtr &U, const int c[4], int mu, int nu)
-{
-    const int n = lex_of(g, c);
-    const int n_pm = shift2(g, c, mu, 1, nu, 0), n_pn = shift2(g, c, mu, 0, nu, 1);
-    const int n_mm = shift2(g, c, mu, -1, nu, 0), n_mn = shift2(g, c, mu, 0, nu, -1);
-    const int n_mm_pn = shift2(g, c, mu, -1, nu, 1), n_pm_mn = shift2(g, c, mu, 1, nu, -1);
-    const int n_mm_mn = shift2(g, c, mu, -1, nu, -1);
-    M3 Q;
-    // U_mu(n) U_nu(n+mu) U_mu(n+nu)^dag U_nu(n)^dag
-    M3 t = mul(mul(link_at(g, U, n, mu), link_at(g, U, n_pm, nu)), mul(dag(link_at(g, U, n_pn, mu)), dag(link_at(g, U, n, nu))));
-    Q = t;
-    // U_nu(n) U_mu(n-mu+nu)^dag U_nu(n-mu)^dag U_mu(n-mu)
-    t = mul(mul(link_at(g, U, n, nu), dag(link_at(g, U, n_mm_pn, mu))), mul(dag(link_at(g, U, n_mm, nu)), link_at(g, U, n_mm, mu)));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + t.m[i][j];
-    // U_mu(n-mu)^dag U_nu(n-mu-nu)^dag U_mu(n-mu-nu) U_nu(n-nu)
-    t = mul(mul(dag(link_at(g, U, n_mm, mu)), dag(link_at(g, U, n_mm_mn, nu))), mul(link_at(g, U, n_mm_mn, mu), link_at(g, U, n_mn, nu)));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + t.m[i][j];
-    // U_nu(n-nu)^dag U_mu(n-nu) U_nu(n+mu-nu) U_mu(n)^dag
-    t = mul(mul(dag(link_at(g, U, n_mn, nu)), link_at(g, U, n_mn, mu)), mul(link_at(g, U, n_pm_mn, nu), dag(link_at(g, U, n, mu))));
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Q.m[i][j] = Q.m[i][j] + t.m[i][j];
-    M3 F;
-    // (Q - Q^dag)/(8i) = -i (Q - Q^dag)/8
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) F.m[i][j] = 0.125 * tmi(Q.m[i][j] - conj(Q.m[j][i]));
-    return F;
-}
-
-// A += coef * (s_l (x) G), 6x6 indexed 3*spin + colour
-__device__ __forceinline__ void add_kron(cx<double> A[6][6], double coef, int l, const M3 &G)
-{
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            const cx<double> gv = coef * G.m[i][j];
-            if (l == 1) {  // s_1 = [[0,1],[1,0]]
-                A[i][3 + j] = A[i][3 + j] + gv;
-                A[3 + i][j] = A[3 + i][j] + gv;
-            } else if (l == 2) {  // s_2 = [[0,-i],[i,0]]
-                A[i][3 + j] = A[i][3 + j] + tmi(gv);
-                A[3 + i][j] = A[3 + i][j] + ti(gv);
-            } else {  // s_3 = diag(1,-1)
-                A[i][j] = A[i][j] + gv;
-                A[3 + i][3 + j] = A[3 + i][3 + j] - gv;
+            for (int j = 0; j < 3; ++j) {
+                long long r, s;
+                fx_mul_elem<DA, DB>(A, B, i, j, r, s);
+                C.m[i][j] = fx_unpack(fx_pack(r, s));
             }
+        return C;
+    }
+    // op(A) B - C^dag D
+    static __device__ __forceinline__ M mul_sub(const M &A, const M &B, const M &C, const M &D)
+    {
+        M R;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                long long r, s, u, v;
+                fx_mul_elem<false, false>(A, B, i, j, r, s);
+                fx_mul_elem<true, false>(C, D, i, j, u, v);
+                R.m[i][j] = fx_unpack(fx_pack(r - u, s - v));
+            }
+        return R;
+    }
+    using T = long long;
+    template <bool DB>
+    static __device__ __forceinline__ void elem(const M &A, const M &B, int i, int j, T &r, T &s)
+    {
+        fx_mul_elem<false, DB>(A, B, i, j, r, s);
+    }
+    static __device__ __forceinline__ double value(T t) { return (double)t * (1.0 / (double)(1ll << FX_BITS)); }
+};
+
+struct AlgD {
+    using M = M3;
+    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu)
+    {
+        Link<double> L;
+        Prec<QCD_F64>::load_link(U, par, cb, mu, L);
+        M r;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) r.m[k / 3][k % 3] = L.u[k / 3][k % 3];
+        return r;
+    }
+    template <bool DA, bool DB>
+    static __device__ __forceinline__ cx<double> el(const M &A, const M &B, int i, int j)
+    {
+        cx<double> s = mk(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const cx<double> a = DA ? conj(A.m[k][i]) : A.m[i][k], b = DB ? conj(B.m[j][k]) : B.m[k][j];
+            fma_(s, a, b);
+        }
+        return s;
+    }
+    template <bool DA, bool DB>
+    static __device__ __forceinline__ M mul(const M &A, const M &B)
+    {
+        M C;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) C.m[i][j] = el<DA, DB>(A, B, i, j);
+        return C;
+    }
+    static __device__ __forceinline__ M mul_sub(const M &A, const M &B, const M &C, const M &D)
+    {
+        M R;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) R.m[i][j] = el<false, false>(A, B, i, j) - el<true, false>(C, D, i, j);
+        return R;
+    }
+    using T = double;
+    template <bool DB>
+    static __device__ __forceinline__ void elem(const M &A, const M &B, int i, int j, T &r, T &s)
+    {
+        const cx<double> z = el<false, DB>(A, B, i, j);
+        r = z.r;
+        s = z.i;
+    }
+    static __device__ __forceinline__ double value(T t) { return t; }
+};
+
+// F_munu at site n of parity par (coordinates c): the three real diagonal
+// entries, then (re, im) of the entries (1,0), (2,0), (2,1) below it
+template <class Alg>
+__device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U, int par, const int c[4], int mu, int nu,
+                                               double F[9])
+{
+    using M = typename Alg::M;
+    auto at = [&](int dm, int dn) {  // cb of n + dm mu + dn nu
+        int lex = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int d = k == mu ? dm : k == nu ? dn : 0;
+            int x = c[k] + d;
+            x = x < 0 ? x + g.L[k] : x >= g.L[k] ? x - g.L[k] : x;
+            lex += x * g.st[k];
+        }
+        return lex >> 1;
+    };
+    const int n = at(0, 0), op = 1 - par;
+    M R1, R2;
+    {
+        const M A = Alg::load(U, par, n, mu), B = Alg::load(U, op, at(-1, 0), mu);
+        {
+            const M P1 = Alg::template mul<false, true>(Alg::load(U, op, at(1, 0), nu), Alg::load(U, op, at(0, 1), mu));
+            const M Q1 = Alg::template mul<false, false>(Alg::load(U, op, at(-1, 0), nu), Alg::load(U, par, at(-1, 1), mu));
+            R1 = Alg::mul_sub(A, P1, B, Q1);
+        }
+        const M P2 = Alg::template mul<true, true>(Alg::load(U, par, at(1, -1), nu), Alg::load(U, op, at(0, -1), mu));
+        const M Q2 = Alg::template mul<true, false>(Alg::load(U, par, at(-1, -1), nu), Alg::load(U, par, at(-1, -1), mu));
+        R2 = Alg::mul_sub(A, P2, B, Q2);
+    }
+    const M C = Alg::load(U, par, n, nu), D = Alg::load(U, op, at(0, -1), nu);
+    auto K = [&](int i, int j, typename Alg::T &r, typename Alg::T &s) {
+        typename Alg::T r2, s2;
+        Alg::template elem<true>(R1, C, i, j, r, s);
+        Alg::template elem<false>(R2, D, i, j, r2, s2);
+        r -= r2;
+        s -= s2;
+    };
+    // (K - K^dag)/(8i)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        typename Alg::T r, s;
+        K(i, i, r, s);
+        F[i] = 0.25 * Alg::value(s);
+    }
+#pragma unroll
+    for (int i = 1; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            typename Alg::T r, s, rt, sT;
+            K(i, j, r, s);
+            K(j, i, rt, sT);
+            const int k = 3 + 2 * (i + j - 1);
+            F[k] = 0.125 * Alg::value(s + sT);
+            F[k + 1] = -0.125 * Alg::value(r - rt);
         }
 }
 
-// Hermitian 6x6 inverse by A = L D L^dag (no pivoting; the clover blocks
-// are close to the identity).  Returns false on a (near-)zero pivot.
-__device__ bool herm_inverse6(const cx<double> A[6][6], cx<double> Ai[6][6])
+// A Hermitian 6x6 matrix as its diagonal and its lower triangle, row by row
+struct Herm6 {
+    double d[6];
+    cx<double> o[15];
+};
+__device__ __forceinline__ constexpr int tri(int i, int j) { return i * (i - 1) / 2 + j; }
+
+// A -> A^-1 by A = L D L^dag (no pivoting; the clover blocks are close to the
+// identity), all in registers: L, then M = L^-1 over it, then M^dag D^-1 M.
+// Returns false on a (near-)zero pivot.
+__device__ __forceinline__ bool herm_inverse6(Herm6 &A)
 {
-    cx<double> L[6][6];
-    double D[6];
     double amax = 0.0;
-    for (int i = 0; i < 6; ++i) amax = fmax(amax, fabs(A[i][i].r));
+#pragma unroll
+    for (int i = 0; i < 6; ++i) amax = fmax(amax, fabs(A.d[i]));
+    double inv[6];
+    bool ok = true;
+#pragma unroll
     for (int j = 0; j < 6; ++j) {
-        double dj = A[j][j].r;
-        for (int k = 0; k < j; ++k) dj -= (L[j][k].r * L[j][k].r + L[j][k].i * L[j][k].i) * D[k];
-        if (!(fabs(dj) > 1e-12 * amax) || !isfinite(dj)) return false;
-        D[j] = dj;
-        L[j][j] = mk(1.0, 0.0);
-        for (int i = j + 1; i < 6; ++i) {
-            cx<double> s = A[i][j];
-            for (int k = 0; k < j; ++k) {
-                const cx<double> t = D[k] * L[i][k];
-                s = s - t * conj(L[j][k]);
-            }
-            L[i][j] = (1.0 / dj) * s;
+        // column j: w_ij = A_ij - sum_k L_ik D_k conj(L_jk); L_ij = w_ij / D_j
+        cx<double> v[6];  // D_k conj(L_jk)
+        double dj = A.d[j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+            const cx<double> l = A.o[tri(j, k)];
+            v[k] = mk(A.d[k] * l.r, -(A.d[k] * l.i));
+            dj = ::fma(-v[k].r, l.r, dj);
+            dj = ::fma(v[k].i, l.i, dj);
         }
-        for (int i = 0; i < j; ++i) L[i][j] = mk(0.0, 0.0);
-    }
-    // M = L^-1 (unit lower triangular)
-    cx<double> M[6][6];
-    for (int j = 0; j < 6; ++j) {
-        for (int i = 0; i < 6; ++i) M[i][j] = mk(i == j ? 1.0 : 0.0, 0.0);
+        ok = ok && fabs(dj) > 1e-12 * amax && isfinite(dj);
+        A.d[j] = dj;
+        inv[j] = 1.0 / dj;
+#pragma unroll
         for (int i = j + 1; i < 6; ++i) {
-            cx<double> s = mk(0.0, 0.0);
-            for (int k = j; k < i; ++k) fma_(s, L[i][k], M[k][j]);
-            M[i][j] = -s;
+            cx<double> s = A.o[tri(i, j)];
+#pragma unroll
+            for (int k = 0; k < j; ++k) fma_(s, -A.o[tri(i, k)], v[k]);
+            A.o[tri(i, j)] = inv[j] * s;
         }
     }
-    // A^-1 = M^dag D^-1 M
-    for (int i = 0; i < 6; ++i)
-        for (int j = 0; j <= i; ++j) {
-            cx<double> s = mk(0.0, 0.0);
-            for (int k = i; k < 6; ++k) {
-                const cx<double> t = (1.0 / D[k]) * M[k][j];
-                fmac_(s, M[k][i], t);
-            }
-            Ai[i][j] = s;
-            Ai[j][i] = conj(s);
+    // M = L^-1 (unit lower triangular): M_ij = -(L_ij + sum_{j<k<i} L_ik M_kj),
+    // row by row (row i uses its own L entries and the finished rows above)
+#pragma unroll
+    for (int i = 1; i < 6; ++i) {
+        cx<double> row[6];
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            cx<double> s = A.o[tri(i, j)];
+#pragma unroll
+            for (int k = j + 1; k < i; ++k) fma_(s, A.o[tri(i, k)], A.o[tri(k, j)]);
+            row[j] = -s;
         }
-    return true;
+#pragma unroll
+        for (int j = 0; j < i; ++j) A.o[tri(i, j)] = row[j];
+    }
+    // (A^-1)_ij = sum_{k >= i} conj(M_ki) M_kj / D_k, i >= j: row i needs M's
+    // rows from i on only, so the result replaces M row by row
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        cx<double> w[6];  // conj(M_ki) / D_k
+#pragma unroll
+        for (int k = i + 1; k < 6; ++k) {
+            const cx<double> m = A.o[tri(k, i)];
+            w[k] = mk(inv[k] * m.r, -(inv[k] * m.i));
+        }
+        double dd = inv[i];
+#pragma unroll
+        for (int k = i + 1; k < 6; ++k) {
+            dd = ::fma(w[k].r, A.o[tri(k, i)].r, dd);
+            dd = ::fma(-w[k].i, A.o[tri(k, i)].i, dd);
+        }
+        A.d[i] = dd;
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            cx<double> s = inv[i] * A.o[tri(i, j)];
+#pragma unroll
+            for (int k = i + 1; k < 6; ++k) fma_(s, w[k], A.o[tri(k, j)]);
+            A.o[tri(i, j)] = s;
+        }
+    }
+    return ok;
 }
+
+struct CloverOut {
+    double2 *f64;
+    float4 *f32;
+    uint4 *f16;
+    void *x;  // fixed point, or float pairs where the links are out of its range
+    int *e;   // the fixed-point blocks' unit exponents, two per site
+};
 
 // store one block (diag reals then the lower triangle) in all precisions
-__device__ void store_block(const cx<double> A[6][6], int blk, int cb, double2 *p64, float4 *p32, uint4 *p16,
-                            float4 *pdf)
+template <bool FX>
+__device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, const CloverOut &O)
 {
+    double2 *p64 = O.f64;
+    float4 *p32 = O.f32;
+    uint4 *p16 = O.f16;
     double r[36];
-    for (int i = 0; i < 6; ++i) r[i] = A[i][i].r;
-    int k = 0;
-    for (int i = 1; i < 6; ++i)
-        for (int j = 0; j < i; ++j) {
-            r[6 + 2 * k] = A[i][j].r;
-            r[7 + 2 * k] = A[i][j].i;
-            ++k;
-        }
-    for (int q = 0; q < 18; ++q) p64[soa(cb, 36, blk * 18 + q)] = make_double2(r[2 * q], r[2 * q + 1]);
-    for (int q = 0; q < 18; ++q) pdf[soa(cb, 36, blk * 18 + q)] = df_pair(make_double2(r[2 * q], r[2 * q + 1]));
-    for (int q = 0; q < 9; ++q)
-        p32[soa(cb, 18, blk * 9 + q)] = make_float4((float)r[4 * q], (float)r[4 * q + 1], (float)r[4 * q + 2], (float)r[4 * q + 3]);
-    // halves: element e of the site = blk*36 + j; uint4 q holds elements 8q..8q+7
-    __half *h = reinterpret_cast<__half *>(p16);
-    for (int j = 0; j < 36; ++j) {
-        const int e = blk * 36 + j;
-        const int q = e >> 3, w = e & 7;
-        h[soa(cb, 9, q) * 8 + w] = __double2half(r[j]);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) r[i] = A.d[i];
+#pragma unroll
+    for (int k = 0; k < 15; ++k) {
+        r[6 + 2 * k] = A.o[k].r;
+        r[7 + 2 * k] = A.o[k].i;
     }
+#pragma unroll
+    for (int q = 0; q < 18; ++q) p64[soa(cb, 36, blk * 18 + q)] = make_double2(r[2 * q], r[2 * q + 1]);
+    if constexpr (FX) {
+        int E = 1;
+#pragma unroll
+        for (int k = 0; k < 36; ++k) E = max(E, fx_field(r[k]));
+#pragma unroll
+        for (int q = 0; q < 18; ++q)
+            ((int4 *)O.x)[soa(cb, 36, blk * 18 + q)] = fx_pack(fx_int(r[2 * q], E), fx_int(r[2 * q + 1], E));
+        O.e[2 * cb + blk] = E - (1023 + 54);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 18; ++q)
+            ((float4 *)O.x)[soa(cb, 36, blk * 18 + q)] = df_pair(make_double2(r[2 * q], r[2 * q + 1]));
+    }
+    float f[36];
+    unsigned w[18];
+#pragma unroll
+    for (int k = 0; k < 36; ++k) f[k] = (float)r[k];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) p32[soa(cb, 18, blk * 9 + q)] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+    // halves, rounded from FP64: element e = 36 blk + j of the site is half e & 7
+    // of uint4 e >> 3, so block 0 ends and block 1 begins in the middle of uint4 4
+#pragma unroll
+    for (int k = 0; k < 18; ++k)
+        w[k] = h2u(__halves2half2(__double2half(r[2 * k]), __double2half(r[2 * k + 1])));
+    const int q0 = blk ? 5 : 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int a = 4 * q;
+        p16[soa(cb, 9, q0 + q)] = blk ? make_uint4(w[a + 2], w[a + 3], w[a + 4], w[a + 5]) : make_uint4(w[a], w[a + 1], w[a + 2], w[a + 3]);
+    }
+    ((uint2 *)p16)[soa(cb, 9, 4) * 2 + blk] = blk ? make_uint2(w[0], w[1]) : make_uint2(w[16], w[17]);
 }
 
-__global__ void k_clover_build(Geom g, GaugePtr U, int par, double ck, double2 *F64, float4 *F32, uint4 *F16,
-                               float4 *FDF, double2 *Fi64, float4 *Fi32, uint4 *Fi16, float4 *FiDF, int *bad)
+// Both kernels replace one that walked the planes twice per site in FP64 with
+// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 4.9 ms
+// now (k_field_strength 3.3 ms at 1.2 instructions a clock and SM, waiting on
+// instruction fetch and two blocks an SM; k_clover_build 1.6 ms, the inverses
+// and conversions on the FP64 pipe).
+// Field strengths: thread = (site, plane), blockIdx.y the plane; planes (0,1)
+// (0,2) (0,3) (1,2) (1,3) (2,3).  FS: [plane][9][Vh_pad] doubles of one parity.
+template <class Alg>
+__global__ void __launch_bounds__(128, 2) k_field_strength(Geom g, GaugePtr U, int par, double *FS)
 {
-    const int cb = blockIdx.x * blockDim.x + threadIdx.x;
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
     if (cb >= g.Vh) return;
+    const int mu = w < 3 ? 0 : w < 5 ? 1 : 2, nu = w < 3 ? w + 1 : w < 5 ? w - 1 : 3;
     int c[4];
     site_coords(g, par, cb, c);
-    for (int blk = 0; blk < 2; ++blk) {
-        // blk 0: A_+ (gamma5 = +1), blk 1: A_-
-        const double se = blk == 0 ? -1.0 : 1.0;  // sign of E_l in B_l -+ E_l
-        cx<double> A[6][6];
-        for (int i = 0; i < 6; ++i)
-            for (int j = 0; j < 6; ++j) A[i][j] = mk(i == j ? 1.0 : 0.0, 0.0);
-        add_kron(A, ck, 3, field_strength(g, U, c, 0, 1));   // B_3 = F_xy
-        add_kron(A, -ck, 2, field_strength(g, U, c, 0, 2));  // B_2 = F_zx = -F_xz
-        add_kron(A, ck, 1, field_strength(g, U, c, 1, 2));   // B_1 = F_yz
-        add_kron(A, se * ck, 1, field_strength(g, U, c, 0, 3));  // E_1 = F_xt
-        add_kron(A, se * ck, 2, field_strength(g, U, c, 1, 3));  // E_2 = F_yt
-        add_kron(A, se * ck, 3, field_strength(g, U, c, 2, 3));  // E_3 = F_zt
-        // exact Hermiticity
-        for (int i = 0; i < 6; ++i) {
-            A[i][i].i = 0.0;
-            for (int j = 0; j < i; ++j) {
-                const cx<double> m = 0.5 * (A[i][j] + conj(A[j][i]));
-                A[i][j] = m;
-                A[j][i] = conj(m);
-            }
-        }
-        store_block(A, blk, cb, F64, F32, F16, FDF);
-        cx<double> Ai[6][6];
-        if (!herm_inverse6(A, Ai)) {
-            atomicExch(bad, 1);
-            for (int i = 0; i < 6; ++i)
-                for (int j = 0; j < 6; ++j) Ai[i][j] = mk(0.0, 0.0);
-        }
-        store_block(Ai, blk, cb, Fi64, Fi32, Fi16, FiDF);
+    double f[9];
+    field_strength<Alg>(g, U, par, c, mu, nu, f);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) FS[((size_t)w * 9 + k) * g.Vh_pad + cb] = f[k];
+}
+
+// The chiral block blockIdx.y (0: A_+, gamma5 = +1; 1: A_-) of every site of
+// a parity, assembled from the field strengths, stored, inverted, stored.
+template <bool FX>
+__global__ void __launch_bounds__(128) k_clover_build(Geom g, const double *__restrict__ FS, double ck, CloverOut F,
+                                                      CloverOut Fi, int *bad)
+{
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x, blk = blockIdx.y;
+    if (cb >= g.Vh) return;
+    const double se = blk == 0 ? -1.0 : 1.0;  // sign of E_l in B_l -+ E_l
+    auto fs = [&](int plane, int k) { return __ldg(FS + ((size_t)plane * 9 + k) * g.Vh_pad + cb); };
+    // G_l = B_l -+ E_l: B_1 = F_yz, B_2 = -F_xz, B_3 = F_xy, E = F_xt, F_yt, F_zt
+    double G1[9], G2[9], G3[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        G1[k] = ck * (fs(3, k) + se * fs(2, k));
+        G2[k] = ck * (se * fs(4, k) - fs(1, k));
+        G3[k] = ck * (fs(0, k) + se * fs(5, k));
     }
+    auto ent = [](const double G[9], int i, int j) {  // G_ij of the Hermitian G
+        if (i == j) return mk(G[i], 0.0);
+        const int k = 3 + 2 * (i + j - 1);
+        return i > j ? mk(G[k], G[k + 1]) : mk(G[k], -G[k + 1]);
+    };
+    // A = 1 + s_1 (x) G1 + s_2 (x) G2 + s_3 (x) G3, indexed 3 spin + colour
+    Herm6 A;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        A.d[i] = 1.0 + G3[i];
+        A.d[3 + i] = 1.0 - G3[i];
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            A.o[tri(i, j)] = ent(G3, i, j);
+            A.o[tri(3 + i, 3 + j)] = -ent(G3, i, j);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) A.o[tri(3 + i, j)] = ent(G1, i, j) + ti(ent(G2, i, j));
+    }
+    store_block<FX>(A, blk, cb, F);
+    if (!herm_inverse6(A)) {
+        atomicExch(bad, 1);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) A.d[i] = 0.0;
+#pragma unroll
+        for (int k = 0; k < 15; ++k) A.o[k] = mk(0.0, 0.0);
+    }
+    store_block<FX>(A, blk, cb, Fi);
 }
 
 int clover_build(qcd_ctx *c, double kappa, double csw)
 {
     GaugePtr U;
     for (int p = 0; p < 2; ++p) {
-        U.a[p] = c->U64[p];
+        U.a[p] = c->fx_links ? c->UX[p] : c->U64[p];
         U.b[p] = nullptr;
     }
     QCD_CUDA_CHECK(cudaMemsetAsync(c->flag_dev, 0, sizeof(int), c->stream));
+    auto out = [&](void *const f[4][2], int *const e[2], int par) {
+        return CloverOut{(double2 *)f[QCD_F64][par], (float4 *)f[QCD_F32][par], (uint4 *)f[QCD_F16][par],
+                         f[QCD_DF64][par], e[par]};
+    };
+    // the field strengths of one parity at a time
+    int rc = ensure_staging(c, (size_t)c->g.Vh_pad * 54 * sizeof(double));
+    if (rc) return rc;
+    double *FS = (double *)c->staging;
     for (int par = 0; par < 2; ++par) {
-        k_clover_build<<<nblocks(c->g.Vh, 64), 64, 0, c->stream>>>(
-            c->g, U, par, csw * kappa, (double2 *)c->C[QCD_F64][par], (float4 *)c->C[QCD_F32][par],
-            (uint4 *)c->C[QCD_F16][par], (float4 *)c->C[QCD_DF64][par], (double2 *)c->Ci[QCD_F64][par],
-            (float4 *)c->Ci[QCD_F32][par], (uint4 *)c->Ci[QCD_F16][par], (float4 *)c->Ci[QCD_DF64][par],
-            c->flag_dev);
+        const dim3 gs(nblocks(c->g.Vh, 128), 6), gc(nblocks(c->g.Vh, 128), 2);
+        const double ck = csw * kappa;
+        const CloverOut F = out(c->C, c->Cx, par), Fi = out(c->Ci, c->Cix, par);
+        if (c->fx_links) {
+            k_field_strength<AlgX><<<gs, 128, 0, c->stream>>>(c->g, U, par, FS);
+            k_clover_build<true><<<gc, 128, 0, c->stream>>>(c->g, FS, ck, F, Fi, c->flag_dev);
+        } else {
+            k_field_strength<AlgD><<<gs, 128, 0, c->stream>>>(c->g, U, par, FS);
+            k_clover_build<false><<<gc, 128, 0, c->stream>>>(c->g, FS, ck, F, Fi, c->flag_dev);
+        }
         QCD_CUDA_CHECK(cudaGetLastError());
     }
     int bad = 0;

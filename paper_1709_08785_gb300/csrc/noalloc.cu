@@ -22,7 +22,11 @@ namespace qcd {
 // library holds this array until the process exits.
 constexpr size_t NOALLOC_SCRATCH_BYTES = 24u << 20;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
+// behind it the two fixed-point exponents per site that the FP64 and DF64
+// operators' fields carry (or the FP16 norms)
+constexpr size_t NOALLOC_NORM_BYTES = NOALLOC_SCRATCH_BYTES / 48;
+
+static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + NOALLOC_NORM_BYTES];
 
 namespace {
 
@@ -94,19 +98,24 @@ extern "C" int qcd_dslash_eo_noalloc(qcd_ctx *c, void *out, const void *in, int 
     void *base = nullptr;
     int rc = scratch_address(dev, &base);
     if (rc) return rc;
+    // FP64 and DF64 hop in fixed point, as in qcd_dslash_eo
+    const bool fx = c->fx_links && (prec == QCD_F64 || prec == QCD_DF64);
     HVec vin, vout;
-    vin.prec = vout.prec = prec;
+    vin.prec = vout.prec = fx ? QCD_FX : prec;
     vin.p = base;
     vout.p = (char *)base + hb;
     if (nb) {
         vin.norm = (float *)((char *)base + 2 * hb);
         vout.norm = (float *)((char *)base + 2 * hb + nb);
+    } else if (fx) {
+        vin.norm = (float *)((char *)base + NOALLOC_SCRATCH_BYTES);
+        vout.norm = vin.norm + c->g.Vh_pad;
     }
     // timing events are created on demand by the profiler: keep it off here
     const bool prof = c->profiling;
     c->profiling = false;
     const int f32io = prec == QCD_F32 || prec == QCD_F16;  // QCD_DF64 takes complex128, as QCD_F64
-    rc = canon_to_half(c, prec, f32io, in, -1, vin, 1, 0);
+    rc = canon_to_half(c, vin.prec, f32io, in, -1, vin, 1, 0);
     if (rc == QCD_OK) {
         StencilCall s;
         s.prec = prec;
@@ -117,7 +126,7 @@ extern "C" int qcd_dslash_eo_noalloc(qcd_ctx *c, void *out, const void *in, int 
         s.in = vin;
         rc = launch_stencil(c, s);
     }
-    if (rc == QCD_OK) rc = half_to_canon(c, prec, f32io, vout, out, -1, 1, 0);
+    if (rc == QCD_OK) rc = half_to_canon(c, vout.prec, f32io, vout, out, -1, 1, 0);
     c->profiling = prof;
     return rc;
 }

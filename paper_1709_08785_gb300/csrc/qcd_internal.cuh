@@ -35,6 +35,10 @@
 
 namespace qcd {
 
+// internal precision: fixed-point spinor fields (fx.cuh), the input of the FP64
+// and DF64 operators
+constexpr int QCD_FX = 4;
+
 constexpr int SB = 32;  // sites per block of the site-blocked layout
 
 __host__ __device__ inline long pad_sites(long n) { return (n + SB - 1) / SB * SB; }
@@ -70,6 +74,12 @@ __device__ __forceinline__ double2 ld_stream(const double2 *p)
 {
     double2 v;
     QCD_LD_STREAM("v2.f64", "{%0, %1}, [%2]", "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int4 ld_stream(const int4 *p)
+{
+    int4 v;
+    QCD_LD_STREAM("v4.s32", "{%0, %1, %2, %3}, [%4]", "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p)
@@ -287,6 +297,7 @@ struct GaugePtr {
 
 struct CloverPtr {
     const void *p[2];  // per parity
+    const int *e[2];   // fixed-point blocks only: unit exponents, two per site
 };
 
 template <int P>

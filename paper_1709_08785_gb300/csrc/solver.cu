@@ -54,6 +54,7 @@ int read_state(qcd_ctx *c, int slot, SolverState *out)
 int dhat(qcd_ctx *c, int prec, HVec in, HVec out, HVec tmp, int red, HVec aux, SolverState *st, int fin,
          const int *done, int form)
 {
+    if (c->fx_links && (prec == QCD_F64 || prec == QCD_DF64)) TRY(get_work(c, QCD_FX, FX_TMP, &tmp));
     StencilCall s1;
     s1.prec = prec;
     s1.mode = M_MULT;
@@ -242,11 +243,13 @@ int residual_eo(Solver &S, HVec xe, HVec out, SolverState *st, int fin)
     // in the outer level's arithmetic
     qcd_ctx *c = S.c;
     Level &L = S.lv[0];
+    HVec tmp = L.tmp;
+    if (c->fx_links) TRY(get_work(c, QCD_FX, FX_TMP, &tmp));
     StencilCall s1;
     s1.prec = L.prec;
     s1.mode = M_MULT;
     s1.out_par = 1;
-    s1.out = L.tmp;
+    s1.out = tmp;
     s1.in = xe;
     TRY(launch_stencil(c, s1));
     StencilCall s2;
@@ -254,7 +257,7 @@ int residual_eo(Solver &S, HVec xe, HVec out, SolverState *st, int fin)
     s2.mode = L.form ? M_FULL : M_DHAT;
     s2.out_par = 0;
     s2.out = out;
-    s2.in = L.tmp;
+    s2.in = tmp;
     s2.y = xe;
     s2.a = -1.0;
     s2.cc = c->kappa * c->kappa;
@@ -391,6 +394,7 @@ int solve_eo(Solver &S, const void *b, void *x, double tol)
     }
     // b^_e = F_ee^-1 (b_e + kappa H_eo F_oo^-1 b_o)   (Eq. 6, Alg. 1 line 3),
     // for form 1 without the left F_ee^-1
+    if (c->fx_links) TRY(get_work(c, QCD_FX, FX_TMP, &tmpX));
     TRY(clover_apply_half(c, PX, 1, 1, boX, tmpX, 1, 0));
     {
         StencilCall s;
@@ -918,13 +922,15 @@ int solve_multi_eo(Multi &M, const void *b, void *x, double tol, std::vector<int
         TRY(blas_norm2(c, QCD_F64, ns, S.be, S.aux, FIN_SETN + 0));
         TRY(blas_norm2(c, QCD_F64, ns, S.bo, S.aux, FIN_ADDN + 0));
         // b^_e = F_ee^-1 (b_e + kappa H_eo F_oo^-1 b_o)   (Eq. 6), in FP64
-        TRY(clover_apply_half(c, QCD_F64, 1, 1, S.bo, S.re, 1, 0));
+        HVec tmpX = S.re;
+        if (c->fx_links) TRY(get_work(c, QCD_FX, FX_TMP, &tmpX));
+        TRY(clover_apply_half(c, QCD_F64, 1, 1, S.bo, tmpX, 1, 0));
         StencilCall s;
         s.prec = QCD_F64;
         s.mode = M_SRC;
         s.out_par = 0;
         s.out = S.bhat;
-        s.in = S.re;
+        s.in = tmpX;
         s.y = S.be;
         s.a = 1.0;
         s.cc = c->kappa;

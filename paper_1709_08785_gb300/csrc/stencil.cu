@@ -20,6 +20,7 @@ namespace qcd {
 
 // per-precision instantiations (stencil_<prec>.cu) and the multi-RHS kernel
 int dispatch_f64(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int v);
+int dispatch_fxout(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s);
 int dispatch_f32(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int v);
 int dispatch_f32_rg(const StencilCall &sc, const StencilArgs &A, int bx, cudaStream_t s, int v);
 int dispatch_f16(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int v);
@@ -67,14 +68,33 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     StencilArgs A;
     A.g = c->g;
     const int p = sc.prec;
+    // FP64 and DF64 in fixed point where the links allow it
+    A.fx = c->fx_links && (p == QCD_F64 || p == QCD_DF64);
+    const int pf = A.fx ? QCD_DF64 : p;  // the precision slot of the fields
     for (int par = 0; par < 2; ++par) {
-        A.U.a[par] = p == QCD_F64 ? c->U64[par] : p == QCD_F32 ? c->U32[par] : p == QCD_DF64 ? c->UDF[par] : c->U16a[par];
+        A.U.a[par] = pf == QCD_F64 ? c->U64[par] : pf == QCD_F32 ? c->U32[par] : pf == QCD_DF64 ? c->UX[par] : c->U16a[par];
         A.U.b[par] = c->U16b[par];
-        A.C.p[par] = (sc.mode == M_FULL) ? c->C[p][par] : c->Ci[p][par];
-        A.Cf.p[par] = c->C[p][par];
+        A.C.p[par] = (sc.mode == M_FULL) ? c->C[pf][par] : c->Ci[pf][par];
+        A.C.e[par] = (sc.mode == M_FULL) ? c->Cx[par] : c->Cix[par];
+        A.Cf.p[par] = c->C[pf][par];
+        A.Cf.e[par] = c->Cx[par];
+    }
+    A.y_fx = sc.y.prec == QCD_FX;
+    HVec in = sc.in;
+    if (A.fx && in.prec != QCD_FX) {
+        // the caller's input in FP64 or DF64: one conversion pass (each site
+        // converted once instead of by its eight neighbours)
+        if (sc.nrhs > 1) {
+            set_error_message("several right-hand sides in FP64 or DF64 take fixed-point input");
+            return QCD_EINVAL;
+        }
+        HVec fx;
+        int rc = get_work(c, QCD_FX, FX_IN, &fx);
+        if (rc || (rc = convert_half(c, in, fx, sc.done))) return rc;
+        in = fx;
     }
     A.out = sc.out.sp();
-    A.in = sc.in.sp();
+    A.in = in.sp();
     A.y = sc.y.sp();
     A.aux = sc.aux.sp();
     A.z = sc.z.sp();
@@ -181,6 +201,8 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     int rc;
     const int rv = variant;
     if (is_mrhs(sc)) rc = launch_mrhs(sc, A, nrhs, c->stream, rv, bx, c->num_sms);
+    else if (A.fx && sc.out.prec == QCD_FX && sc.red == R_NONE && (sc.mode == M_MULT || sc.mode == M_HOP))
+        rc = dispatch_fxout(sc, A, grid, block, c->stream);
     else if (p == QCD_F64) rc = dispatch_f64(sc, A, grid, block, c->stream, rv);
     else if (p == QCD_F32) rc = dispatch_f32(sc, A, grid, block, c->stream, rv);
     else if (p == QCD_DF64) rc = dispatch_df64(sc, A, grid, block, c->stream, rv);

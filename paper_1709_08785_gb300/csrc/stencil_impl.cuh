@@ -41,16 +41,35 @@ __device__ __forceinline__ void omega_sums(const Spinor<T> &o_, const Spinor<T> 
     red[2] += acc_cast<RA>(nn);
 }
 
+// the epilogue vector y at a site (FP64 and DF64: it may be a fixed-point field)
+template <int P>
+__device__ __forceinline__ void load_y(const StencilArgs &A, int cb, int r, Spinor<typename Prec<P>::T> &y)
+{
+    const SpinorPtr p = rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride);
+    if constexpr (P == QCD_F64 || P == QCD_DF64) {
+        if (A.y_fx) {
+            Spinor<double> d;
+            Prec<QCD_FX>::load(p, cb, d);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) y.s[k / 3][k % 3] = mk(typename Prec<P>::T(d.s[k / 3][k % 3].r), typename Prec<P>::T(d.s[k / 3][k % 3].i));
+            return;
+        }
+    }
+    Prec<P>::load(p, cb, y);
+}
+
 // One output site cb (right-hand side r): the hops, the mode's epilogue, the
 // site's contributions to the fused reductions.  The result is left in acc
 // for the caller to store (true), so that a kernel with a grid reduction
 // can publish its block's partial before its output stores are issued.
 // hop(acc) computes acc = H in at the site, clov(x) applies the site's clover
-// term (F^-1, or F for M_FULL) to x in place: from global memory, or from
-// the staged shared-memory copies.
-template <int P, int MODE, int RED, bool DAG, class RA, class HopF, class CloF>
+// term (F^-1, or F for M_FULL) to x in place, clov2(x) F for M_RECON.  (The
+// fixed-point forms apply F^-1 of M_MULT and M_DHAT inside hop, and clov is
+// empty there.)
+template <int P, int MODE, int RED, bool DAG, class RA, class HopF, class CloF, class Clo2F>
 __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r, RA red[4],
-                                             Spinor<typename Prec<P>::T> &acc, const HopF &hop, const CloF &clov)
+                                             Spinor<typename Prec<P>::T> &acc, const HopF &hop, const CloF &clov,
+                                             const Clo2F &clov2)
 {
     using T = typename Prec<P>::T;
     const SpinorPtr out = rhs_ptr(A.out, r, A.rhs_stride, A.norm_stride);
@@ -60,7 +79,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
     } else if (MODE == M_DHAT) {
         clov(acc);
         Spinor<T> y;
-        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
+        load_y<P>(A, cb, r, y);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), y);
         if (A.has_z) {
             Spinor<T> z;
@@ -73,7 +92,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
         }
     } else if (MODE == M_SRC) {
         Spinor<T> y;
-        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
+        load_y<P>(A, cb, r, y);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), y);
         clov(acc);
     } else if (MODE == M_RECON) {
@@ -81,12 +100,12 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
         // residual, b_o - (F_oo x_o - kappa H_oe x_e) = u - F x_o, from the
         // same hopping term
         Spinor<T> y;
-        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
+        load_y<P>(A, cb, r, y);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), y);  // u
         Spinor<T> xo = acc;
-        clover_any<P>(A.C, A.out_par, cb, xo);
+        clov(xo);
         Prec<P>::store(out, cb, xo);
-        clover_any<P>(A.Cf, A.out_par, cb, xo);  // F x_o
+        clov2(xo);  // F x_o
         if (RED == R_NORM) {
             T nn = 0;
 #pragma unroll
@@ -103,7 +122,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
         // also the second half of the gamma5-hermitian S_ee = F_ee - k^2 H_eo F_oo^-1 H_oe
         // (a = 1, cc = -k^2, y = the operator's input), with its dot products
         Spinor<T> y;
-        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
+        load_y<P>(A, cb, r, y);
         Spinor<T> fy = y;
         clov(fy);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), fy);
@@ -142,7 +161,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
     return true;
 }
 
-template <int P, int MODE, int RED, bool DAG>
+template <int P, int MODE, int RED, bool DAG, bool FX = false>
 __device__ __forceinline__ void stencil_body(const StencilArgs &A)
 {
     pdl_enter();
@@ -162,9 +181,21 @@ __device__ __forceinline__ void stencil_body(const StencilArgs &A)
     bool pending = false;
     if (cb < A.g.Vh) {
         const SpinorPtr in = rhs_ptr(A.in, r, A.rhs_stride, A.norm_stride);
+        constexpr bool FUSED = FX && (MODE == M_MULT || MODE == M_DHAT);
         pending = stencil_site<P, MODE, RED, DAG>(
-            A, cb, r, red, acc, [&](Spinor<T> &a) { hopping_any<P, DAG>(A.g, A.U, in, A.out_par, cb, a); },
-            [&](Spinor<T> &x) { clover_any<P>(A.C, A.out_par, cb, x); });
+            A, cb, r, red, acc,
+            [&](Spinor<T> &a) {
+                if constexpr (FX) fx_hop<DAG, FUSED, false>(A.g, A.U, A.C, in, A.out_par, cb, a);
+                else hopping_any<P, DAG>(A.g, A.U, in, A.out_par, cb, a);
+            },
+            [&](Spinor<T> &x) {
+                if constexpr (!FX) clover_any<P>(A.C, A.out_par, cb, x);
+                else if constexpr (!FUSED) fx_clover_spinor(A.C, A.out_par, cb, x);
+            },
+            [&](Spinor<T> &x) {
+                if constexpr (FX) fx_clover_spinor(A.Cf, A.out_par, cb, x);
+                else clover_any<P>(A.Cf, A.out_par, cb, x);
+            });
     }
     if constexpr (RED != R_NONE) grid_reduce<RED == R_OMEGA ? 3 : RED == R_DOT_AUX ? 2 : 1>(red, A.red);
     // the output after the partial: the release that publishes the block's
@@ -209,7 +240,7 @@ __device__ __forceinline__ void stencil_body_pipe(const StencilArgs &A)
     if (cb < A.g.Vh)
         pending = stencil_site<P, MODE, RED, DAG>(
             A, cb, 0, red, acc, [&](Spinor<float> &a) { hopping_pipe<P, DAG>(A.g, A.U, A.in, A.out_par, cb, a); },
-            [&](Spinor<float> &x) { clover_any<P>(A.C, A.out_par, cb, x); });
+            [&](Spinor<float> &x) { clover_any<P>(A.C, A.out_par, cb, x); }, [](Spinor<float> &) {});
     if constexpr (RED != R_NONE) grid_reduce<RED == R_OMEGA ? 3 : RED == R_DOT_AUX ? 2 : 1>(red, A.red);
     if (pending) Prec<P>::store(A.out, cb, acc);
 }
@@ -243,7 +274,7 @@ __device__ __forceinline__ void stencil_body_rg(const StencilArgs &A)
         const SpinorPtr in = rhs_ptr(A.in, r, A.rhs_stride, A.norm_stride);
         pending = stencil_site<P, MODE, RED, false>(
             A, cb, r, red, acc, [&](Spinor<T> &a) { hopping_any<P, false>(A.g, A.U, in, A.out_par, cb, a); },
-            [&](Spinor<T> &x) { clover_any<P>(A.C, A.out_par, cb, x); });
+            [&](Spinor<T> &x) { clover_any<P>(A.C, A.out_par, cb, x); }, [](Spinor<T> &) {});
     }
     RedArgs ra = A.red;
     ra.partials += (size_t)r * A.red_pstride;
@@ -295,6 +326,31 @@ __global__ void __maxnreg__(128) stencil_kernel_r128(StencilArgs A)
     stencil_body<P, MODE, RED, DAG>(A);
 }
 
+// FP64 and DF64 with the products on the integer pipe (fx.cuh), for links
+// within the fixed-point range: every field of SU(3) links
+template <int P, int MODE, int RED, bool DAG>
+__global__ void __launch_bounds__(384) stencil_kernel_fx(StencilArgs A)
+{
+    stencil_body<P, MODE, RED, DAG, true>(A);
+}
+
+// H in or F^-1 H in from a fixed-point field into one
+template <int MODE, bool DAG>
+__global__ void __launch_bounds__(384) stencil_kernel_fxout(StencilArgs A)
+{
+    pdl_enter();
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0;
+    if (A.done && *A.done) {
+        if (A.skip && lead) *A.skip = 1;
+        return;
+    }
+    if (A.skip && lead) *A.skip = 0;
+    const int r = threadIdx.y, cb = blockIdx.x * blockDim.x + threadIdx.x;
+    if (cb >= A.g.Vh) return;
+    fx_hop_store<DAG, MODE == M_MULT, false>(A.g, A.U, A.C, rhs_ptr(A.in, r, A.rhs_stride, A.norm_stride), A.out_par, cb,
+                                             rhs_ptr(A.out, r, A.rhs_stride, A.norm_stride));
+}
+
 // ---- host launcher -------------------------------------------------------
 template <int P, int MODE, int RED, bool DAG>
 static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int variant)
@@ -309,6 +365,12 @@ static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s
                 launch_pdl(stencil_kernel_pipe<P, MODE, RED, DAG>, grid, block, 0, s, A);
                 return;
             }
+        }
+    }
+    if constexpr (P == QCD_F64 || P == QCD_DF64) {
+        if (A.fx) {
+            launch_pdl(stencil_kernel_fx<P, MODE, RED, DAG>, grid, block, 0, s, A);
+            return;
         }
     }
     if constexpr (P == QCD_DF64) {

@@ -134,7 +134,9 @@ int tune_buffers(qcd_ctx *c, int prec, int nrhs, HVec *in, HVec *out, HVec *y, H
         v[k]->p = base + j * nrhs * hb;
         v[k]->norm = (float *)(base + nv * nrhs * hb + j * nrhs * nb);
     }
-    int rc = fill_pattern(c, prec, *in, nrhs, hvec_elems(c->g, prec), 11);
+    // FP64 and DF64 as the solvers run them: fixed-point input
+    if (c->fx_links && (prec == QCD_F64 || prec == QCD_DF64)) in->prec = QCD_FX;
+    int rc = fill_pattern(c, in->prec, *in, nrhs, hvec_elems(c->g, prec), 11);
     for (int k = 2; k < nv && rc == QCD_OK; ++k) rc = fill_pattern(c, prec, *v[k], nrhs, hvec_elems(c->g, prec), 11 + k);
     return rc;
 }
@@ -170,6 +172,7 @@ int tune_one(qcd_ctx *c, StencilCall s, qcd_ctx::TuneEntry *out)
     if (rc) return rc;
     s.in = in;
     s.out = o;
+    if (in.prec == QCD_FX && s.mode == M_MULT) s.out.prec = QCD_FX;
     s.y = y;
     s.aux = aux;
     s.z = aux;
@@ -183,7 +186,7 @@ int tune_one(qcd_ctx *c, StencilCall s, qcd_ctx::TuneEntry *out)
     const bool low = s.prec == QCD_F32 || s.prec == QCD_F16;
     const bool pipe = low && s.nrhs == 1 && (s.mode == M_MULT || s.mode == M_DHAT || s.mode == M_FULL);
     const bool mr = is_mrhs(s);
-    const int nv = mr ? 2 : pipe ? 3 : (low || s.prec == QCD_DF64) ? 2 : 1;
+    const int nv = mr ? 2 : pipe ? 3 : (low || (s.prec == QCD_DF64 && !c->fx_links)) ? 2 : 1;
     // sites per block; for the multi-RHS kernel the right-hand sides per block
     // (all, a half, a third, a quarter)
     const int bxs1[] = {64, 128, 256}, bxsn[] = {32, 64};
