@@ -417,7 +417,14 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
                 s.out = B.out;
                 s.in = B.in;
             }
+            // the result straight to the caller's vectors where the kernels can
+            if (canon_out(c, s, dst)) {
+                s.canon = dst;
+                s.canon_stride = (size_t)c->g.Vh * 24;
+            }
             rc = launch_stencil(c, s);
+            if (rc) return rc;
+            if (s.canon) continue;
         }
         if (rc) return rc;
         rc = half_to_canon(c, B.out.prec, f32io, B.out, dst, -1, nr, B.stride);

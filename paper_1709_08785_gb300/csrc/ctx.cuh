@@ -243,11 +243,17 @@ struct StencilCall {
     int done_stride = 0;
     size_t red_pstride = 0;
     bool rhs_grid = false;
+    // operator calls without a reduction, FP32, or FP64 / DF64 in fixed point: the
+    // result goes to canonical half vectors (complex64 / complex128, 16-byte
+    // aligned) canon_stride reals apart instead of out
+    void *canon = nullptr;
+    size_t canon_stride = 0;
 };
 int launch_stencil(qcd_ctx *c, const StencilCall &s);
 unsigned tune_key(const StencilCall &s);
 // F32 hopping / MULT on several right-hand sides: the shared-memory staged kernel
 bool is_mrhs(const StencilCall &s);
+bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst);  // whether launch_stencil takes s.canon = dst
 double stencil_bytes(const qcd_ctx *c, const StencilCall &s);  // algorithmic bytes of one launch
 int fill_pattern(qcd_ctx *c, int prec, HVec v, int nrhs, size_t rhs_stride, int seed);
 

@@ -116,17 +116,21 @@ extern "C" int qcd_dslash_eo_noalloc(qcd_ctx *c, void *out, const void *in, int 
     c->profiling = false;
     const int f32io = prec == QCD_F32 || prec == QCD_F16;  // QCD_DF64 takes complex128, as QCD_F64
     rc = canon_to_half(c, vin.prec, f32io, in, -1, vin, 1, 0);
+    StencilCall s;
     if (rc == QCD_OK) {
-        StencilCall s;
         s.prec = prec;
         s.mode = M_HOP;
         s.dagger = dagger ? 1 : 0;
         s.out_par = out_parity;
         s.out = vout;
         s.in = vin;
+        if (canon_out(c, s, out)) {  // as qcd_dslash_eo: the same kernels, the same bits
+            s.canon = out;
+            s.canon_stride = (size_t)c->g.Vh * 24;
+        }
         rc = launch_stencil(c, s);
     }
-    if (rc == QCD_OK) rc = half_to_canon(c, vout.prec, f32io, vout, out, -1, 1, 0);
+    if (rc == QCD_OK && !s.canon) rc = half_to_canon(c, vout.prec, f32io, vout, out, -1, 1, 0);
     c->profiling = prof;
     return rc;
 }

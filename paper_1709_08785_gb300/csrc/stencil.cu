@@ -63,6 +63,13 @@ bool is_mrhs(const StencilCall &sc)
     return sc.prec == QCD_F32 && sc.nrhs > 1 && sc.red == R_NONE && (sc.mode == M_MULT || sc.mode == M_HOP);
 }
 
+bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst)
+{
+    const bool fx = c->fx_links && (s.prec == QCD_F64 || s.prec == QCD_DF64);
+    return (fx || s.prec == QCD_F32) && s.red == R_NONE && (uintptr_t)dst % 16 == 0 &&
+           (s.mode == M_HOP || s.mode == M_MULT || s.mode == M_DHAT || s.mode == M_FULL);
+}
+
 int launch_stencil(qcd_ctx *c, const StencilCall &sc)
 {
     StencilArgs A;
@@ -111,6 +118,8 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     A.nrhs = sc.nrhs < 1 ? 1 : sc.nrhs;
     A.red = sc.red_args;
     A.done = sc.done;
+    A.canon = sc.canon;
+    A.canon_stride = sc.canon_stride;
     A.done_stride = sc.done_stride;
     A.red_pstride = sc.red_pstride;
     A.skip = nullptr;
@@ -178,6 +187,7 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
                 if (v->p) v->p = (char *)v->p + (size_t)r0 * sc.rhs_stride * 16;
                 if (v->norm) v->norm += (size_t)r0 * sc.norm_stride;
             }
+            if (g.canon) g.canon = (char *)g.canon + (size_t)r0 * sc.canon_stride * (p == QCD_F32 ? 4 : 8);
             const int rc = launch_stencil(c, g);
             if (rc != QCD_OK) return rc;
         }
@@ -201,6 +211,7 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     int rc;
     const int rv = variant;
     if (is_mrhs(sc)) rc = launch_mrhs(sc, A, nrhs, c->stream, rv, bx, c->num_sms);
+    else if (A.fx && sc.canon) rc = dispatch_f64(sc, A, grid, block, c->stream, rv);  // DF64's operators are the same
     else if (A.fx && sc.out.prec == QCD_FX && sc.red == R_NONE && (sc.mode == M_MULT || sc.mode == M_HOP))
         rc = dispatch_fxout(sc, A, grid, block, c->stream);
     else if (p == QCD_F64) rc = dispatch_f64(sc, A, grid, block, c->stream, rv);

@@ -881,6 +881,56 @@ __device__ __forceinline__ void fx_hop_store(const Geom &g, const GaugePtr &U, c
     fx_store(out, cb, x, E);
 }
 
+// ---- canonical vectors by 16-byte words ----------------------------------------
+// (a warp holds the 32 sites of one layout block, which follow one another in a
+// canonical half vector, or take every other place in a full one)
+template <class TC>
+constexpr int canon_words = 24 * sizeof(TC) / 16;  // 16-byte words per site: 6 or 12
+
+// word f of the warp's 32 canonical sites: site f / W of the block, word f % W;
+// lex is the calling lane's own site's position in the canonical vector
+template <int W>
+__device__ __forceinline__ size_t canon_word(int f, int lex, int &site, int &word)
+{
+    site = f / W;
+    word = f - site * W;
+    return (size_t)__shfl_sync(0xffffffffu, lex, site) * W + word;
+}
+
+__device__ __forceinline__ int canon_site(const Geom &g, int full, int cb)
+{
+    if (full < 0 || cb >= g.Vh) return cb;
+    int c[4];
+    site_coords(g, full, cb, c);
+    return lex_of(g, c);
+}
+
+// the calling warp's 32 spinors to a canonical vector (16-byte aligned) through
+// sm (32 (W + 1) words of the warp's own); every lane takes part, sites past
+// the lattice are not written
+template <class TC, class T>
+__device__ __forceinline__ void canon_store(const Geom &g, TC *dst, int full, int cb, const Spinor<T> &S, float4 *sm)
+{
+    constexpr int W = canon_words<TC>;
+    const int lane = threadIdx.x & 31;
+    TC *mine = (TC *)(sm + lane * (W + 1));
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        mine[2 * k] = (TC)S.s[k / 3][k % 3].r;
+        mine[2 * k + 1] = (TC)S.s[k / 3][k % 3].i;
+    }
+    __syncwarp();
+    const int lex = canon_site(g, full, cb);
+    float4 *q = (float4 *)dst;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+        const int f = 32 * j + lane;
+        int s, w;
+        const size_t at = canon_word<W>(f, lex, s, w);
+        if (cb - lane + s < g.Vh) q[at] = sm[f + f / W];
+    }
+}
+
 struct StencilArgs {
     Geom g;
     GaugePtr U;
@@ -901,6 +951,8 @@ struct StencilArgs {
     int nrhs;   // right-hand sides of the launch (multi-RHS: blockIdx.y selects a tile of them)
     int done_stride;      // lockstep solves: right-hand side r's done flag is done[r done_stride]
     size_t red_pstride;   // and its reduction's partials start red.partials + r red_pstride
+    void *canon;          // operator calls: the result in canonical half vectors, canon_stride
+    size_t canon_stride;  // reals apart, in place of out
 };
 
 // a host-supplied scalar in the kernel's arithmetic type (float: the

@@ -42,6 +42,9 @@ constexpr int MR_GRP = MR_COLS / 4;
 constexpr int MR_NB = 8 * SB;  // int [dir][site]
 constexpr size_t MR_BYTES = (size_t)(MR_GRP * SB + 8 * 3 * SB + 18 * SB) * sizeof(float4) + 2 * (MR_NB + SB) * sizeof(int);
 
+// float4 per warp that canonical output passes through
+constexpr int MR_OUT = SB * 7;
+
 // the staged words of this thread's site (s_col[group][site])
 struct Cols {
     const float4 *s_col;
@@ -281,9 +284,9 @@ __device__ __forceinline__ void mrhs_unpack(const float4 *raw_l, const float4 *r
 }
 
 // the stencil of (site cb0 + lane, right-hand side r) from the staged words
-template <int MODE, bool DAG>
+template <int MODE, bool DAG, bool CANON>
 __device__ __forceinline__ void mrhs_compute(const StencilArgs &A, const Cols &cols, const int *s_nb,
-                                             const int *s_tf, int cb0, int lane, int r)
+                                             const int *s_tf, int cb0, int lane, int r, float4 *s_out)
 {
     const int cb = cb0 + lane;
     // every thread takes part in the block's barriers: a thread past the
@@ -333,6 +336,13 @@ __device__ __forceinline__ void mrhs_compute(const StencilArgs &A, const Cols &c
             acc.s[3][c] = mk(P.Lr[c].x, P.Li[c].x);
         }
     }
+    if constexpr (CANON) {  // the warp's right-hand side is one: all lanes or none
+        if (r < A.nrhs) {
+            canon_store(A.g, (float *)A.canon + r * A.canon_stride, -1, cb, acc, s_out + threadIdx.y * MR_OUT);
+            __syncwarp();  // before the next site block's words
+        }
+        return;
+    }
     if (valid) Prec<QCD_F32>::store(out, cb, acc);
 }
 
@@ -341,7 +351,7 @@ __device__ __forceinline__ void mrhs_compute(const StencilArgs &A, const Cols &c
 // neighbours they share in L2); it copies the next site block's raw words
 // while it computes the current one, so only the on-chip unpack lies between
 // two site blocks.
-template <int MODE, bool DAG>
+template <int MODE, bool DAG, bool CANON = false>
 __device__ __forceinline__ void mrhs_body(const StencilArgs &A)
 {
     constexpr bool CL = MODE == M_MULT;
@@ -351,6 +361,7 @@ __device__ __forceinline__ void mrhs_body(const StencilArgs &A)
     float4 *raw_c = raw_l + MR_RL;
     int *s_nb = (int *)(raw_c + MR_RC);  // [2][8 SB]
     int *s_tf = s_nb + 2 * MR_NB;        // [2][SB]
+    float4 *s_out = (float4 *)(s_tf + 2 * SB);  // [threadIdx.y][MR_OUT], canonical output only
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nthr = blockDim.x * blockDim.y;
     const int nsb = (A.g.Vh + SB - 1) / SB;
@@ -373,7 +384,7 @@ __device__ __forceinline__ void mrhs_body(const StencilArgs &A)
         __syncthreads();
         const int nx = sb + gridDim.x;
         if (nx < nsb) mrhs_prefetch<CL>(A, nx * SB, raw_l, raw_c, s_nb + (buf ^ 1) * MR_NB, s_tf + (buf ^ 1) * SB, tid, nthr);
-        mrhs_compute<MODE, DAG>(A, cols, s_nb + buf * MR_NB, s_tf + buf * SB, sb * SB, threadIdx.x, r);
+        mrhs_compute<MODE, DAG, CANON>(A, cols, s_nb + buf * MR_NB, s_tf + buf * SB, sb * SB, threadIdx.x, r, s_out);
         cp_wait_all();
         __syncthreads();
         sb = nx;
@@ -391,6 +402,14 @@ template <int MODE, bool DAG>
 __global__ void __maxnreg__(80) mrhs_kernel_r80(StencilArgs A)
 {
     mrhs_body<MODE, DAG>(A);
+}
+
+// canonical output (operator calls): 24^3x48, 12 right-hand sides, MULT with both
+// conversions 861 us before, 537 with conversions through shared memory, 443 now
+template <int MODE, bool DAG>
+__global__ void __maxnreg__(80) mrhs_kernel_canon(StencilArgs A)
+{
+    mrhs_body<MODE, DAG, true>(A);
 }
 
 // the staging area is above the 48 KB default: opt in once per device and kernel
@@ -411,12 +430,12 @@ static void smem_opt_in(size_t bytes)
 template <auto K>
 static int resident(int threads, size_t smem)
 {
-    static std::atomic<int> occ[17];
-    const int t = threads / SB;
-    int n = t <= 16 ? occ[t].load(std::memory_order_relaxed) : 0;
+    static std::atomic<int> occ[34];
+    const int t = threads / SB + (smem > MR_BYTES ? 17 : 0);
+    int n = t < 34 ? occ[t].load(std::memory_order_relaxed) : 0;
     if (n <= 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K, threads, smem) != cudaSuccess || n < 1) n = 1;
-        if (t <= 16) occ[t].store(n, std::memory_order_relaxed);
+        if (t < 34) occ[t].store(n, std::memory_order_relaxed);
     }
     return n;
 }
@@ -429,17 +448,18 @@ int launch_mrhs(const StencilCall &sc, const StencilArgs &A, int nrhs, cudaStrea
 {
     if (tile < 1 || tile > nrhs) tile = nrhs;
     const int nsb = (int)nblocks(A.g.Vh, SB), gy = (nrhs + tile - 1) / tile;
-    const size_t smem = MR_BYTES;
+    const size_t smem = MR_BYTES + (A.canon ? (size_t)tile * MR_OUT * sizeof(float4) : 0);
 #define QCD_MR_K(KERN, MODE, DAG)                                                                      \
     do {                                                                                               \
-        smem_opt_in<KERN<MODE, DAG>>(smem);                                                            \
+        smem_opt_in<KERN<MODE, DAG>>(MR_BYTES + 16 * MR_OUT * sizeof(float4));                                                            \
         int gx = resident<KERN<MODE, DAG>>(SB * tile, smem) * num_sms / gy;                            \
         gx = gx < 1 ? 1 : gx > nsb ? nsb : gx;                                                         \
         KERN<MODE, DAG><<<dim3(gx, gy), dim3(SB, tile), smem, s>>>(A);                                 \
     } while (0)
 #define QCD_MR(MODE, DAG)                                                                              \
     do {                                                                                               \
-        if (variant == 1) QCD_MR_K(mrhs_kernel_r80, MODE, DAG);                                        \
+        if (A.canon) QCD_MR_K(mrhs_kernel_canon, MODE, DAG);                                           \
+        else if (variant == 1) QCD_MR_K(mrhs_kernel_r80, MODE, DAG);                                        \
         else QCD_MR_K(mrhs_kernel, MODE, DAG);                                                         \
     } while (0)
     if (sc.mode == M_MULT) {
