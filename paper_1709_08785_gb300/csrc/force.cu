@@ -16,6 +16,7 @@
 // to one link collects the two plaquettes of each plane through it with Y
 // inserted at each corner (a staple with insertions).
 #include "blas.cuh"
+#include "stencil.cuh"
 
 namespace qcd {
 
@@ -241,6 +242,296 @@ __global__ void k_force_link(Geom g, const double2 *__restrict__ U, const double
     for (int k = 0; k < 9; ++k) out[k] = make_double2(Gm.m[k / 3][k % 3].r, Gm.m[k / 3][k % 3].i);
 }
 
+// ---------------------------------------------------------------- fixed-point form
+// For links within the fixed-point range (fx.cuh) the clover part runs on the
+// integer pipe, with fewer products.  Y is anti-Hermitian, so with
+//   Z_nu(n) = U_nu(n) Y(n+nu) + Y(n) U_nu(n)   (one per direction and plane)
+// the four insertions into each of a link's two plaquettes in a plane pair up:
+//   G_mu(m) += +-[ U_nu(m) (U_mu(m+nu) Z_nu(m+mu)^dag) - Z_nu(m) (U_mu(m+nu) U_nu(m+mu)^dag)
+//                - Z_nu(q)^dag (U_mu(q) U_nu(q+mu)) + U_nu(q)^dag (U_mu(q) Z_nu(q+mu)) ],
+// q = m - nu, + for mu < nu: 8 products a plane instead of 18, and 24 a site for
+// Z.  The hopping part keeps FP64 and uses the projector's rank: with h the
+// two projected spin rows, sum_s ((1-g)lambda)_s conj(x_s) = sum_a h_a(lambda)
+// conj(h_a(x)).  16^3x32: 8.4 ms before, 1.21 ms now (Y 0.19, Z 0.18, links 0.84,
+// issue-bound at half a slot per cycle).
+
+// (sigma_p v)_a = ph v[perm]: ph as a power of i (the tables above)
+__device__ constexpr int sig_perm(int p, int a)
+{
+    return p == 0 ? a : p == 1 || p == 3 ? a ^ 1 : p == 5 ? a ^ 2 : 3 - a;
+}
+__device__ constexpr int sig_pow(int p, int a)  // 0: 1, 1: i, 2: -1, 3: -i
+{
+    return p == 0 || p == 5 ? ((a & 1) ? 0 : 2) : p == 1 ? ((a & 1) ? 1 : 3) : p == 4 ? ((a & 1) ? 3 : 1) : 2;
+}
+
+// Y of plane P at a site: (imaginary diagonal 0..2, then (re, im) of (1,0), (2,0),
+// (2,1)), anti-Hermitian: [plane][9][2][Vh_pad] by parity
+template <int P>
+__device__ __forceinline__ void force_y_plane(const Geom &g, const Spinor<double> &X, const Spinor<double> &L, double f,
+                                              double *out, size_t stride)
+{
+    C S[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            C acc = mk(0.0, 0.0);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const C v = X.s[sig_perm(P, a)][j];
+                const int ph = sig_pow(P, a);
+                fmac_(acc, L.s[a][i], ph == 0 ? v : ph == 1 ? ti(v) : ph == 2 ? -v : tmi(v));
+            }
+            S[i][j] = acc;
+        }
+    // y_ij = -i f (S_ji + conj(S_ij))
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[i * stride] = -2.0 * f * S[i][i].r;
+#pragma unroll
+    for (int i = 1; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            const C t = S[j][i] + conj(S[i][j]);
+            const int k = 3 + 2 * (i + j - 1);
+            out[k * stride] = f * t.i;
+            out[(k + 1) * stride] = -f * t.r;
+        }
+}
+
+__global__ void __launch_bounds__(128) k_force_Yx(Geom g, const double2 *__restrict__ x, const double2 *__restrict__ lam,
+                                                  double f, double *Y)
+{
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x, par = blockIdx.y;
+    if (cb >= g.Vh) return;
+    int c[4];
+    site_coords(g, par, cb, c);
+    const int s = lex_of(g, c);
+    Spinor<double> X, L;
+    load_spinor(x, s, X.s);
+    load_spinor(lam, s, L.s);
+    const size_t st = 2 * (size_t)g.Vh_pad;
+    double *o = Y + (size_t)par * g.Vh_pad + cb;
+    force_y_plane<0>(g, X, L, f, o, st);
+    force_y_plane<1>(g, X, L, f, o + 9 * st, st);
+    force_y_plane<2>(g, X, L, f, o + 18 * st, st);
+    force_y_plane<3>(g, X, L, f, o + 27 * st, st);
+    force_y_plane<4>(g, X, L, f, o + 36 * st, st);
+    force_y_plane<5>(g, X, L, f, o + 45 * st, st);
+}
+
+// a link, or a Z matrix, of the fixed-point fields (nc int4 a site, the matrix
+// at k0), daggered on loading
+__device__ __forceinline__ void load_m3x(const int4 *p, int cb, int nc, int k0, bool dg, M3x &r)
+{
+    const int sg = dg ? -1 : 1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int4 v = __ldg(p + soa(cb, nc, k0 + (dg ? 3 * j + i : 3 * i + j)));
+            r.m[i][j] = fxc{v.x, v.y, v.z * sg, v.w * sg};
+        }
+}
+
+// cb of the site c + a + b (unit steps, +-mu): every index of one parity
+__device__ __forceinline__ int cb_step(const Geom &g, const int c[4], int mu, int dm, int nu, int dn)
+{
+    int lex = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        int v = c[k] + (k == mu ? dm : 0) + (k == nu ? dn : 0);
+        v = v < 0 ? v + g.L[k] : v >= g.L[k] ? v - g.L[k] : v;
+        lex += v * g.st[k];
+    }
+    return lex >> 1;
+}
+
+// direction nu's Z of the plane it spans with mu: index 3 nu + (mu without nu)
+__device__ __forceinline__ int z_index(int nu, int mu) { return 3 * nu + (mu < nu ? mu : mu - 1); }
+
+struct ForceZ {
+    int4 *z[2];  // [parity]: 12 matrices a site
+    int *e;      // unit exponents [12][2][Vh_pad]
+};
+
+__global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const double *__restrict__ Y, ForceZ Z)
+{
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x, zi = blockIdx.y, par = blockIdx.z;
+    if (cb >= g.Vh) return;
+    const int nu = zi / 3, k3 = zi - 3 * nu, mu = k3 < nu ? k3 : k3 + 1;
+    const int plane = mu < nu ? plane_index(mu, nu) : plane_index(nu, mu);
+    int c[4];
+    site_coords(g, par, cb, c);
+    const int up = cb_step(g, c, nu, 1, nu, 0);
+    const size_t st = 2 * (size_t)g.Vh_pad;
+    const double *y0 = Y + (size_t)plane * 9 * st + (size_t)par * g.Vh_pad + cb;
+    const double *y1 = Y + (size_t)plane * 9 * st + (size_t)(1 - par) * g.Vh_pad + up;
+    double a[9], b[9];
+    int E = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        a[k] = __ldg(y0 + k * st);
+        b[k] = __ldg(y1 + k * st);
+        E = max(E, max(fx_field(a[k]), fx_field(b[k])));
+    }
+    // the anti-Hermitian matrix of nine reals, in units of 2^(E - 1023 - 54)
+    auto full = [&](const double v[9], M3x &m) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int4 d = fx_pack(0, fx_int(v[i], E));
+            m.m[i][i] = fx_unpack(d);
+#pragma unroll
+            for (int j = 0; j < i; ++j) {
+                const int k = 3 + 2 * (i + j - 1);
+                const int4 o = fx_pack(fx_int(v[k], E), fx_int(v[k + 1], E));
+                m.m[i][j] = fx_unpack(o);
+                m.m[j][i] = fxc{-o.x, -o.y, o.z, o.w};
+            }
+        }
+    };
+    M3x Um, M;
+    load_m3x((const int4 *)U.a[par], cb, 36, nu * 9, false, Um);
+    long long tr[3][3], tI[3][3];
+    full(b, M);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) fx_mul_elem<false, false>(Um, M, i, j, tr[i][j], tI[i][j]);
+    full(a, M);
+    unsigned mh = 0, ml = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            long long r, s;
+            fx_mul_elem<false, false>(M, Um, i, j, r, s);
+            tr[i][j] += r;
+            tI[i][j] += s;
+            const long long t[2] = {tr[i][j], tI[i][j]};
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const unsigned h = (unsigned)((unsigned long long)t[q] >> 32), sg = (unsigned)((int)h >> 31);
+                mh |= h ^ sg;
+                ml |= (unsigned)t[q] ^ sg;
+            }
+        }
+    // scaled below 2^55
+    const int up1 = (mh ? __clz(mh) : 32 + min(__clz(ml), 31)) - 1;
+    constexpr int DN = 63 - FX_BITS;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            Z.z[par][soa(cb, 108, zi * 9 + 3 * i + j)] = fx_pack((tr[i][j] << up1) >> DN, (tI[i][j] << up1) >> DN);
+    Z.e[(size_t)(zi * 2 + par) * g.Vh_pad + cb] = E == 0 ? FX_ZERO : E == 0x7ff ? FX_NAN : E - (1023 + 54) + DN - up1;
+}
+
+// G_mu(m) of the sites of parity blockIdx.z, direction blockIdx.y
+__global__ void __launch_bounds__(128, 3) k_force_link_x(Geom g, GaugePtr U, ForceZ Z, const double2 *__restrict__ x,
+                                                         const double2 *__restrict__ lam, double kappa, int with_clover,
+                                                         double2 *G)
+{
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y, par = blockIdx.z;
+    if (cb >= g.Vh) return;
+    int c[4];
+    site_coords(g, par, cb, c);
+    const int op = 1 - par;
+    const int mp = cb_step(g, c, mu, 1, mu, 0);
+    // ---- clover part in units of 2^E
+    long long tr[3][3], tI[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) tr[i][j] = tI[i][j] = 0;
+    int E = FX_ZERO;
+    if (with_clover) {
+#pragma unroll 1
+        for (int k = 0; k < 12; ++k) {  // four terms P (Q T) of each of three planes
+            const int n3 = k >> 2, t = k & 3, nu = n3 < mu ? n3 : n3 + 1;
+            const int zi = z_index(nu, mu);
+            // t = 0: U_nu(m), U_mu(m+nu), Z(m+mu)^dag      t = 1: Z(m), U_mu(m+nu), U_nu(m+mu)^dag
+            // t = 2: Z(q)^dag, U_mu(q), U_nu(q+mu)          t = 3: U_nu(q)^dag, U_mu(q), Z(q+mu)
+            const int q = cb_step(g, c, nu, -1, nu, 0);
+            const bool low = t >= 2, zp = t == 1 || t == 2;  // P is the Z matrix
+            const int4 *pp = zp ? Z.z[low ? op : par] : (const int4 *)U.a[low ? op : par];
+            const int4 *pt = zp ? (const int4 *)U.a[low ? par : op] : Z.z[low ? par : op];
+            const int sp = low ? q : cb, st = low ? cb_step(g, c, mu, 1, nu, -1) : mp;
+            const int sq = low ? q : cb_step(g, c, nu, 1, nu, 0);
+            const int e = __ldg(Z.e + (size_t)(zi * 2 + ((t == 1 || t == 3) ? par : op)) * g.Vh_pad + (zp ? sp : st));
+            M3x B;
+            {
+                M3x Q, T;
+                load_m3x((const int4 *)U.a[op], sq, 36, mu * 9, false, Q);
+                load_m3x(pt, st, zp ? 36 : 108, zp ? nu * 9 : zi * 9, !low, T);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        long long r, s;
+                        fx_mul_elem<false, false>(Q, T, i, j, r, s);
+                        B.m[i][j] = fx_unpack(fx_pack(r, s));
+                    }
+            }
+            M3x Pm;
+            load_m3x(pp, sp, zp ? 108 : 36, zp ? zi * 9 : nu * 9, low, Pm);
+            const int En = max(E, e), sa = fx_clamp63(En - E), sb = fx_clamp63(En - e);
+            const bool neg = zp != (mu > nu);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    long long r, s;
+                    fx_mul_elem<false, false>(Pm, B, i, j, r, s);
+                    r >>= sb;
+                    s >>= sb;
+                    tr[i][j] = (tr[i][j] >> sa) + (neg ? -r : r);
+                    tI[i][j] = (tI[i][j] >> sa) + (neg ? -s : s);
+                }
+            E = En;
+        }
+    }
+    // ---- hopping part
+    C Gm[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) Gm[i][j] = mk(0.0, 0.0);
+    int cp[4] = {c[0], c[1], c[2], c[3]};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (k == mu) cp[k] = c[k] + 1 == g.L[k] ? 0 : c[k] + 1;
+    const int m = lex_of(g, c), m1 = lex_of(g, cp);
+    // (1 - g_mu): lambda(m) (x) conj(x(m+mu)); (1 + g_mu): x(m) (x) conj(lambda(m+mu))
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        Spinor<double> A, B;
+        load_spinor(k ? x : lam, m, A.s);
+        load_spinor(k ? lam : x, m1, B.s);
+        C ha[2][3], hb[2][3];
+        project_rt(mu, k ? -1 : 1, A, ha);
+        project_rt(mu, k ? -1 : 1, B, hb);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+#pragma unroll
+                for (int a = 0; a < 2; ++a) fmac_(Gm[i][j], hb[a][j], ha[a][i]);
+    }
+    // mu = t: the projector's factor 2 (see project)
+    const double f = kappa * ((mu == 3 && c[3] == g.L[3] - 1) ? (double)g.t_bc : 1.0) * (mu == 3 ? 2.0 : 1.0);
+    const bool nan = E >= FX_NAN / 2;
+    const double s1 = nan ? __longlong_as_double(0x7ff8000000000000ll) : fx_pow2(E < -1000 ? -1000 : E);
+    const double s2 = E >= -1000 ? 1.0 : E < -2000 ? 0.0 : fx_pow2(E + 1000);
+    double2 *out = G + ((size_t)m * 4 + mu) * 9;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            out[3 * i + j] = make_double2(::fma(f, Gm[i][j].r, (double)tr[i][j] * s1 * s2),
+                                          ::fma(f, Gm[i][j].i, (double)tI[i][j] * s1 * s2));
+}
+
 // v -> gamma5 v on canonical full-lattice vectors, gamma5 = -[[0,1],[1,0]];
 // in and out may be the same buffer (no __restrict__: each thread reads its
 // site completely before writing it)
@@ -262,7 +553,11 @@ __global__ void k_gamma5(int V, const double2 *in, double2 *out)
 
 int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_canon)
 {
-    const size_t ybytes = (size_t)c->g.V * 6 * 9 * 16;
+    // FP64 form: Y as full matrices; fixed-point form: Y as nine reals, Z and its
+    // exponents
+    const size_t vp = (size_t)c->g.Vh_pad;
+    const size_t yx = 54 * 2 * vp * sizeof(double), zx = 2 * vp * 108 * 16;
+    const size_t ybytes = c->fx_links ? yx + zx + 24 * vp * sizeof(int) : (size_t)c->g.V * 6 * 9 * 16;
     if (c->force_bytes < ybytes) {
         if (c->force_buf) {
             cudaStreamSynchronize(c->stream);
@@ -275,6 +570,36 @@ int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_can
         int rc = dev_alloc(c, &c->force_buf, ybytes);
         if (rc) return rc;
         c->force_bytes = ybytes;
+    }
+    if (c->fx_links) {
+        double *Y = (double *)c->force_buf;
+        ForceZ Z;
+        Z.z[0] = (int4 *)((char *)c->force_buf + yx);
+        Z.z[1] = Z.z[0] + vp * 108;
+        Z.e = (int *)((char *)c->force_buf + yx + zx);
+        GaugePtr U;
+        for (int p = 0; p < 2; ++p) {
+            U.a[p] = c->UX[p];
+            U.b[p] = nullptr;
+        }
+        const unsigned nb = nblocks(c->g.Vh, 128);
+        const int with = c->csw != 0.0;
+        if (with) {
+            ProfScope p1(c, QCD_K_OTHER, 0.0);
+            k_force_Yx<<<dim3(nb, 2), 128, 0, c->stream>>>(c->g, (const double2 *)x, (const double2 *)lam,
+                                                            0.125 * c->csw * c->kappa, Y);
+            QCD_CUDA_CHECK(cudaGetLastError());
+        }
+        if (with) {
+            ProfScope p2(c, QCD_K_OTHER, 0.0);
+            k_force_Z<<<dim3(nb, 12, 2), 128, 0, c->stream>>>(c->g, U, Y, Z);
+            QCD_CUDA_CHECK(cudaGetLastError());
+        }
+        ProfScope p3(c, QCD_K_OTHER, 0.0);
+        k_force_link_x<<<dim3(nb, 4, 2), 128, 0, c->stream>>>(c->g, U, Z, (const double2 *)x, (const double2 *)lam,
+                                                              c->kappa, with, (double2 *)G);
+        QCD_CUDA_CHECK(cudaGetLastError());
+        return QCD_OK;
     }
     {
         ProfScope prof(c, QCD_K_OTHER, 0.0);

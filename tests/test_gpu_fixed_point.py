@@ -63,3 +63,61 @@ def test_unit_links_give_the_identity():
         # time by half a unit of at most 2 max|v| (per real)
         assert np.abs(out.cpu().numpy() - v).max() <= 4 * 2.0 ** -52 * np.abs(v).max()
     ctx.close()
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 4, 10)])
+@pytest.mark.parametrize("scale", [1.0, 1.3])
+@pytest.mark.parametrize("graded", [False, True])
+def test_force(dims, scale, graded):
+    """The link gradient in fixed point and, for links beyond its range, in FP64;
+    graded: sources falling by 2^-40 from site to site, as a propagator does."""
+    kappa, csw, t_bc = 0.12, 1.3, -1
+    V = inputs.volume(dims)
+    U = scale * inputs.random_gauge(dims, 0.3, 303)
+    x, lam = inputs.gaussian_source(dims, 304), inputs.gaussian_source(dims, 305)
+    if graded:
+        x = x * (2.0 ** (-40.0 * (np.arange(V) % 3)))[:, None, None]
+    ctx = make_ctx(dims, U, kappa, csw, t_bc)
+    G = torch.zeros(U.shape, dtype=torch.complex128, device="cuda")
+    ctx.force(torch.from_numpy(U).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(lam).cuda(), G)
+    torch.cuda.synchronize()
+    assert rel(G.cpu().numpy(), oracle.link_grad(dims, t_bc, U, kappa, csw, x, lam)) < TOL
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 3])
+@pytest.mark.parametrize("scale", [1.0, 1.3])
+def test_operators_on_graded_vectors(prec, scale):
+    """FP64 and DF64 D^ and S_ee of vectors that fall by 2^-30 from site to site
+    (each site its own exponent), zero sites among them."""
+    dims, kappa, csw, t_bc = (6, 2, 4, 10), 0.12, 1.0, -1
+    Vh = inputs.volume(dims) // 2
+    U = scale * inputs.random_gauge(dims, 0.3, 306)
+    v = inputs.gaussian_source(dims, 307)[:Vh] * (2.0 ** (-30.0 * (np.arange(Vh) % 4)))[:, None, None]
+    v[::7] = 0.0
+    ctx = make_ctx(dims, U, kappa, csw, t_bc)
+    F = oracle.clover_field(dims, U, kappa, csw)
+    Fi = oracle.invert_sites(F)
+    inp = torch.from_numpy(v).cuda()
+    out = torch.zeros_like(inp)
+    ctx.dhat(out, inp, prec)
+    assert rel(out.cpu().numpy(), oracle.dhat(dims, t_bc, U, Fi, kappa, v)) < 1e-13
+    ctx.schur_ee(out, inp, prec)
+    assert rel(out.cpu().numpy(), oracle.schur_ee(dims, t_bc, U, F, Fi, kappa, v)) < 1e-13
+    ctx.close()
+
+
+def test_non_finite_input_gives_non_finite_output():
+    dims = (4, 4, 4, 4)
+    ctx = make_ctx(dims, inputs.random_gauge(dims, 0.3, 308), 0.12, 1.0)
+    v = inputs.gaussian_source(dims, 309)[: inputs.volume(dims) // 2]
+    for bad in (np.nan, np.inf, -np.inf):
+        w = v.copy()
+        w[5, 1, 2] = bad
+        inp = torch.from_numpy(w).cuda()
+        out = torch.zeros_like(inp)
+        ctx.dhat(out, inp, 0)
+        got = out.cpu().numpy()
+        assert not np.isfinite(got[5]).all()  # D^ holds the input at its own site
+        assert np.isfinite(got).any()         # sites out of reach keep finite values
+    ctx.close()
