@@ -98,111 +98,68 @@ int gauge_convert(qcd_ctx *c, const void *U_dev)
 //     - [U_mu(n) P2 - U_mu(n-mu)^dag P2'] U_nu(n-nu),
 //   P1  = U_nu(n+mu) U_mu(n+nu)^dag,          P1' = U_nu(n-mu) U_mu(n-mu+nu),
 //   P2  = U_nu(n+mu-nu)^dag U_mu(n-nu)^dag,   P2' = U_nu(n-mu-nu)^dag U_mu(n-mu-nu)
-// (twelve products leaf by leaf).  The products run in an algebra: AlgX, the
-// fixed-point form of fx.cuh on the integer pipe, whose accumulators hold
-// every product of links with a Frobenius norm up to sqrt(3) (each of SU(3)
-// has exactly that); AlgD, FP64, for fields with larger links.
+// (twelve products leaf by leaf).  One loop runs over the four P, daggers taken
+// while loading, so that the code stays within the instruction cache (unrolled,
+// the warps waited on fetches: 1.65 ms a parity at 24^3x48 against 1.22).  The
+// products run in an algebra: AlgX, the fixed-point form of fx.cuh on the
+// integer pipe, whose accumulators hold every product of links with a Frobenius
+// norm up to sqrt(3) (each of SU(3) has exactly that); AlgD, FP64, for fields
+// with larger links.
 struct M3 {
     cx<double> m[3][3];
 };
 
 struct AlgX {
     using M = M3x;
-    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu)
+    using T = long long;
+    // the link, or its conjugate transpose
+    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu, bool dg)
     {
         const int4 *p = (const int4 *)U.a[par];
+        const int sg = dg ? -1 : 1;
         M r;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) r.m[k / 3][k % 3] = fx_unpack(__ldg(p + soa(cb, 36, mu * 9 + k)));
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int4 v = __ldg(p + soa(cb, 36, mu * 9 + (dg ? 3 * j + i : 3 * i + j)));
+                r.m[i][j] = fxc{v.x, v.y, v.z * sg, v.w * sg};
+            }
         return r;
     }
-    template <bool DA, bool DB>
-    static __device__ __forceinline__ M mul(const M &A, const M &B)
-    {
-        M C;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                long long r, s;
-                fx_mul_elem<DA, DB>(A, B, i, j, r, s);
-                C.m[i][j] = fx_unpack(fx_pack(r, s));
-            }
-        return C;
-    }
-    // op(A) B - C^dag D
-    static __device__ __forceinline__ M mul_sub(const M &A, const M &B, const M &C, const M &D)
-    {
-        M R;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                long long r, s, u, v;
-                fx_mul_elem<false, false>(A, B, i, j, r, s);
-                fx_mul_elem<true, false>(C, D, i, j, u, v);
-                R.m[i][j] = fx_unpack(fx_pack(r - u, s - v));
-            }
-        return R;
-    }
-    using T = long long;
-    template <bool DB>
     static __device__ __forceinline__ void elem(const M &A, const M &B, int i, int j, T &r, T &s)
     {
-        fx_mul_elem<false, DB>(A, B, i, j, r, s);
+        fx_mul_elem<false, false>(A, B, i, j, r, s);
     }
+    static __device__ __forceinline__ void set(M &A, int i, int j, T r, T s) { A.m[i][j] = fx_unpack(fx_pack(r, s)); }
     static __device__ __forceinline__ double value(T t) { return (double)t * (1.0 / (double)(1ll << FX_BITS)); }
 };
 
 struct AlgD {
     using M = M3;
-    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu)
+    using T = double;
+    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu, bool dg)
     {
-        Link<double> L;
-        Prec<QCD_F64>::load_link(U, par, cb, mu, L);
+        const double2 *p = (const double2 *)U.a[par];
         M r;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) r.m[k / 3][k % 3] = L.u[k / 3][k % 3];
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const double2 v = __ldg(p + soa(cb, 36, mu * 9 + (dg ? 3 * j + i : 3 * i + j)));
+                r.m[i][j] = mk(v.x, dg ? -v.y : v.y);
+            }
         return r;
     }
-    template <bool DA, bool DB>
-    static __device__ __forceinline__ cx<double> el(const M &A, const M &B, int i, int j)
-    {
-        cx<double> s = mk(0.0, 0.0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const cx<double> a = DA ? conj(A.m[k][i]) : A.m[i][k], b = DB ? conj(B.m[j][k]) : B.m[k][j];
-            fma_(s, a, b);
-        }
-        return s;
-    }
-    template <bool DA, bool DB>
-    static __device__ __forceinline__ M mul(const M &A, const M &B)
-    {
-        M C;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) C.m[i][j] = el<DA, DB>(A, B, i, j);
-        return C;
-    }
-    static __device__ __forceinline__ M mul_sub(const M &A, const M &B, const M &C, const M &D)
-    {
-        M R;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) R.m[i][j] = el<false, false>(A, B, i, j) - el<true, false>(C, D, i, j);
-        return R;
-    }
-    using T = double;
-    template <bool DB>
     static __device__ __forceinline__ void elem(const M &A, const M &B, int i, int j, T &r, T &s)
     {
-        const cx<double> z = el<false, DB>(A, B, i, j);
+        cx<double> z = mk(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) fma_(z, A.m[i][k], B.m[k][j]);
         r = z.r;
         s = z.i;
     }
+    static __device__ __forceinline__ void set(M &A, int i, int j, T r, T s) { A.m[i][j] = mk(r, s); }
     static __device__ __forceinline__ double value(T t) { return t; }
 };
 
@@ -213,6 +170,7 @@ __device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U,
                                                double F[9])
 {
     using M = typename Alg::M;
+    using T = typename Alg::T;
     auto at = [&](int dm, int dn) {  // cb of n + dm mu + dn nu
         int lex = 0;
 #pragma unroll
@@ -224,45 +182,74 @@ __device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U,
         }
         return lex >> 1;
     };
-    const int n = at(0, 0), op = 1 - par;
-    M R1, R2;
-    {
-        const M A = Alg::load(U, par, n, mu), B = Alg::load(U, op, at(-1, 0), mu);
+    const int op = 1 - par;
+    T Fd[3] = {0, 0, 0}, Fr[3] = {0, 0, 0}, Fi[3] = {0, 0, 0};  // of K - K^dag: Im diagonal; entries (1,0), (2,0), (2,1)
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {  // the bracket of U_nu(n)^dag, then of U_nu(n-nu)
+        M R;
         {
-            const M P1 = Alg::template mul<false, true>(Alg::load(U, op, at(1, 0), nu), Alg::load(U, op, at(0, 1), mu));
-            const M Q1 = Alg::template mul<false, false>(Alg::load(U, op, at(-1, 0), nu), Alg::load(U, par, at(-1, 1), mu));
-            R1 = Alg::mul_sub(A, P1, B, Q1);
+            T Rr[3][3], Ri[3][3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) Rr[i][j] = Ri[i][j] = 0;
+#pragma unroll 1
+            for (int k = 0; k < 2; ++k) {  // + U_mu(n) P, - U_mu(n-mu)^dag P'
+                const int dm = k ? -1 : 1;
+                M P;
+                {
+                    // X Y: U_nu(n+dm mu [-nu]) (daggered below) times U_mu of the other end
+                    const M X = Alg::load(U, h ? par : op, at(dm, h ? -1 : 0), nu, h);
+                    const M Y = Alg::load(U, k ? par : op, at(k ? -1 : 0, h ? -1 : 1), mu, !k);
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) {
+                            T r, s;
+                            Alg::elem(X, Y, i, j, r, s);
+                            Alg::set(P, i, j, r, s);
+                        }
+                }
+                const M A = Alg::load(U, k ? op : par, at(k ? -1 : 0, 0), mu, k);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        T r, s;
+                        Alg::elem(A, P, i, j, r, s);
+                        Rr[i][j] += k ? -r : r;
+                        Ri[i][j] += k ? -s : s;
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) Alg::set(R, i, j, Rr[i][j], Ri[i][j]);
         }
-        const M P2 = Alg::template mul<true, true>(Alg::load(U, par, at(1, -1), nu), Alg::load(U, op, at(0, -1), mu));
-        const M Q2 = Alg::template mul<true, false>(Alg::load(U, par, at(-1, -1), nu), Alg::load(U, par, at(-1, -1), mu));
-        R2 = Alg::mul_sub(A, P2, B, Q2);
+        const M B = Alg::load(U, h ? op : par, at(0, h ? -1 : 0), nu, !h);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            T r, s;
+            Alg::elem(R, B, i, i, r, s);
+            Fd[i] += h ? -s : s;
+#pragma unroll
+            for (int j = 0; j < i; ++j) {
+                T r2, s2;
+                Alg::elem(R, B, i, j, r, s);
+                Alg::elem(R, B, j, i, r2, s2);
+                const T dr = r - r2, di = s + s2;
+                Fr[i + j - 1] += h ? -dr : dr;
+                Fi[i + j - 1] += h ? -di : di;
+            }
+        }
     }
-    const M C = Alg::load(U, par, n, nu), D = Alg::load(U, op, at(0, -1), nu);
-    auto K = [&](int i, int j, typename Alg::T &r, typename Alg::T &s) {
-        typename Alg::T r2, s2;
-        Alg::template elem<true>(R1, C, i, j, r, s);
-        Alg::template elem<false>(R2, D, i, j, r2, s2);
-        r -= r2;
-        s -= s2;
-    };
     // (K - K^dag)/(8i)
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        typename Alg::T r, s;
-        K(i, i, r, s);
-        F[i] = 0.25 * Alg::value(s);
+        F[i] = 0.25 * Alg::value(Fd[i]);
+        F[3 + 2 * i] = 0.125 * Alg::value(Fi[i]);
+        F[4 + 2 * i] = -0.125 * Alg::value(Fr[i]);
     }
-#pragma unroll
-    for (int i = 1; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < i; ++j) {
-            typename Alg::T r, s, rt, sT;
-            K(i, j, r, s);
-            K(j, i, rt, sT);
-            const int k = 3 + 2 * (i + j - 1);
-            F[k] = 0.125 * Alg::value(s + sT);
-            F[k + 1] = -0.125 * Alg::value(r - rt);
-        }
 }
 
 // A Hermitian 6x6 matrix as its diagonal and its lower triangle, row by row
@@ -407,14 +394,14 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
 }
 
 // Both kernels replace one that walked the planes twice per site in FP64 with
-// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 4.9 ms
-// now (k_field_strength 3.3 ms at 1.2 instructions a clock and SM, waiting on
-// instruction fetch and two blocks an SM; k_clover_build 1.6 ms, the inverses
+// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 4.1 ms
+// now (k_field_strength 2.45 ms, issue-bound at 0.45 of a slot per cycle with
+// twelve warps an SM; k_clover_build 1.6 ms, the inverses
 // and conversions on the FP64 pipe).
 // Field strengths: thread = (site, plane), blockIdx.y the plane; planes (0,1)
 // (0,2) (0,3) (1,2) (1,3) (2,3).  FS: [plane][9][Vh_pad] doubles of one parity.
 template <class Alg>
-__global__ void __launch_bounds__(128, 2) k_field_strength(Geom g, GaugePtr U, int par, double *FS)
+__global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, int par, double *FS)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
     if (cb >= g.Vh) return;
