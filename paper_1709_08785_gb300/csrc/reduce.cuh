@@ -134,11 +134,59 @@ __device__ inline void finalize(int op, SolverState *st)
     }
 }
 
+// A sum beyond the warp, by the accumulator type A of the threads.  FP64 for
+// the FP64 and DF64 levels.  For the FP32 and FP16 levels, whose warp sums are
+// floats, a pair of floats (double-float, 2^-48): an FP64 instruction keeps a
+// warp scheduler's FP64 lanes busy for 64 cycles, and the FP64 tree of a block and
+// of its grid held each fused-dot kernel for some 2 us.
+template <class A>
+struct WideOf {
+    using type = double;
+};
+template <>
+struct WideOf<float> {
+    using type = df;
+};
+__device__ __forceinline__ double wide_shfl(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ __forceinline__ df wide_shfl(df v, int off)
+{
+    return df(__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off));
+}
+// a partial in its 8-byte slot
+__device__ __forceinline__ double wide_pack(double v) { return v; }
+__device__ __forceinline__ double wide_pack(df v)
+{
+    return __hiloint2double(__float_as_int(v.hi), __float_as_int(v.lo));
+}
+template <class W>
+__device__ __forceinline__ W wide_unpack(double d)
+{
+    if constexpr (std::is_same<W, df>::value)
+        return df(__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d)));
+    else return d;
+}
+
+// The sums over nw warps of the values src(warp, k), k < N <= 4, by one warp:
+// lane 8 k + j adds the warps j, j + 8, ..., then three steps add the eight
+// lanes of every k at once; all of lanes 8 k .. 8 k + 7 return sum k.
+template <int N, class W, class Src>
+__device__ __forceinline__ W warps_sum(int nw, const Src &src)
+{
+    const int lane = threadIdx.x + threadIdx.y * blockDim.x & 31, k = lane >> 3;
+    W t = W(0.f);
+    if (k < N)
+        for (int w = lane & 7; w < nw; w += 8) t = t + src(w, k);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) t = t + wide_shfl(t, off);
+    return t;
+}
+
 // Reduce N values over the grid; blocks may be 1-D or 2-D.  The per-thread
 // values and the warp stage are in the accumulator type A (float for the
 // FP32 and FP16 levels, whose sums feed FP32 recurrences: GB300's FP64 rate
 // is 1/64 of its FP32 rate, and per-thread FP64 adds slowed those kernels
-// in proportion to their size); warp sums and everything after are FP64.
+// in proportion to their size); the warp sums and everything after are in
+// WideOf<A>.
 // bidx / nblk: the block's index among the nblk blocks of this reduction
 // (blockIdx.x / gridDim.x, or another grid dimension when several
 // reductions share one launch); the block with index nblk - 1 is dispatched
@@ -146,7 +194,9 @@ __device__ inline void finalize(int op, SolverState *st)
 template <int N, class A>
 __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bidx, int nblk)
 {
-    __shared__ double sh[32][4];
+    using W = typename WideOf<A>::type;
+    __shared__ A sh[32][4];
+    __shared__ double sw[32][4];
     __shared__ int last;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nthr = blockDim.x * blockDim.y;
@@ -157,7 +207,8 @@ __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bi
         for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
     if (lane == 0)
 #pragma unroll
-        for (int k = 0; k < N; ++k) sh[wid][k] = (double)v[k];
+        for (int k = 0; k < N; ++k) sh[wid][k] = v[k];
+    const auto mine = [&](int w, int k) { return W(sh[w][k]); };
     if (bidx != nblk - 1) {
         // Every block but the last: warps 1.. post their sums and leave at
         // once (bar.arrive does not wait; their output stores proceed), warp
@@ -169,35 +220,24 @@ __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bi
             return;
         }
         asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-        double bsum[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            double t = lane < nw ? sh[lane][k] : 0.0;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-            bsum[k] = t;
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int k = 0; k < N; ++k) ra.partials[(size_t)bidx * 4 + k] = bsum[k];
-            // the partial ordered before the count; no reply awaited
+        const W t = warps_sum<N, W>(nw, mine);
+        if ((lane & 7) == 0 && (lane >> 3) < N) ra.partials[(size_t)bidx * 4 + (lane >> 3)] = wide_pack(t);
+        __syncwarp();
+        if (lane == 0)  // the partial ordered before the count; no reply awaited
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ra.counter) : "memory");
-        }
         return;
     }
+    // the solver state, a word a lane, on its way while the other blocks finish
+    constexpr int WORDS = sizeof(SolverState) / 8;
+    static_assert(sizeof(SolverState) % 8 == 0 && WORDS <= 32, "one warp moves the state");
+    __shared__ double sst[WORDS];
+    const double word = tid < WORDS ? __ldcg((const double *)ra.st + tid) : 0.0;
     __syncthreads();
     if (wid == 0) {
-        double bsum[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            double t = lane < nw ? sh[lane][k] : 0.0;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-            bsum[k] = t;
-        }
+        const W t = warps_sum<N, W>(nw, mine);
+        if ((lane & 7) == 0 && (lane >> 3) < N) ra.partials[(size_t)bidx * 4 + (lane >> 3)] = wide_pack(t);
+        __syncwarp();
         if (lane == 0) {
-#pragma unroll
-            for (int k = 0; k < N; ++k) ra.partials[(size_t)bidx * 4 + k] = bsum[k];
             // the highest-indexed block is dispatched last: it waits
             // (bounded) until every other block has counted
             const unsigned want = (unsigned)nblk - 1;
@@ -221,45 +261,57 @@ __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bi
         }
         return;
     }
-    double s[N];
+    // the partials in rows of four 8-byte slots, two slots a thread; eight loads
+    // in flight per thread, added as a tree
+    const bool hi = tid & 1;
+    const int rows = nthr >> 1;
+    W s0 = W(0.f), s1 = W(0.f);
+    if (N > 2 || !hi)
+        for (int b0 = tid >> 1; b0 < nblk; b0 += 8 * rows) {
+            double2 t[8];  // all zero bits are zero in either form
 #pragma unroll
-    for (int k = 0; k < N; ++k) s[k] = 0.0;
-    // eight independent loads in flight per thread, the last batch
-    // predicated: the partials arrive in ceil(G / 8 nthr) L2 round trips
-    const int G = nblk;
-    for (int b0 = tid; b0 < G; b0 += 8 * nthr) {
-        double t[8][N];
+            for (int u = 0; u < 8; ++u) {
+                const int b = b0 + u * rows;
+                t[u] = b < nblk ? __ldcg((const double2 *)ra.partials + (size_t)b * 2 + hi) : make_double2(0.0, 0.0);
+            }
+            W x[8], y[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int b = b0 + u * nthr;
+            for (int u = 0; u < 8; ++u) {
+                x[u] = wide_unpack<W>(t[u].x);
+                y[u] = wide_unpack<W>(t[u].y);
+            }
 #pragma unroll
-            for (int k = 0; k < N; ++k) t[u][k] = b < G ? __ldcg(ra.partials + (size_t)b * 4 + k) : 0.0;
+            for (int d = 4; d > 0; d >>= 1)
+#pragma unroll
+                for (int u = 0; u < d; ++u) {
+                    x[u] = x[u] + x[u + d];
+                    if (N > 1) y[u] = y[u] + y[u + d];
+                }
+            s0 = s0 + x[0];
+            if (N > 1) s1 = s1 + y[0];
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-            for (int k = 0; k < N; ++k) s[k] += t[u][k];
+    for (int off = 16; off > 1; off >>= 1) {
+        s0 = s0 + wide_shfl(s0, off);
+        if (N > 1) s1 = s1 + wide_shfl(s1, off);
     }
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s[k] += __shfl_down_sync(0xffffffffu, s[k], off);
+    if (lane < 2) {
+        sw[wid][2 * lane] = wide_pack(s0);
+        sw[wid][2 * lane + 1] = wide_pack(s1);
+    }
+    if (tid < WORDS) sst[tid] = word;
     __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < N; ++k) sh[wid][k] = s[k];
-    __syncthreads();
-    if (tid == 0) {
-        for (int k = 0; k < N; ++k) {
-            double t = 0.0;
-            for (int w = 0; w < nw; ++w) t += sh[w][k];
-            ra.st->sum[k] = t;
-        }
-        for (int k = N; k < 4; ++k) ra.st->sum[k] = 0.0;
-        finalize(ra.op, ra.st);
+    if (wid == 0) {
+        const W t = warps_sum<N, W>(nw, [&](int w, int k) { return wide_unpack<W>(sw[w][k]); });
+        SolverState *st = (SolverState *)sst;
+        if ((lane & 7) == 0) st->sum[lane >> 3] = (lane >> 3) < N ? (double)t : 0.0;
+        __syncwarp();
+        if (lane == 0) finalize(ra.op, st);
+        __syncwarp();
         // no fence: the kernel ends here, and its completion publishes the
         // state and the counter to the next kernel in stream order
-        *ra.counter = 0u;
+        if (lane < WORDS) ((double *)ra.st)[lane] = sst[lane];
+        if (lane == 0) *ra.counter = 0u;
     }
 }
 
