@@ -70,6 +70,28 @@ bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst)
            (s.mode == M_HOP || s.mode == M_MULT || s.mode == M_DHAT || s.mode == M_FULL);
 }
 
+// The launch shape where the tuner has no entry: sites per block (for the
+// multi-RHS kernel the right-hand sides per block) and register budget.
+// FP32 and FP16 with more threads than one wave at the compiler's budget holds
+// (five blocks of 128 an SM): the 80-register kernels, six such blocks, and
+// 256 sites per block where dot products are fused (half the partials).  Solves
+// with every such launch at one shape, budget / 80 registers: 20^3x40 10.43 / 9.98
+// ms, 24^3x48 18.55 / 17.65, FP16 inner level at 40^3x80 104.8 / 96.6.  Below, the
+// SMs are not full and spills only lengthen the chain: 16^3x32 5.74 / 5.91 ms,
+// 12^3x24 4.42 / 4.54.
+static void default_shape(const qcd_ctx *c, const StencilCall &sc, int &variant, int &bx)
+{
+    const int nrhs = sc.nrhs < 1 ? 1 : sc.nrhs;
+    variant = 0;
+    bx = 128;
+    if (nrhs > 1) bx = is_mrhs(sc) ? nrhs : nrhs <= 4 ? 64 : 32;
+    const bool low = sc.prec == QCD_F32 || sc.prec == QCD_F16;
+    if (low && !is_mrhs(sc) && (long)c->g.Vh * nrhs > 640L * c->num_sms) {
+        variant = 1;
+        if (sc.red != R_NONE) bx = 256;
+    }
+}
+
 int launch_stencil(qcd_ctx *c, const StencilCall &sc)
 {
     StencilArgs A;
@@ -140,7 +162,8 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
         StencilCall one = sc;
         one.nrhs = 1;
         one.rhs_grid = false;
-        int v = 0, b = 128;
+        int v, b;
+        default_shape(c, one, v, b);
         auto it = c->tune.find(tune_key(one));
         if (it != c->tune.end()) {
             v = it->second.variant;
@@ -157,8 +180,8 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
         QCD_CUDA_CHECK(cudaGetLastError());
         return QCD_OK;
     }
-    int bx = 128, variant = 0;  // bx: sites per block, or for the multi-RHS kernel the RHS tile
-    if (nrhs > 1) bx = is_mrhs(sc) ? nrhs : nrhs <= 4 ? 64 : 32;
+    int bx, variant;  // bx: sites per block, or for the multi-RHS kernel the RHS tile
+    default_shape(c, sc, variant, bx);
     if (sc.force_variant >= 0) {
         variant = sc.force_variant;
         bx = sc.force_bx;

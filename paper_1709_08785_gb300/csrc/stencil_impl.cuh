@@ -353,6 +353,12 @@ __global__ void __launch_bounds__(384) stencil_kernel_canon(StencilArgs A)
     stencil_body<P, MODE, R_NONE, DAG, FX, true>(A);
 }
 
+template <int P, int MODE, bool DAG, bool FX>
+__global__ void __maxnreg__(80) stencil_kernel_canon_r80(StencilArgs A)
+{
+    stencil_body<P, MODE, R_NONE, DAG, FX, true>(A);
+}
+
 // H in or F^-1 H in from a fixed-point field into one
 template <int MODE, bool DAG>
 __global__ void __launch_bounds__(384) stencil_kernel_fxout(StencilArgs A)
@@ -395,8 +401,10 @@ static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s
                   (P == QCD_F32 || P == QCD_F64)) {
         if (A.canon) {
             const size_t sm = (size_t)block.x * block.y * (P == QCD_F32 ? 7 : 13) * 16;
-            if constexpr (P == QCD_F32) launch_pdl(stencil_kernel_canon<P, MODE, DAG, false>, grid, block, sm, s, A);
-            else launch_canon_fx<P, MODE, DAG>(A, grid, block, sm, s);
+            if constexpr (P == QCD_F32) {
+                if (variant == 1) launch_pdl(stencil_kernel_canon_r80<P, MODE, DAG, false>, grid, block, sm, s, A);
+                else launch_pdl(stencil_kernel_canon<P, MODE, DAG, false>, grid, block, sm, s, A);
+            } else launch_canon_fx<P, MODE, DAG>(A, grid, block, sm, s);
             return;
         }
     }
