@@ -29,7 +29,7 @@
 
 #include "blas.cuh"
 #include "blas_ops.cuh"
-#include "stencil.cuh"
+#include "stencil_fx.cuh"
 
 namespace qcd {
 
@@ -262,22 +262,50 @@ __device__ void run_phase(const BatchArgs &A, int ph)
             break;
         case PH_OMULT:
             if constexpr (!OUTER) break;
-            if (site) {
-                if (pr.fx) {
-                    fx_hop_store<false, true, true>(pr.g, pr.UO, pr.CiO, pr.VX, 1, cb, pr.TX);
-                } else {
-                    Spinor<TO> a;
-                    hop_outer<PO>(pr, pr.Vv, 1, cb, a);
-                    Prec<PO>::store(pr.TMP, cb, a);
+            if (pr.fx) {  // two threads a site: the tile in two passes
+                const int row = fx_row();
+                for (int h = 0; h < 2; ++h) {
+                    const int s = lt * TILE + h * (TILE / 2) + fx_site(), sc = s < pr.g.Vh ? s : pr.g.Vh - 1;
+                    HalfSp<long long> acc;
+                    HalfSp<fx2> o;
+                    int e;
+                    fx_hop<false, true, true>(pr.g, pr.UO, pr.CiO, pr.VX, 1, sc, row, acc, e);
+                    fx_normalise(acc, e);
+                    fx_split(acc, o);
+                    if (s < pr.g.Vh) fx_store_half(pr.TX, s, row, o, e);
                 }
+            } else if (site) {
+                Spinor<TO> a;
+                hop_outer<PO>(pr, pr.Vv, 1, cb, a);
+                Prec<PO>::store(pr.TMP, cb, a);
             }
             break;
         case PH_ODHAT:
             if constexpr (!OUTER) break;
-            if (site) {
+            if (pr.fx) {
+                const int row = fx_row();
+                for (int h = 0; h < 2; ++h) {
+                    const int s = lt * TILE + h * (TILE / 2) + fx_site(), sc = s < pr.g.Vh ? s : pr.g.Vh - 1;
+                    HalfSp<long long> hop;
+                    HalfSp<TO> a, v;
+                    int e;
+                    fx_hop<false, true, true>(pr.g, pr.UO, pr.CiO, pr.TX, 0, sc, row, hop, e);
+                    fx_to_half(hop, e, a);
+                    load_half<PO>(pr.Vv, sc, row, v);
+                    axpby_half(a, TO(-pr.k2), a, TO(1.0), v);
+                    load_half<PO>(A.half == 0 ? pr.RT : pr.R, sc, row, v);
+                    if (s >= pr.g.Vh) continue;
+                    store_half<PO>(A.half == 0 ? pr.Q : pr.T, s, row, a);
+                    if (A.half == 0) {
+                        dot_half(v, a, acc[0], acc[1]);
+                    } else {
+                        dot_half(a, v, acc[0], acc[1]);
+                        norm_half(a, acc[2]);
+                    }
+                }
+            } else if (site) {
                 Spinor<TO> a, v;
-                if (pr.fx) fx_hop<false, true, true>(pr.g, pr.UO, pr.CiO, pr.TX, 0, cb, a);
-                else hop_outer<PO>(pr, pr.TMP, 0, cb, a);
+                hop_outer<PO>(pr, pr.TMP, 0, cb, a);
                 Prec<PO>::load(pr.Vv, cb, v);
                 axpby_sp(a, TO(-pr.k2), a, TO(1.0), v);
                 Prec<PO>::store(A.half == 0 ? pr.Q : pr.T, cb, a);
@@ -437,8 +465,11 @@ __global__ void __launch_bounds__(TILE, 3) batched_inner(BatchArgs A)
     run_phase<PO, PO, false>(A, PH_LIFT);
 }
 
+// one block of 256 threads an SM in any case above 128 registers: with all 255
+// the fixed-point hops keep the next hop's loads in flight (48 problems: 107.0
+// ms; 168 registers 118.6, two blocks at 128 114.4)
 template <int PO, int PX>
-__global__ void __launch_bounds__(TILE) batched_outer(BatchArgs A)
+__global__ void __maxnreg__(255) batched_outer(BatchArgs A)
 {
     run_phase<PO, PX, true>(A, PH_OMULT);
     QCD_SYNC();

@@ -11,7 +11,7 @@
 
 #include "blas.cuh"
 #include "blas_ops.cuh"
-#include "stencil.cuh"
+#include "stencil_fx.cuh"
 
 namespace qcd {
 
@@ -520,9 +520,9 @@ int convert_half(qcd_ctx *c, HVec src, HVec dst, const int *done)
 }
 
 // ---------------------------------------------------------------- clover apply
-template <int P, bool FX>
+template <int P>
 __global__ void k_clover_apply(Geom g, CloverPtr C, int par, SpinorPtr in, SpinorPtr out, size_t rhs_stride,
-                               size_t norm_stride, int out_fx)
+                               size_t norm_stride)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = blockIdx.y;
@@ -535,21 +535,33 @@ __global__ void k_clover_apply(Geom g, CloverPtr C, int par, SpinorPtr in, Spino
     o.norm = out.norm ? out.norm + r * norm_stride : nullptr;
     Spinor<T> S;
     Prec<P>::load(i, cb, S);
-    if constexpr (FX) {
-        Spinor<fx2> x;
-        Spinor<long long> y;
-        int e = fx_from_spinor(S, x);
-        fx_clover(C, par, cb, x, e, y);
-        if (out_fx) {
-            fx_normalise(y, e, x);
-            fx_store(o, cb, x, e);
-            return;
-        }
-        fx_to_spinor(y, e, S);
-    } else {
-        apply_clover<P>(C, par, cb, S);
-    }
+    apply_clover<P>(C, par, cb, S);
     Prec<P>::store(o, cb, S);
+}
+
+// FP64 and DF64 in fixed point, two threads a site (stencil_fx.cuh)
+template <int P>
+__global__ void __launch_bounds__(256) k_clover_apply_fx(Geom g, CloverPtr C, int par, SpinorPtr in, SpinorPtr out,
+                                                         size_t rhs_stride, size_t norm_stride, int out_fx)
+{
+    const int a = fx_row(), site = blockIdx.x * (blockDim.x >> 1) + fx_site(), r = blockIdx.y;
+    const bool live = site < g.Vh;  // the others take part in the exchanges
+    const int cb = live ? site : g.Vh - 1;
+    const SpinorPtr o = rhs_ptr(out, r, rhs_stride, norm_stride);
+    HalfSp<typename Prec<P>::T> s;
+    load_half<P>(rhs_ptr(in, r, rhs_stride, norm_stride), cb, a, s);
+    HalfSp<fx2> x;
+    HalfSp<long long> y;
+    int e = fx_from_half(s, x);
+    fx_clover(C, par, cb, a, x, e, y);
+    if (out_fx) {
+        fx_normalise(y, e);
+        fx_split(y, x);
+        if (live) fx_store_half(o, cb, a, x, e);
+    } else {
+        fx_to_half(y, e, s);
+        if (live) store_half<P>(o, cb, a, s);
+    }
 }
 
 int clover_apply_half(qcd_ctx *c, int prec, int parity, int inverse, HVec in, HVec out, int nrhs, size_t rhs_stride)
@@ -565,16 +577,16 @@ int clover_apply_half(qcd_ctx *c, int prec, int parity, int inverse, HVec in, HV
     const double cl = prec == QCD_F32 ? 288 : prec == QCD_F16 ? 144 : 576;
     ProfScope prof(c, QCD_K_OTHER, (cl + 2 * nrhs * sp_bytes(prec)) * c->g.Vh);
     const size_t ns = (size_t)c->g.Vh_pad;
-    if (fx && prec == QCD_F64)
-        k_clover_apply<QCD_F64, true><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns,
-                                                                  out.prec == QCD_FX);
-    else if (fx)
-        k_clover_apply<QCD_DF64, true><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns,
-                                                                   out.prec == QCD_FX);
-    else
-        PREC_SWITCH(prec, k_clover_apply<P, false><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(),
-                                                                               rhs_stride, ns, 0);
+    if (fx) {
+        const int of = out.prec == QCD_FX;
+        if (prec == QCD_F64)
+            k_clover_apply_fx<QCD_F64><<<grid, 256, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns, of);
+        else
+            k_clover_apply_fx<QCD_DF64><<<grid, 256, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns, of);
+    } else {
+        PREC_SWITCH(prec, k_clover_apply<P><<<grid, 128, 0, c->stream>>>(c->g, C, parity, in.sp(), out.sp(), rhs_stride, ns);
                     break);
+    }
     QCD_CUDA_CHECK(cudaGetLastError());
     return QCD_OK;
 }

@@ -20,7 +20,7 @@ namespace qcd {
 
 // per-precision instantiations (stencil_<prec>.cu) and the multi-RHS kernel
 int dispatch_f64(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int v);
-int dispatch_fxout(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s);
+int dispatch_fx(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s);
 int dispatch_f32(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int v);
 int dispatch_f32_rg(const StencilCall &sc, const StencilArgs &A, int bx, cudaStream_t s, int v);
 int dispatch_f16(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int v);
@@ -85,6 +85,9 @@ static void default_shape(const qcd_ctx *c, const StencilCall &sc, int &variant,
     variant = 0;
     bx = 128;
     if (nrhs > 1) bx = is_mrhs(sc) ? nrhs : nrhs <= 4 ? 64 : 32;
+    // fixed point (two threads a site, 168 registers): blocks of 128 threads, three
+    // an SM; 256 threads fit once (MULT at 24^3x48 175 / 223 us)
+    if (c->fx_links && (sc.prec == QCD_F64 || sc.prec == QCD_DF64)) bx = nrhs > 1 ? 32 : 64;
     const bool low = sc.prec == QCD_F32 || sc.prec == QCD_F16;
     if (low && !is_mrhs(sc) && (long)c->g.Vh * nrhs > 640L * c->num_sms) {
         variant = 1;
@@ -192,14 +195,16 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
             bx = it->second.bx;
         }
     }
-    if (!is_mrhs(sc) && bx * nrhs > 384) {
+    const int cap = A.fx ? 192 : 384;  // sites times right-hand sides of a block (fixed point: two threads each)
+    if (A.fx && bx > 64) bx = 64;  // a tuning cache may hold shapes of other kernels
+    if (!is_mrhs(sc) && bx * nrhs > cap) {
         // more right-hand sides than a block of the generic kernels holds:
         // launch them in groups (no reduction spans the groups)
         if (sc.red != R_NONE) {
             set_error_message("a fused reduction over %d right-hand sides is not supported", nrhs);
             return QCD_EINVAL;
         }
-        const int per = 384 / bx;
+        const int per = cap / bx;
         for (int r0 = 0; r0 < nrhs; r0 += per) {
             StencilCall g = sc;
             g.nrhs = nrhs - r0 < per ? nrhs - r0 : per;
@@ -234,9 +239,7 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     int rc;
     const int rv = variant;
     if (is_mrhs(sc)) rc = launch_mrhs(sc, A, nrhs, c->stream, rv, bx, c->num_sms);
-    else if (A.fx && sc.canon) rc = dispatch_f64(sc, A, grid, block, c->stream, rv);  // DF64's operators are the same
-    else if (A.fx && sc.out.prec == QCD_FX && sc.red == R_NONE && (sc.mode == M_MULT || sc.mode == M_HOP))
-        rc = dispatch_fxout(sc, A, grid, block, c->stream);
+    else if (A.fx) rc = dispatch_fx(sc, A, grid, dim3(2 * bx, nrhs), c->stream);
     else if (p == QCD_F64) rc = dispatch_f64(sc, A, grid, block, c->stream, rv);
     else if (p == QCD_F32) rc = dispatch_f32(sc, A, grid, block, c->stream, rv);
     else if (p == QCD_DF64) rc = dispatch_df64(sc, A, grid, block, c->stream, rv);

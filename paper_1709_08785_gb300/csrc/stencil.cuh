@@ -643,244 +643,6 @@ __device__ __forceinline__ void clover_any(const CloverPtr &cl, int par, int cb,
     else apply_clover<P>(cl, par, cb, s);
 }
 
-// ---- fixed-point forms (fx.cuh) ------------------------------------------------
-// The hopping term and the clover term for FP64 and DF64 with the products on
-// the integer pipe.  The input is a fixed-point field (each site converted
-// once, not by each of its eight neighbours).  24^3x48, L2 evicted: MULT 260 us
-// (FP64 698, float pairs 265), FP64 second half of b^ 347 (726), x_o with its
-// residual 488 (959), even residual 381 (774).  168 registers, twelve warps an
-// SM waiting on their loads; 128 registers spill (290 us), staging the next
-// hop's words in shared memory by cp.async is slower (287 against 250 us).  |acc| stays below 2^63: a
-// projected pair is below 2^58, a link of Frobenius norm sqrt(3) takes it to
-// 2^59.2 in the result's units, eight hops to 2^62.2.
-
-// acc += hop D (D = 2 mu + backward, S the sign of its projector), in units of
-// 2^(E - 55 + 56); sh = E - the neighbour's exponent
-template <int D, int S, bool COH>
-__device__ __forceinline__ void fx_hop1(const GaugePtr &U, const SpinorPtr &in, int out_par, int cb, int nb, bool flip,
-                                        int sh, Spinor<long long> &acc)
-{
-    constexpr int MU = D >> 1;
-    constexpr bool BWD = D & 1;
-    cx<fx2> h[2][3];
-    {
-        Spinor<fx2> psi;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const int4 *p = (const int4 *)in.p + soa(nb, 12, k);
-            const int4 v = COH ? __ldcg(p) : __ldg(p);
-            psi.s[k / 3][k % 3] = cx<fx2>{fx2{v.x, v.y}, fx2{v.z, v.w}};
-        }
-        project<MU, S>(psi, h);
-    }
-    const int4 *lp = (const int4 *)U.a[BWD ? 1 - out_par : out_par];
-    const int ls = BWD ? nb : cb;
-    cx<long long> q[2][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        long long mr[2], mi[2], hr[2], hi[2];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            // U_ij, or conj(U_ji) for the backward hop
-            const int4 u = ld_stream(lp + soa(ls, 36, MU * 9 + (BWD ? 3 * j + i : 3 * i + j)));
-            const int pih = BWD ? -u.z : u.z, pil = BWD ? -u.w : u.w, nih = BWD ? u.z : -u.z, nil = BWD ? u.w : -u.w;
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const cx<fx2> x = h[a][j];
-                if (j == 0) {
-                    mr[a] = fx_mul(u.x, x.r.l);
-                    mi[a] = fx_mul(u.x, x.i.l);
-                    hr[a] = fx_mul(u.x, x.r.h);
-                    hi[a] = fx_mul(u.x, x.i.h);
-                } else {
-                    fx_mac(mr[a], u.x, x.r.l);
-                    fx_mac(mi[a], u.x, x.i.l);
-                    fx_mac(hr[a], u.x, x.r.h);
-                    fx_mac(hi[a], u.x, x.i.h);
-                }
-                fx_mac(mr[a], u.y, x.r.h);
-                fx_mac(mi[a], u.y, x.i.h);
-                fx_mac(hr[a], nih, x.i.h);
-                fx_mac(hi[a], pih, x.r.h);
-                fx_mac(mr[a], nih, x.i.l);
-                fx_mac(mi[a], pih, x.r.l);
-                fx_mac(mr[a], nil, x.i.h);
-                fx_mac(mi[a], pil, x.r.h);
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-            q[a][i] = mk((hr[a] + (mr[a] >> FX_LIMB)) >> sh, (hi[a] + (mi[a] >> FX_LIMB)) >> sh);
-    }
-    if (MU == 3 && flip) {
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) q[a][i] = -q[a][i];
-    }
-    expand<MU, S>(acc, q);
-}
-
-// acc 2^E = H in at site cb
-template <bool DAG, bool COH>
-__device__ __forceinline__ void fx_hopping(const Geom &g, const GaugePtr &U, const SpinorPtr &in, int out_par, int cb,
-                                           Spinor<long long> &acc, int &E)
-{
-    int c[4];
-    site_coords(g, out_par, cb, c);
-    const int lex = lex_of(g, c);
-    constexpr int SF = DAG ? -1 : 1;
-    auto nb = [&](int d) { return lex_hop(g, lex, c, d >> 1, (d & 1) ? -1 : +1) >> 1; };
-    auto ex = [&](int d) { return COH ? __ldcg((const int *)in.norm + nb(d)) : __ldg((const int *)in.norm + nb(d)); };
-    E = FX_ZERO;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) E = max(E, ex(d));
-    const bool up = g.t_bc < 0 && c[3] == g.L[3] - 1, dn = g.t_bc < 0 && c[3] == 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) acc.s[a][i] = mk(0ll, 0ll);
-    fx_hop1<0, SF, COH>(U, in, out_par, cb, nb(0), false, fx_clamp63(E - ex(0)), acc);
-    fx_hop1<1, -SF, COH>(U, in, out_par, cb, nb(1), false, fx_clamp63(E - ex(1)), acc);
-    fx_hop1<2, SF, COH>(U, in, out_par, cb, nb(2), false, fx_clamp63(E - ex(2)), acc);
-    fx_hop1<3, -SF, COH>(U, in, out_par, cb, nb(3), false, fx_clamp63(E - ex(3)), acc);
-    fx_hop1<4, SF, COH>(U, in, out_par, cb, nb(4), false, fx_clamp63(E - ex(4)), acc);
-    fx_hop1<5, -SF, COH>(U, in, out_par, cb, nb(5), false, fx_clamp63(E - ex(5)), acc);
-    fx_hop1<6, SF, COH>(U, in, out_par, cb, nb(6), up, fx_clamp63(E - ex(6)), acc);
-    fx_hop1<7, -SF, COH>(U, in, out_par, cb, nb(7), dn, fx_clamp63(E - ex(7)), acc);
-    // links are in units of 2^-55, a product is cut by 2^56
-    if (E > FX_ZERO / 2 && E < FX_NAN / 2) E += 2 * FX_LIMB - FX_BITS;
-}
-
-// out 2^e = the clover term of x 2^e (the site's two blocks have their unit
-// exponents in C.e)
-__device__ __forceinline__ void fx_clover(const CloverPtr &C, int par, int cb, const Spinor<fx2> &x, int &e,
-                                          Spinor<long long> &out)
-{
-    const int4 *p = (const int4 *)C.p[par];
-    const int e0 = __ldg(C.e[par] + 2 * cb), e1 = __ldg(C.e[par] + 2 * cb + 1), em = max(e0, e1);
-#pragma unroll 1
-    for (int blk = 0; blk < 2; ++blk) {
-        const int sh = fx_clamp63(em - (blk ? e1 : e0));
-        cx<fx2> v[6];
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) v[3 * a + i] = blk ? x.s[a][i] + x.s[a + 2][i] : x.s[a][i] - x.s[a + 2][i];
-        long long mr[6], mi[6], hr[6], hi[6];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int4 d = ld_stream(p + soa(cb, 36, blk * 18 + k));
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const int i = 2 * k + b, dh = b ? d.z : d.x, dl = b ? d.w : d.y;
-                mr[i] = fx_mul(dh, v[i].r.l);
-                mi[i] = fx_mul(dh, v[i].i.l);
-                hr[i] = fx_mul(dh, v[i].r.h);
-                hi[i] = fx_mul(dh, v[i].i.h);
-                fx_mac(mr[i], dl, v[i].r.h);
-                fx_mac(mi[i], dl, v[i].i.h);
-            }
-        }
-        int k = 0;
-#pragma unroll
-        for (int i = 1; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j < i; ++j) {
-                const int4 o = ld_stream(p + soa(cb, 36, blk * 18 + 3 + k));
-                const int nih = -o.z, nil = -o.w;
-                // y_i += A_ij v_j
-                fx_mac(mr[i], o.x, v[j].r.l);
-                fx_mac(mr[i], o.y, v[j].r.h);
-                fx_mac(mr[i], nih, v[j].i.l);
-                fx_mac(mr[i], nil, v[j].i.h);
-                fx_mac(mi[i], o.x, v[j].i.l);
-                fx_mac(mi[i], o.y, v[j].i.h);
-                fx_mac(mi[i], o.z, v[j].r.l);
-                fx_mac(mi[i], o.w, v[j].r.h);
-                fx_mac(hr[i], o.x, v[j].r.h);
-                fx_mac(hr[i], nih, v[j].i.h);
-                fx_mac(hi[i], o.x, v[j].i.h);
-                fx_mac(hi[i], o.z, v[j].r.h);
-                // y_j += conj(A_ij) v_i
-                fx_mac(mr[j], o.x, v[i].r.l);
-                fx_mac(mr[j], o.y, v[i].r.h);
-                fx_mac(mr[j], o.z, v[i].i.l);
-                fx_mac(mr[j], o.w, v[i].i.h);
-                fx_mac(mi[j], o.x, v[i].i.l);
-                fx_mac(mi[j], o.y, v[i].i.h);
-                fx_mac(mi[j], nih, v[i].r.l);
-                fx_mac(mi[j], nil, v[i].r.h);
-                fx_mac(hr[j], o.x, v[i].r.h);
-                fx_mac(hr[j], o.z, v[i].i.h);
-                fx_mac(hi[j], o.x, v[i].i.h);
-                fx_mac(hi[j], nih, v[i].r.h);
-                ++k;
-            }
-        // up = (y+ + y-)/2, dn = (y- - y+)/2, the 1/2 in the exponent
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int m = 3 * a + i;
-                const cx<long long> y = mk((hr[m] + (mr[m] >> FX_LIMB)) >> sh, (hi[m] + (mi[m] >> FX_LIMB)) >> sh);
-                if (blk == 0) {
-                    out.s[a][i] = y;
-                    out.s[a + 2][i] = -y;
-                } else {
-                    out.s[a][i] = out.s[a][i] + y;
-                    out.s[a + 2][i] = out.s[a + 2][i] + y;
-                }
-            }
-    }
-    if (e > FX_ZERO / 2 && e < FX_NAN / 2) e += em + 2 * FX_LIMB - 1;
-}
-
-// the clover term of a spinor in T's arithmetic, in place
-template <class T>
-__device__ __forceinline__ void fx_clover_spinor(const CloverPtr &C, int par, int cb, Spinor<T> &s)
-{
-    Spinor<fx2> x;
-    Spinor<long long> y;
-    int e = fx_from_spinor(s, x);
-    fx_clover(C, par, cb, x, e, y);
-    fx_to_spinor(y, e, s);
-}
-
-// out = H in, or with CLOVER the clover term (F^-1, or what C holds) of it, in
-// the arithmetic type T
-template <bool DAG, bool CLOVER, bool COH, class T>
-__device__ __forceinline__ void fx_hop(const Geom &g, const GaugePtr &U, const CloverPtr &C, const SpinorPtr &in,
-                                       int out_par, int cb, Spinor<T> &out)
-{
-    Spinor<long long> acc;
-    int E;
-    fx_hopping<DAG, COH>(g, U, in, out_par, cb, acc, E);
-    if constexpr (CLOVER) {
-        Spinor<fx2> x;
-        fx_normalise(acc, E, x);
-        fx_clover(C, out_par, cb, x, E, acc);
-    }
-    fx_to_spinor(acc, E, out);
-}
-
-// the same into a fixed-point field
-template <bool DAG, bool CLOVER, bool COH>
-__device__ __forceinline__ void fx_hop_store(const Geom &g, const GaugePtr &U, const CloverPtr &C, const SpinorPtr &in,
-                                             int out_par, int cb, const SpinorPtr &out)
-{
-    Spinor<long long> acc;
-    Spinor<fx2> x;
-    int E;
-    fx_hopping<DAG, COH>(g, U, in, out_par, cb, acc, E);
-    fx_normalise(acc, E, x);
-    if constexpr (CLOVER) {
-        fx_clover(C, out_par, cb, x, E, acc);
-        fx_normalise(acc, E, x);
-    }
-    fx_store(out, cb, x, E);
-}
-
 // ---- canonical vectors by 16-byte words ----------------------------------------
 // (a warp holds the 32 sites of one layout block, which follow one another in a
 // canonical half vector, or take every other place in a full one)

@@ -18,8 +18,6 @@
 // FP32/FP16 (Sec. III-A), multiplied, and expanded back.
 #pragma once
 
-#include <atomic>
-
 #include "stencil.cuh"
 
 namespace qcd {
@@ -43,31 +41,12 @@ __device__ __forceinline__ void omega_sums(const Spinor<T> &o_, const Spinor<T> 
     red[2] += acc_cast<RA>(nn);
 }
 
-// the epilogue vector y at a site (FP64 and DF64: it may be a fixed-point field)
-template <int P>
-__device__ __forceinline__ void load_y(const StencilArgs &A, int cb, int r, Spinor<typename Prec<P>::T> &y)
-{
-    const SpinorPtr p = rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride);
-    if constexpr (P == QCD_F64 || P == QCD_DF64) {
-        if (A.y_fx) {
-            Spinor<double> d;
-            Prec<QCD_FX>::load(p, cb, d);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) y.s[k / 3][k % 3] = mk(typename Prec<P>::T(d.s[k / 3][k % 3].r), typename Prec<P>::T(d.s[k / 3][k % 3].i));
-            return;
-        }
-    }
-    Prec<P>::load(p, cb, y);
-}
-
 // One output site cb (right-hand side r): the hops, the mode's epilogue, the
 // site's contributions to the fused reductions.  The result is left in acc
 // for the caller to store (true), so that a kernel with a grid reduction
 // can publish its block's partial before its output stores are issued.
 // hop(acc) computes acc = H in at the site, clov(x) applies the site's clover
-// term (F^-1, or F for M_FULL) to x in place, clov2(x) F for M_RECON.  (The
-// fixed-point forms apply F^-1 of M_MULT and M_DHAT inside hop, and clov is
-// empty there.)
+// term (F^-1, or F for M_FULL) to x in place, clov2(x) F for M_RECON.
 template <int P, int MODE, int RED, bool DAG, class RA, class HopF, class CloF, class Clo2F>
 __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r, RA red[4],
                                              Spinor<typename Prec<P>::T> &acc, const HopF &hop, const CloF &clov,
@@ -81,7 +60,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
     } else if (MODE == M_DHAT) {
         clov(acc);
         Spinor<T> y;
-        load_y<P>(A, cb, r, y);
+        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), y);
         if (A.has_z) {
             Spinor<T> z;
@@ -94,7 +73,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
         }
     } else if (MODE == M_SRC) {
         Spinor<T> y;
-        load_y<P>(A, cb, r, y);
+        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), y);
         clov(acc);
     } else if (MODE == M_RECON) {
@@ -102,7 +81,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
         // residual, b_o - (F_oo x_o - kappa H_oe x_e) = u - F x_o, from the
         // same hopping term
         Spinor<T> y;
-        load_y<P>(A, cb, r, y);
+        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), y);  // u
         Spinor<T> xo = acc;
         clov(xo);
@@ -124,7 +103,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
         // also the second half of the gamma5-hermitian S_ee = F_ee - k^2 H_eo F_oo^-1 H_oe
         // (a = 1, cc = -k^2, y = the operator's input), with its dot products
         Spinor<T> y;
-        load_y<P>(A, cb, r, y);
+        Prec<P>::load(rhs_ptr(A.y, r, A.rhs_stride, A.norm_stride), cb, y);
         Spinor<T> fy = y;
         clov(fy);
         axpby_sp(acc, sarg<T>(A.cc, A.ccf), acc, sarg<T>(A.a, A.af), fy);
@@ -163,7 +142,7 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
     return true;
 }
 
-template <int P, int MODE, int RED, bool DAG, bool FX = false, bool CANON = false>
+template <int P, int MODE, int RED, bool DAG, bool CANON = false>
 __device__ __forceinline__ void stencil_body(const StencilArgs &A)
 {
     pdl_enter();
@@ -183,21 +162,10 @@ __device__ __forceinline__ void stencil_body(const StencilArgs &A)
     bool pending = false;
     if (cb < A.g.Vh) {
         const SpinorPtr in = rhs_ptr(A.in, r, A.rhs_stride, A.norm_stride);
-        constexpr bool FUSED = FX && (MODE == M_MULT || MODE == M_DHAT);
         pending = stencil_site<P, MODE, RED, DAG>(
-            A, cb, r, red, acc,
-            [&](Spinor<T> &a) {
-                if constexpr (FX) fx_hop<DAG, FUSED, false>(A.g, A.U, A.C, in, A.out_par, cb, a);
-                else hopping_any<P, DAG>(A.g, A.U, in, A.out_par, cb, a);
-            },
-            [&](Spinor<T> &x) {
-                if constexpr (!FX) clover_any<P>(A.C, A.out_par, cb, x);
-                else if constexpr (!FUSED) fx_clover_spinor(A.C, A.out_par, cb, x);
-            },
-            [&](Spinor<T> &x) {
-                if constexpr (FX) fx_clover_spinor(A.Cf, A.out_par, cb, x);
-                else clover_any<P>(A.Cf, A.out_par, cb, x);
-            });
+            A, cb, r, red, acc, [&](Spinor<T> &a) { hopping_any<P, DAG>(A.g, A.U, in, A.out_par, cb, a); },
+            [&](Spinor<T> &x) { clover_any<P>(A.C, A.out_par, cb, x); },
+            [&](Spinor<T> &x) { clover_any<P>(A.Cf, A.out_par, cb, x); });
     }
     if constexpr (RED != R_NONE) grid_reduce<RED == R_OMEGA ? 3 : RED == R_DOT_AUX ? 2 : 1>(red, A.red);
     // the output after the partial: the release that publishes the block's
@@ -205,7 +173,7 @@ __device__ __forceinline__ void stencil_body(const StencilArgs &A)
     // finishing block, reads them)
     if constexpr (CANON) {  // whole warps: blockDim.x is a multiple of 32
         extern __shared__ float4 sm_canon[];
-        using TC = typename std::conditional<P == QCD_F32, float, double>::type;
+        using TC = float;
         const int w = (threadIdx.x + threadIdx.y * blockDim.x) >> 5;
         canon_store(A.g, (TC *)A.canon + r * A.canon_stride, -1, cb, acc, sm_canon + w * SB * (canon_words<TC> + 1));
         return;
@@ -335,76 +303,32 @@ __global__ void __maxnreg__(128) stencil_kernel_r128(StencilArgs A)
     stencil_body<P, MODE, RED, DAG>(A);
 }
 
-// FP64 and DF64 with the products on the integer pipe (fx.cuh), for links
-// within the fixed-point range: every field of SU(3) links
-template <int P, int MODE, int RED, bool DAG>
-__global__ void __launch_bounds__(384) stencil_kernel_fx(StencilArgs A)
-{
-    stencil_body<P, MODE, RED, DAG, true>(A);
-}
-
 // The operator calls' form: the result goes to the caller's canonical vector
 // from the kernel itself, through shared memory, instead of through a vector
 // in the internal layout and a conversion pass (24^3x48 FP32: 64 MB of HBM
 // traffic and a launch less; hopping term with its input conversion 68.7 -> 58.9 us).
-template <int P, int MODE, bool DAG, bool FX>
+template <int P, int MODE, bool DAG>
 __global__ void __launch_bounds__(384) stencil_kernel_canon(StencilArgs A)
 {
-    stencil_body<P, MODE, R_NONE, DAG, FX, true>(A);
+    stencil_body<P, MODE, R_NONE, DAG, true>(A);
 }
 
-template <int P, int MODE, bool DAG, bool FX>
+template <int P, int MODE, bool DAG>
 __global__ void __maxnreg__(80) stencil_kernel_canon_r80(StencilArgs A)
 {
-    stencil_body<P, MODE, R_NONE, DAG, FX, true>(A);
-}
-
-// H in or F^-1 H in from a fixed-point field into one
-template <int MODE, bool DAG>
-__global__ void __launch_bounds__(384) stencil_kernel_fxout(StencilArgs A)
-{
-    pdl_enter();
-    const bool lead = blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0;
-    if (A.done && *A.done) {
-        if (A.skip && lead) *A.skip = 1;
-        return;
-    }
-    if (A.skip && lead) *A.skip = 0;
-    const int r = threadIdx.y, cb = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cb >= A.g.Vh) return;
-    fx_hop_store<DAG, MODE == M_MULT, false>(A.g, A.U, A.C, rhs_ptr(A.in, r, A.rhs_stride, A.norm_stride), A.out_par, cb,
-                                             rhs_ptr(A.out, r, A.rhs_stride, A.norm_stride));
+    stencil_body<P, MODE, R_NONE, DAG, true>(A);
 }
 
 // ---- host launcher -------------------------------------------------------
-// FP64: up to 78 KB of staging for 384 threads, above the 48 KB default (opted
-// in once per device and kernel)
-template <int P, int MODE, bool DAG>
-static void launch_canon_fx(const StencilArgs &A, dim3 grid, dim3 block, size_t smem, cudaStream_t s)
-{
-    static std::atomic<unsigned long long> done{0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (!(done.load(std::memory_order_relaxed) & bit)) {
-        cudaFuncSetAttribute(stencil_kernel_canon<P, MODE, DAG, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             384 * 13 * 16);
-        done.fetch_or(bit);
-    }
-    launch_pdl(stencil_kernel_canon<P, MODE, DAG, true>, grid, block, smem, s, A);
-}
-
 template <int P, int MODE, int RED, bool DAG>
 static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int variant)
 {
-    if constexpr (RED == R_NONE && (MODE == M_HOP || MODE == M_MULT || MODE == M_DHAT || MODE == M_FULL) &&
-                  (P == QCD_F32 || P == QCD_F64)) {
+    if constexpr (P == QCD_F32 && RED == R_NONE &&
+                  (MODE == M_HOP || MODE == M_MULT || MODE == M_DHAT || MODE == M_FULL)) {
         if (A.canon) {
-            const size_t sm = (size_t)block.x * block.y * (P == QCD_F32 ? 7 : 13) * 16;
-            if constexpr (P == QCD_F32) {
-                if (variant == 1) launch_pdl(stencil_kernel_canon_r80<P, MODE, DAG, false>, grid, block, sm, s, A);
-                else launch_pdl(stencil_kernel_canon<P, MODE, DAG, false>, grid, block, sm, s, A);
-            } else launch_canon_fx<P, MODE, DAG>(A, grid, block, sm, s);
+            const size_t sm = (size_t)block.x * block.y * 7 * 16;  // canon_store's words
+            if (variant == 1) launch_pdl(stencil_kernel_canon_r80<P, MODE, DAG>, grid, block, sm, s, A);
+            else launch_pdl(stencil_kernel_canon<P, MODE, DAG>, grid, block, sm, s, A);
             return;
         }
     }
@@ -418,12 +342,6 @@ static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s
                 launch_pdl(stencil_kernel_pipe<P, MODE, RED, DAG>, grid, block, 0, s, A);
                 return;
             }
-        }
-    }
-    if constexpr (P == QCD_F64 || P == QCD_DF64) {
-        if (A.fx) {
-            launch_pdl(stencil_kernel_fx<P, MODE, RED, DAG>, grid, block, 0, s, A);
-            return;
         }
     }
     if constexpr (P == QCD_DF64) {

@@ -189,12 +189,14 @@ int tune_one(qcd_ctx *c, StencilCall s, qcd_ctx::TuneEntry *out)
     const int nv = mr ? 2 : pipe ? 3 : (low || (s.prec == QCD_DF64 && !c->fx_links)) ? 2 : 1;
     // sites per block; for the multi-RHS kernel the right-hand sides per block
     // (all, a half, a third, a quarter)
-    const int bxs1[] = {64, 128, 256}, bxsn[] = {32, 64};
+    // (the fixed-point FP64 and DF64 kernels run two threads a site: smaller blocks)
+    const bool fx = c->fx_links && (s.prec == QCD_F64 || s.prec == QCD_DF64);
+    const int bxs1[] = {64, fx ? 32 : 128, 256}, bxsn[] = {32, 64};
     int bxst[4], nt = 0;
     for (int d : {1, 2, 3, 4})
         if (s.nrhs % d == 0) bxst[nt++] = s.nrhs / d;
     const int *bxs = mr ? bxst : s.nrhs > 1 ? bxsn : bxs1;
-    const int nbx = mr ? nt : s.nrhs > 1 ? 2 : 3;
+    const int nbx = mr ? nt : s.nrhs > 1 || fx ? 2 : 3;
     qcd_ctx::TuneEntry best{0, 128, 1e30};
     // QCD_TUNE_LOG set in the environment: every candidate's time on stderr
     static const bool log = std::getenv("QCD_TUNE_LOG") != nullptr;
