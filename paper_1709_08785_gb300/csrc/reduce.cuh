@@ -138,7 +138,8 @@ __device__ inline void finalize(int op, SolverState *st)
 // the FP64 and DF64 levels.  For the FP32 and FP16 levels, whose warp sums are
 // floats, a pair of floats (double-float, 2^-48): an FP64 instruction keeps a
 // warp scheduler's FP64 lanes busy for 64 cycles, and the FP64 tree of a block and
-// of its grid held each fused-dot kernel for some 2 us.
+// of its grid held each fused-dot kernel for some 2 us (two-level solves at one
+// launch shape: 8^4 2.94 -> 2.58 ms, 12^3x24 4.42 -> 3.97, 24^3x48 17.65 -> 17.27).
 template <class A>
 struct WideOf {
     using type = double;

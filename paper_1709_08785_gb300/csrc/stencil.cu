@@ -73,12 +73,13 @@ bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst)
 // The launch shape where the tuner has no entry: sites per block (for the
 // multi-RHS kernel the right-hand sides per block) and register budget.
 // FP32 and FP16 with more threads than one wave at the compiler's budget holds
-// (five blocks of 128 an SM): the 80-register kernels, six such blocks, and
-// 256 sites per block where dot products are fused (half the partials).  Solves
+// (five blocks of 128 an SM): the 80-register kernels, six such blocks.  Solves
 // with every such launch at one shape, budget / 80 registers: 20^3x40 10.43 / 9.98
 // ms, 24^3x48 18.55 / 17.65, FP16 inner level at 40^3x80 104.8 / 96.6.  Below, the
 // SMs are not full and spills only lengthen the chain: 16^3x32 5.74 / 5.91 ms,
-// 12^3x24 4.42 / 4.54.
+// 12^3x24 4.42 / 4.54.  Where dot products are fused, 256 sites per block (half
+// the partials of 128) once that leaves most SMs a block: 128 / 256 sites 12^3x24
+// 3.86 / 3.79 ms, 16^3x32 4.97 / 4.82, 24^3x48 17.48 / 17.27; 8^3x16 2.64 / 2.76.
 static void default_shape(const qcd_ctx *c, const StencilCall &sc, int &variant, int &bx)
 {
     const int nrhs = sc.nrhs < 1 ? 1 : sc.nrhs;
@@ -87,12 +88,14 @@ static void default_shape(const qcd_ctx *c, const StencilCall &sc, int &variant,
     if (nrhs > 1) bx = is_mrhs(sc) ? nrhs : nrhs <= 4 ? 64 : 32;
     // fixed point (two threads a site, 168 registers): blocks of 128 threads, three
     // an SM; 256 threads fit once (MULT at 24^3x48 175 / 223 us)
-    if (c->fx_links && (sc.prec == QCD_F64 || sc.prec == QCD_DF64)) bx = nrhs > 1 ? 32 : 64;
-    const bool low = sc.prec == QCD_F32 || sc.prec == QCD_F16;
-    if (low && !is_mrhs(sc) && (long)c->g.Vh * nrhs > 640L * c->num_sms) {
-        variant = 1;
-        if (sc.red != R_NONE) bx = 256;
+    if (c->fx_links && (sc.prec == QCD_F64 || sc.prec == QCD_DF64)) {
+        bx = nrhs > 1 ? 32 : 64;
+        // down to one warp a block while SMs would stay without one
+        while (nrhs == 1 && bx > 16 && (int)nblocks(c->g.Vh, bx) < c->num_sms) bx >>= 1;
     }
+    const bool low = sc.prec == QCD_F32 || sc.prec == QCD_F16;
+    if (low && !is_mrhs(sc) && (long)c->g.Vh * nrhs > 640L * c->num_sms) variant = 1;
+    if (low && sc.red != R_NONE && c->g.Vh >= 128 * c->num_sms) bx = 256;
 }
 
 int launch_stencil(qcd_ctx *c, const StencilCall &sc)
