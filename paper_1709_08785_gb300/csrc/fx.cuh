@@ -27,6 +27,9 @@ constexpr int FX_LIMB = 28;
 // With it every product of links below stays in range: |A B| <= 3, |A B C| <=
 // 5.2 entry by entry, so that limbs stay below 2^31 and sums below 2^63.
 constexpr float FX_LINK_FRO2 = 3.001f;
+// So do links of a smaller one but zero: a link's entries are rounded to 2^-55,
+// which for norms down to this is no more than FP64's own rounding of a product.
+constexpr float FX_LINK_FRO2_MIN = 0.5f;
 
 // a += x y as one instruction (written in C the sums are reassociated into
 // products and 64-bit additions, three instructions each)
@@ -61,6 +64,20 @@ __device__ __forceinline__ long long fx_from_unit(double d, int &bad)
     const int sh = 1023 - ex;                                    // |d| = m 2^(-52 - sh)
     m = sh >= 0 ? (m << 3) >> (sh > 63 ? 63 : sh) : m << 3;
     return b < 0 ? -m : m;
+}
+
+// The link m (row by row) as direction mu of site cb; true if it is out of range
+__device__ __forceinline__ bool fx_store_link(const double2 m[9], int4 *ux, int cb, int mu)
+{
+    float fro = 0.f;
+    int bad = 0;
+    bool zero = true;
+    for (int k = 0; k < 9; ++k) {
+        ux[soa(cb, 36, mu * 9 + k)] = fx_pack(fx_from_unit(m[k].x, bad), fx_from_unit(m[k].y, bad));
+        fro += (float)m[k].x * (float)m[k].x + (float)m[k].y * (float)m[k].y;
+        zero = zero && m[k].x == 0.0 && m[k].y == 0.0;
+    }
+    return bad || !(fro <= FX_LINK_FRO2) || (!zero && fro < FX_LINK_FRO2_MIN);
 }
 
 // ---------------------------------------------------------------- 3x3 matrices

@@ -49,13 +49,7 @@ __global__ void k_gauge_convert(Geom g, const double2 *__restrict__ U, double2 *
         for (int k = 0; k < 9; ++k) m[k] = U[((size_t)s * 4 + mu) * 9 + k];
         for (int k = 0; k < 9; ++k) u64[soa(cb, 36, mu * 9 + k)] = m[k];
         if constexpr (FX) {
-            float fro = 0.f;
-            int bad = 0;
-            for (int k = 0; k < 9; ++k) {
-                ((int4 *)ux)[soa(cb, 36, mu * 9 + k)] = fx_pack(fx_from_unit(m[k].x, bad), fx_from_unit(m[k].y, bad));
-                fro += (float)m[k].x * (float)m[k].x + (float)m[k].y * (float)m[k].y;
-            }
-            if (bad || !(fro <= FX_LINK_FRO2)) *wide = 1;
+            if (fx_store_link(m, (int4 *)ux, cb, mu)) *wide = 1;
         } else {
             for (int k = 0; k < 9; ++k) ((float4 *)ux)[soa(cb, 36, mu * 9 + k)] = df_pair(m[k]);
         }

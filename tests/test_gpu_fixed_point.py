@@ -29,11 +29,11 @@ def make_ctx(dims, U, kappa, csw, t_bc=-1):
 
 
 @pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 4, 10), (4, 4, 6, 8)])
-@pytest.mark.parametrize("scale", [1.0, 0.3, 1.3])
+@pytest.mark.parametrize("scale", [1.0, 0.6, 0.3, 1.3])
 @pytest.mark.parametrize("inverse", [False, True])
 def test_clover_blocks(dims, scale, inverse):
-    """F and F^-1 in FP64 for SU(3) links, smaller ones, and ones beyond the
-    fixed-point range (scale 1.3)."""
+    """F and F^-1 in FP64 for SU(3) links, smaller ones, and ones below and above
+    the fixed-point range (scales 0.3 and 1.3)."""
     kappa, csw = 0.12, 1.0
     U = scale * inputs.random_gauge(dims, 0.3, 300)
     ctx = make_ctx(dims, U, kappa, csw)
@@ -82,6 +82,24 @@ def test_force(dims, scale, graded):
     ctx.force(torch.from_numpy(U).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(lam).cuda(), G)
     torch.cuda.synchronize()
     assert rel(G.cpu().numpy(), oracle.link_grad(dims, t_bc, U, kappa, csw, x, lam)) < TOL
+    ctx.close()
+
+
+@pytest.mark.parametrize("scale", [0.5, 0.3, 1e-7, 1e-30])
+def test_small_links_keep_their_accuracy(scale):
+    """H in FP64 where its links are small against the fixed-point unit, some of
+    them zero (an open boundary)."""
+    dims, t_bc = (6, 2, 4, 10), -1
+    Vh = inputs.volume(dims) // 2
+    U = scale * inputs.random_gauge(dims, 0.3, 311)
+    U[::5] = 0.0
+    v = inputs.gaussian_source(dims, 312)[:Vh]
+    ctx = make_ctx(dims, U, 0.12, 0.0, t_bc)
+    inp = torch.from_numpy(v).cuda()
+    out = torch.zeros_like(inp)
+    ctx.dslash_eo(out, inp, 0, 0, 0)
+    torch.cuda.synchronize()
+    assert rel(out.cpu().numpy(), oracle.hop_eo(dims, t_bc, U, 0, v)) < 1e-13
     ctx.close()
 
 
