@@ -132,10 +132,9 @@ __device__ __forceinline__ int plane_index(int mu, int nu)
 }
 
 // Y_p(n) = csw kappa (S^T + conj(S)) / (8i) for the six planes
-__global__ void k_force_Y(Geom g, const double2 *__restrict__ x, const double2 *__restrict__ lam, double ck, double2 *Y)
+__device__ __forceinline__ void force_Y_site(const Geom &g, const double2 *__restrict__ x,
+                                             const double2 *__restrict__ lam, double ck, double2 *Y, int s)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
     C X[4][3], L[4][3];
     load_spinor(x, s, X);
     load_spinor(lam, s, L);
@@ -173,12 +172,11 @@ __device__ __forceinline__ M3 Yeff(const double2 *Y, int s, int mu, int nu)
     return fwd ? r : dagm(r);
 }
 
-__global__ void k_force_link(Geom g, const double2 *__restrict__ U, const double2 *__restrict__ x,
-                             const double2 *__restrict__ lam, const double2 *__restrict__ Y, double kappa,
-                             int with_clover, double2 *G)
+__device__ __forceinline__ void force_link_one(const Geom &g, const double2 *__restrict__ U,
+                                               const double2 *__restrict__ x, const double2 *__restrict__ lam,
+                                               const double2 *__restrict__ Y, double kappa, int with_clover, double2 *G,
+                                               int tid)
 {
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= 4 * g.V) return;
     const int m = tid >> 2, mu = tid & 3;
     const int mp = site_shift(g, m, mu, +1);
     M3 Gm = zero3();
@@ -242,6 +240,23 @@ __global__ void k_force_link(Geom g, const double2 *__restrict__ U, const double
     for (int k = 0; k < 9; ++k) out[k] = make_double2(Gm.m[k / 3][k % 3].r, Gm.m[k / 3][k % 3].i);
 }
 
+// run != NULL: nothing to do unless *run is set (any grid covers all sites)
+__global__ void k_force_Y(Geom g, const double2 *__restrict__ x, const double2 *__restrict__ lam, double ck, double2 *Y,
+                          const int *run)
+{
+    if (run && !*run) return;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += gridDim.x * blockDim.x)
+        force_Y_site(g, x, lam, ck, Y, s);
+}
+__global__ void k_force_link(Geom g, const double2 *__restrict__ U, const double2 *__restrict__ x,
+                             const double2 *__restrict__ lam, const double2 *__restrict__ Y, double kappa,
+                             int with_clover, double2 *G, const int *run)
+{
+    if (run && !*run) return;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 4 * g.V; t += gridDim.x * blockDim.x)
+        force_link_one(g, U, x, lam, Y, kappa, with_clover, G, t);
+}
+
 // ---------------------------------------------------------------- fixed-point form
 // For links within the fixed-point range (fx.cuh) the clover part runs on the
 // integer pipe, with fewer products.  Y is anti-Hermitian, so with
@@ -299,11 +314,27 @@ __device__ __forceinline__ void force_y_plane(const Geom &g, const Spinor<double
         }
 }
 
+// The caller's links in fixed point; *wide is set if one is out of range
+// (thread = link in the caller's order: a warp reads 4.6 KB in a row)
+__global__ void __launch_bounds__(128) k_force_Ux(Geom g, const double2 *__restrict__ U, int4 *Ue, int4 *Uo, int *wide)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, s = t >> 2;
+    if (s >= g.V) return;
+    int par = 0, q = s;
+    for (int k = 0; k < 4; ++k) {
+        par ^= (q % g.L[k]) & 1;
+        q /= g.L[k];
+    }
+    double2 m[9];
+    for (int k = 0; k < 9; ++k) m[k] = __ldg(U + (size_t)t * 9 + k);
+    if (fx_store_link(m, par ? Uo : Ue, s >> 1, t & 3)) *wide = 1;
+}
+
 __global__ void __launch_bounds__(128) k_force_Yx(Geom g, const double2 *__restrict__ x, const double2 *__restrict__ lam,
-                                                  double f, double *Y)
+                                                  double f, double *Y, const int *wide)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x, par = blockIdx.y;
-    if (cb >= g.Vh) return;
+    if (cb >= g.Vh || *wide) return;
     int c[4];
     site_coords(g, par, cb, c);
     const int s = lex_of(g, c);
@@ -355,10 +386,11 @@ struct ForceZ {
     int *e;      // unit exponents [12][2][Vh_pad]
 };
 
-__global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const double *__restrict__ Y, ForceZ Z)
+__global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const double *__restrict__ Y, ForceZ Z,
+                                                    const int *wide)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x, zi = blockIdx.y, par = blockIdx.z;
-    if (cb >= g.Vh) return;
+    if (cb >= g.Vh || *wide) return;
     const int nu = zi / 3, k3 = zi - 3 * nu, mu = k3 < nu ? k3 : k3 + 1;
     const int plane = mu < nu ? plane_index(mu, nu) : plane_index(nu, mu);
     int c[4];
@@ -430,10 +462,10 @@ __global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const do
 // G_mu(m) of the sites of parity blockIdx.z, direction blockIdx.y
 __global__ void __launch_bounds__(128, 3) k_force_link_x(Geom g, GaugePtr U, ForceZ Z, const double2 *__restrict__ x,
                                                          const double2 *__restrict__ lam, double kappa, int with_clover,
-                                                         double2 *G)
+                                                         double2 *G, const int *wide)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y, par = blockIdx.z;
-    if (cb >= g.Vh) return;
+    if (cb >= g.Vh || *wide) return;
     int c[4];
     site_coords(g, par, cb, c);
     const int op = 1 - par;
@@ -554,10 +586,13 @@ __global__ void k_gamma5(int V, const double2 *in, double2 *out)
 int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_canon)
 {
     // FP64 form: Y as full matrices; fixed-point form: Y as nine reals, Z and its
-    // exponents
+    // exponents, and the links that the caller passes (not the loaded ones) in
+    // fixed point (25 us at 16^3x32).  Whether they are in its range is known on
+    // the device only, so the FP64 kernels follow and return at once if they are.
     const size_t vp = (size_t)c->g.Vh_pad;
-    const size_t yx = 54 * 2 * vp * sizeof(double), zx = 2 * vp * 108 * 16;
-    const size_t ybytes = c->fx_links ? yx + zx + 24 * vp * sizeof(int) : (size_t)c->g.V * 6 * 9 * 16;
+    const size_t yx = 54 * 2 * vp * sizeof(double), zx = 2 * vp * 108 * 16, ex = 24 * vp * sizeof(int);
+    const size_t y64 = (size_t)c->g.V * 6 * 9 * 16, fx = yx + zx + ex + 2 * vp * 36 * 16;
+    const size_t ybytes = c->fx_links && fx > y64 ? fx : y64;
     if (c->force_bytes < ybytes) {
         if (c->force_buf) {
             cudaStreamSynchronize(c->stream);
@@ -571,47 +606,57 @@ int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_can
         if (rc) return rc;
         c->force_bytes = ybytes;
     }
+    int *wide = nullptr;
     if (c->fx_links) {
+        wide = c->flag_dev + 1;
+        QCD_CUDA_CHECK(cudaMemsetAsync(wide, 0, sizeof(int), c->stream));
         double *Y = (double *)c->force_buf;
         ForceZ Z;
         Z.z[0] = (int4 *)((char *)c->force_buf + yx);
         Z.z[1] = Z.z[0] + vp * 108;
         Z.e = (int *)((char *)c->force_buf + yx + zx);
+        int4 *ux = (int4 *)((char *)c->force_buf + yx + zx + ex);
         GaugePtr U;
         for (int p = 0; p < 2; ++p) {
-            U.a[p] = c->UX[p];
+            U.a[p] = ux + (size_t)p * vp * 36;
             U.b[p] = nullptr;
         }
         const unsigned nb = nblocks(c->g.Vh, 128);
         const int with = c->csw != 0.0;
+        {
+            ProfScope p0(c, QCD_K_OTHER, 0.0);
+            k_force_Ux<<<nblocks(4L * c->g.V, 128), 128, 0, c->stream>>>(c->g, (const double2 *)U_canon, ux, ux + vp * 36, wide);
+            QCD_CUDA_CHECK(cudaGetLastError());
+        }
         if (with) {
             ProfScope p1(c, QCD_K_OTHER, 0.0);
             k_force_Yx<<<dim3(nb, 2), 128, 0, c->stream>>>(c->g, (const double2 *)x, (const double2 *)lam,
-                                                            0.125 * c->csw * c->kappa, Y);
+                                                            0.125 * c->csw * c->kappa, Y, wide);
             QCD_CUDA_CHECK(cudaGetLastError());
         }
         if (with) {
             ProfScope p2(c, QCD_K_OTHER, 0.0);
-            k_force_Z<<<dim3(nb, 12, 2), 128, 0, c->stream>>>(c->g, U, Y, Z);
+            k_force_Z<<<dim3(nb, 12, 2), 128, 0, c->stream>>>(c->g, U, Y, Z, wide);
             QCD_CUDA_CHECK(cudaGetLastError());
         }
         ProfScope p3(c, QCD_K_OTHER, 0.0);
         k_force_link_x<<<dim3(nb, 4, 2), 128, 0, c->stream>>>(c->g, U, Z, (const double2 *)x, (const double2 *)lam,
-                                                              c->kappa, with, (double2 *)G);
+                                                              c->kappa, with, (double2 *)G, wide);
         QCD_CUDA_CHECK(cudaGetLastError());
-        return QCD_OK;
+    }
+    // one wave where they most likely have nothing to do
+    const auto blocks = [&](unsigned all) { return wide && all > 4u * c->num_sms ? 4u * c->num_sms : all; };
+    {
+        ProfScope prof(c, QCD_K_OTHER, 0.0);
+        k_force_Y<<<blocks(nblocks(c->g.V, 128)), 128, 0, c->stream>>>(c->g, (const double2 *)x, (const double2 *)lam,
+                                                              c->csw * c->kappa, (double2 *)c->force_buf, wide);
+        QCD_CUDA_CHECK(cudaGetLastError());
     }
     {
         ProfScope prof(c, QCD_K_OTHER, 0.0);
-        k_force_Y<<<nblocks(c->g.V, 128), 128, 0, c->stream>>>(c->g, (const double2 *)x, (const double2 *)lam,
-                                                              c->csw * c->kappa, (double2 *)c->force_buf);
-        QCD_CUDA_CHECK(cudaGetLastError());
-    }
-    {
-        ProfScope prof(c, QCD_K_OTHER, 0.0);
-        k_force_link<<<nblocks(4L * c->g.V, 64), 64, 0, c->stream>>>(
+        k_force_link<<<blocks(nblocks(4L * c->g.V, 64)), 64, 0, c->stream>>>(
             c->g, (const double2 *)U_canon, (const double2 *)x, (const double2 *)lam, (const double2 *)c->force_buf,
-            c->kappa, c->csw != 0.0, (double2 *)G);
+            c->kappa, c->csw != 0.0, (double2 *)G, wide);
         QCD_CUDA_CHECK(cudaGetLastError());
     }
     return QCD_OK;

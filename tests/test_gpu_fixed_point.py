@@ -85,6 +85,20 @@ def test_force(dims, scale, graded):
     ctx.close()
 
 
+@pytest.mark.parametrize("scale", [1.0, 1.3, 1e-7])
+def test_force_takes_the_links_it_is_given(scale):
+    """The gradient at other links than the loaded ones, in range or not."""
+    dims, kappa, csw, t_bc = (6, 2, 4, 10), 0.12, 1.3, -1
+    U = scale * inputs.random_gauge(dims, 0.3, 310)
+    x, lam = inputs.gaussian_source(dims, 304), inputs.gaussian_source(dims, 305)
+    ctx = make_ctx(dims, inputs.random_gauge(dims, 0.3, 303), kappa, csw, t_bc)
+    G = torch.zeros(U.shape, dtype=torch.complex128, device="cuda")
+    ctx.force(torch.from_numpy(U).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(lam).cuda(), G)
+    torch.cuda.synchronize()
+    assert rel(G.cpu().numpy(), oracle.link_grad(dims, t_bc, U, kappa, csw, x, lam)) < TOL
+    ctx.close()
+
+
 @pytest.mark.parametrize("scale", [0.5, 0.3, 1e-7, 1e-30])
 def test_small_links_keep_their_accuracy(scale):
     """H in FP64 where its links are small against the fixed-point unit, some of
