@@ -469,7 +469,10 @@ int clover_build(qcd_ctx *c, double kappa, double csw)
                          f[QCD_DF64][par], e[par]};
     };
     // the field strengths of one parity at a time
-    int rc = ensure_staging(c, (size_t)c->g.Vh_pad * 54 * sizeof(double));
+    // (the buffer at least as large as the operator calls need it, so that the
+    // first of them does not free it, wait and allocate again)
+    const size_t fs = (size_t)c->g.Vh_pad * 54 * sizeof(double), ops = (size_t)c->g.V * 12 * 16 * 2;
+    int rc = ensure_staging(c, fs > ops ? fs : ops);
     if (rc) return rc;
     double *FS = (double *)c->staging;
     for (int par = 0; par < 2; ++par) {
