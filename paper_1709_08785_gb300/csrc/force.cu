@@ -267,8 +267,9 @@ __global__ void k_force_link(Geom g, const double2 *__restrict__ U, const double
 // q = m - nu, + for mu < nu: 8 products a plane instead of 18, and 24 a site for
 // Z.  The hopping part keeps FP64 and uses the projector's rank: with h the
 // two projected spin rows, sum_s ((1-g)lambda)_s conj(x_s) = sum_a h_a(lambda)
-// conj(h_a(x)).  16^3x32: 8.4 ms before, 1.21 ms now (Y 0.19, Z 0.18, links 0.84,
-// issue-bound at half a slot per cycle).
+// conj(h_a(x)).  16^3x32: 8.4 ms before, 1.25 ms now (the caller's links
+// into fixed point 0.03, Y 0.19, Z 0.18, links 0.84, issue-bound at half a slot
+// per cycle).
 
 // (sigma_p v)_a = ph v[perm]: ph as a power of i (the tables above)
 __device__ constexpr int sig_perm(int p, int a)
@@ -587,7 +588,7 @@ int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_can
 {
     // FP64 form: Y as full matrices; fixed-point form: Y as nine reals, Z and its
     // exponents, and the links that the caller passes (not the loaded ones) in
-    // fixed point (25 us at 16^3x32).  Whether they are in its range is known on
+    // fixed point (34 us at 16^3x32).  Whether they are in its range is known on
     // the device only, so the FP64 kernels follow and return at once if they are.
     const size_t vp = (size_t)c->g.Vh_pad;
     const size_t yx = 54 * 2 * vp * sizeof(double), zx = 2 * vp * 108 * 16, ex = 24 * vp * sizeof(int);

@@ -55,12 +55,20 @@ __global__ void k_gauge_convert(Geom g, const double2 *__restrict__ U, double2 *
         }
         // first two columns: a = (m00, m10, m20), b = (m01, m11, m21)
         const double2 a0 = m[0], a1 = m[3], a2 = m[6], b0 = m[1], b1 = m[4], b2 = m[7];
-        u32[soa(cb, 12, mu * 3 + 0)] = make_float4(a0.x, a0.y, a1.x, a1.y);
-        u32[soa(cb, 12, mu * 3 + 1)] = make_float4(a2.x, a2.y, b0.x, b0.y);
-        u32[soa(cb, 12, mu * 3 + 2)] = make_float4(b1.x, b1.y, b2.x, b2.y);
-        auto hh = [](double2 z) { return h2u(__floats2half2_rn((float)z.x, (float)z.y)); };
-        u16a[soa(cb, 4, mu)] = make_uint4(hh(a0), hh(a1), hh(a2), hh(b0));
-        u16b[soa(cb, 4, mu)] = make_uint2(hh(b1), hh(b2));
+        const double2 ab[6] = {a0, a1, a2, b0, b1, b2};
+        float2 f[6];
+        bool slow = false;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) f[k] = make_float2(f32_int<false>(ab[k].x, slow), f32_int<false>(ab[k].y, slow));
+        if (slow)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) f[k] = make_float2((float)ab[k].x, (float)ab[k].y);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            u32[soa(cb, 12, mu * 3 + k)] = make_float4(f[2 * k].x, f[2 * k].y, f[2 * k + 1].x, f[2 * k + 1].y);
+        auto hh = [](float2 z) { return h2u(__floats2half2_rn(z.x, z.y)); };
+        u16a[soa(cb, 4, mu)] = make_uint4(hh(f[0]), hh(f[1]), hh(f[2]), hh(f[3]));
+        u16b[soa(cb, 4, mu)] = make_uint2(hh(f[4]), hh(f[5]));
     }
 }
 
@@ -369,15 +377,16 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
     }
     float f[36];
     unsigned w[18];
+    bool slow = false;
 #pragma unroll
-    for (int k = 0; k < 36; ++k) f[k] = (float)r[k];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) p32[soa(cb, 18, blk * 9 + q)] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+    for (int k = 0; k < 36; ++k) f[k] = f32_int<false>(r[k], slow);
     // halves, rounded from FP64: element e = 36 blk + j of the site is half e & 7
     // of uint4 e >> 3, so block 0 ends and block 1 begins in the middle of uint4 4
 #pragma unroll
     for (int k = 0; k < 18; ++k)
-        w[k] = h2u(__halves2half2(__double2half(r[2 * k]), __double2half(r[2 * k + 1])));
+        w[k] = h2u(__floats2half2_rn(f32_int<true>(r[2 * k], slow), f32_int<true>(r[2 * k + 1], slow)));
+#pragma unroll
+    for (int q = 0; q < 9; ++q) p32[soa(cb, 18, blk * 9 + q)] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
     const int q0 = blk ? 5 : 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -385,13 +394,20 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
         p16[soa(cb, 9, q0 + q)] = blk ? make_uint4(w[a + 2], w[a + 3], w[a + 4], w[a + 5]) : make_uint4(w[a], w[a + 1], w[a + 2], w[a + 3]);
     }
     ((uint2 *)p16)[soa(cb, 9, 4) * 2 + blk] = blk ? make_uint2(w[0], w[1]) : make_uint2(w[16], w[17]);
+    if (slow)  // (rare) entries beyond FP32's normal range: over again from the stored block
+#pragma unroll 1
+        for (int j = 0; j < 36; ++j) {
+            const int e = 36 * blk + j;
+            const double v = ((const double *)(p64 + soa(cb, 36, e >> 1)))[e & 1];
+            ((float *)(p32 + soa(cb, 18, e >> 2)))[e & 3] = (float)v;
+            ((__half *)(p16 + soa(cb, 9, e >> 3)))[e & 7] = __double2half(v);
+        }
 }
 
 // Both kernels replace one that walked the planes twice per site in FP64 with
-// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 4.1 ms
+// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 3.85 ms
 // now (k_field_strength 2.45 ms, issue-bound at 0.45 of a slot per cycle with
-// twelve warps an SM; k_clover_build 1.6 ms, the inverses
-// and conversions on the FP64 pipe).
+// twelve warps an SM; k_clover_build 1.4 ms, the inverses on the FP64 pipe).
 // Field strengths: thread = (site, plane), blockIdx.y the plane; planes (0,1)
 // (0,2) (0,3) (1,2) (1,3) (2,3).  FS: [plane][9][Vh_pad] doubles of one parity.
 template <class Alg>

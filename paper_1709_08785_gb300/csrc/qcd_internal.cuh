@@ -13,17 +13,21 @@
 //           F32:  6 float4  (two complex each)
 //           F16:  3 uint4   (four complex each, IEEE half) + one float norm
 //                 per site; the stored halves are psi/norm, |.| <= 1
+//           FX:  12 int4 (one complex each: two limbs per real) + one int
+//                 exponent per site (fx.cuh)
 //   link    F64: 9 double2, U_ij at k = 3*i + j (18 reals)
 //           F32: 3 float4, the first two columns a, b of U (12 reals,
 //                Sec. III-A "SU(3)-reconstruction"); U = (a, b, conj(a x b))
 //           F16: uint4 (a0 a1 a2 b0) + uint2 (b1 b2), 12 halves
+//           FX:  9 int4, U_ij at k = 3*i + j, entries in units of 2^-55
 //           links are stored with the parity of their base site n; the
 //           four directions of a site share a block: NCOMP = 4*ncomp_link,
 //           k = mu*ncomp_link + component.
 //   clover  two 6x6 Hermitian blocks per site in the chiral (gamma5) basis,
 //           each as 6 real diagonal entries then the 15 complex entries
 //           below the diagonal, row by row: 72 reals per site
-//           F64: 36 double2, F32: 18 float4, F16: 9 uint4
+//           F64: 36 double2, F32: 18 float4, F16: 9 uint4; FX: 36 int4 + one
+//           int exponent per block
 #pragma once
 
 #include <cuda_fp16.h>

@@ -1,7 +1,8 @@
 // Autotuner for the stencil kernels: for each launch configuration the
 // solvers use (precision, mode, fused reduction, dagger, right-hand sides) it
 // times every candidate -- register budget (compiler's / capped at 80 for FP32
-// and FP16, at 128 for DF64) x threads per block along the sites, or for the
+// and FP16; the fixed-point kernels of FP64 and DF64 have one, and 32 or 64
+// sites per block) x threads per block along the sites, or for the
 // multi-RHS kernel x right-hand sides per block (the RHS tile) -- on scratch
 // buffers with L2 evicted before each launch, keeps the fastest, and stores
 // the choice in a JSON cache keyed by device name, lattice and configuration.

@@ -153,3 +153,41 @@ def test_non_finite_input_gives_non_finite_output():
         assert not np.isfinite(got[5]).all()  # D^ holds the input at its own site
         assert np.isfinite(got).any()         # sites out of reach keep finite values
     ctx.close()
+
+
+@pytest.mark.parametrize("tiny", [1e-42, 1e-38, 2.0 ** -149, 2.0 ** -126 * (1 - 2.0 ** -30)])
+def test_entries_below_the_normal_range_of_fp32(tiny):
+    """FP32 copies of links and clover blocks whose entries are denormal in FP32
+    (the integer conversion hands them to the FP64 instruction): rounded to a
+    unit of 2^-149."""
+    dims, t_bc = (4, 4, 4, 4), 1
+    V = inputs.volume(dims)
+    U = inputs.unit_gauge(dims)
+    U[..., 0, 1] = tiny
+    v = np.zeros((V // 2, 4, 3), np.complex64)
+    v[:, :, 1] = 2.0 ** 120  # colour 1 only: colour 0 of H v is the tiny entry times 2^120
+    ctx = make_ctx(dims, U, 0.12, 0.0, t_bc)
+    inp = torch.from_numpy(v).cuda()
+    out = torch.zeros_like(inp)
+    ctx.dslash_eo(out, inp, 0, False, 1)
+    torch.cuda.synchronize()
+    U[..., 0, 1] = np.float32(tiny)
+    want = oracle.hop_eo(dims, t_bc, U, 0, v.astype(np.complex128))[:, :, 0]
+    assert rel(out.cpu().numpy()[:, :, 0], want) < 1e-5
+    ctx.close()
+    # clover entries of about `tiny`
+    U = inputs.random_gauge(dims, 0.3, 313)
+    kappa, csw = 0.12, tiny
+    ctx = make_ctx(dims, U, kappa, csw, t_bc)
+    w = np.zeros((V // 2, 4, 3), np.complex64)
+    w[:, 0, 0] = 2.0 ** 120
+    inp = torch.from_numpy(w).cuda()
+    ctx.clover_apply(out, inp, 0, False, 1)
+    torch.cuda.synchronize()
+    F = oracle.clover_field(dims, U, kappa, csw)
+    want = oracle.site_apply(oracle.field_to_half(dims, 0, F), w.astype(np.complex128))
+    got = out.cpu().numpy()
+    for s, k in ((0, 1), (0, 2), (1, 0), (1, 1), (1, 2)):  # the components without the diagonal
+        # entries of both blocks, each rounded by half a unit, times 2^120 / 2 each
+        assert np.abs(got[:, s, k] - want[:, s, k]).max() <= 2.0 ** (120 - 148) + 1e-5 * np.abs(want[:, s, k]).max()
+    ctx.close()
