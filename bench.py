@@ -8,9 +8,9 @@ One step = one complete qcd_solve (b^_e preparation, the nested iteration,
 x_o reconstruction and the FP64 true-residual check) from a device-resident
 source; every step must reach ||b - D x|| / ||b|| <= 1e-12.  The solve runs
 the library's default outer level: the solution x_e, the source b^_e and the
-reconstruction x_o in FP64 arithmetic, the outer D^ applications and
-recursion vectors in DF64, the inner iteration in FP32; the all-FP64 and
-all-DF64 outer levels are timed beside it.  Under torchrun (N > 1) every rank
+reconstruction x_o in FP64, the recursion vectors in DF64, their operators in
+block fixed point (FP64 accuracy), the inner iteration in FP32; the all-FP64
+and all-DF64 outer levels are timed beside it.  Under torchrun (N > 1) every rank
 solves its own replica (no collective on the data path); the time is the
 maximum over ranks.  Prints one JSON line on rank 0.
 """
@@ -41,7 +41,8 @@ WORKLOAD_NAME = ("24^3x48 clover-Wilson, even-odd preconditioned nested BiCGStab
                  "(inner tol 1e-5), links exp(i 0.25 H) seed 3, kappa 0.124, csw 1.6, antiperiodic t, "
                  "Gaussian source seed 30, tol 1e-12")
 DTYPE = ("f64 (solution x_e, source b^_e, reconstruction x_o, outer dots and norms, true residual) + "
-         "df64 (outer D^ and recursion vectors) + f32 (inner iteration)")
+         "57-bit block fixed point (FP64-level operators, outer D^) + df64 (outer recursion vectors) + "
+         "f32 (inner iteration)")
 # algorithmic bytes per output site of the FP32 stencil kernels of one D^:
 # MULT (in 96 + links 8x48 + clover 288 + out 96) and the fused second half
 STENCIL_SOURCES = ["paper_1709_08785_gb300/csrc/stencil_impl.cuh", "paper_1709_08785_gb300/csrc/stencil.cuh",
@@ -363,7 +364,7 @@ def extra_workloads(torch, qcd, hbm):
         times.append(e0.elapsed_time(e1) * 1e-3)
     tb = min(times)
     # algorithmic bytes: the inner FP32 iterations and the outer D^ (two
-    # DF64 MULT-class passes of 2112 B per output site plus the epilogue's
+    # MULT-class passes on FP64-sized fields of 2112 B per output site plus the epilogue's
     # v, r~ or r: 2 x 2112 + 2 x 192) of every problem
     by = sum(i["inner_iters"][0] * INNER_ITER_BYTES * inputs.volume(p["dims"]) // 2 +
              i["dhat_applies"][0] * (2 * 2112 + 2 * 192) * inputs.volume(p["dims"]) // 2 for p, i in zip(probs, infos))
@@ -372,7 +373,7 @@ def extra_workloads(torch, qcd, hbm):
                          "inner_iters": sum(i["inner_iters"][0] for i in infos),
                          "roofline": {"algorithmic_bytes": by, "achieved_gbs": round(by / tb / 1e9, 1),
                                       "frac": round(by / tb / 1e9 / hbm, 3),
-                                      "counted": "inner FP32 iterations (5088 B per even site) and outer DF64 D^ "
+                                      "counted": "inner FP32 iterations (5088 B per even site) and outer D^ "
                                                  "(4608 B per even site) of every problem, over the whole batch "
                                                  "time (set-up of b^ and the x_o / true-residual finish included)"}}
     for c in ctxs:
@@ -668,7 +669,7 @@ def run_ours(args):
         "warmup": args.warmup, "ms_per_step": round(ms_step, 3), "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None, "dtype": DTYPE, "data": "synthetic",
         "config": {"workload": WORKLOAD_NAME, "lattice": list(dims), "sites": V, "tol": W["tol"],
-                   "outer_level": "outer_df64 = 1: FP64 solution accumulation, DF64 outer D^",
+                   "outer_level": "outer_df64 = 1: FP64 solution accumulation, outer D^ on DF64 vectors in fixed point",
                    "parallelism": "replicas" if ws > 1 else "single",
                    "l2": "inputs larger than L2: one FP32 MULT touches 287 MB, one solve several GB"},
         "roofline": roofline,

@@ -70,10 +70,17 @@ typedef enum {
     QCD_ESTATE = -9             /* call out of order (e.g. no gauge field loaded) */
 } qcd_status;
 
-/* QCD_DF64: FP64-sized storage, arithmetic in pairs of floats (double-float,
- * about 48 significant bits): the outer level of the mixed solvers, since
- * GB300 issues FP32 at about 64x its FP64 rate.  Operator calls with
- * QCD_DF64 take complex128 buffers. */
+/* QCD_DF64: FP64-sized storage of pairs of floats (double-float, about 48
+ * significant bits): the outer level of the mixed solvers, since GB300 issues
+ * FP32 at about 64x its FP64 rate.  Operator calls with QCD_DF64 take
+ * complex128 buffers.
+ * The operators of QCD_F64 and QCD_DF64 compute in block fixed point on the
+ * integer pipe (57-bit components and an exponent per site; norm-wise at least
+ * as accurate as FP64 arithmetic) when every loaded link is zero or has a
+ * squared Frobenius norm between 0.5 and 3.001 (SU(3): 3); with another link in
+ * the field, QCD_F64 computes in FP64 and QCD_DF64 in pairs of floats.  In
+ * fixed point a non-finite component makes every component of the sites it
+ * reaches NaN. */
 typedef enum { QCD_F64 = 0, QCD_F32 = 1, QCD_F16 = 2, QCD_DF64 = 3 } qcd_prec;
 
 /* Create a context for one lattice on the current CUDA device.
@@ -89,16 +96,17 @@ int qcd_set_stream(qcd_ctx *ctx, void *stream);
 
 /* Load the gauge field U (canonical complex128 [V][4][3][3]), from device
  * memory (on_device = 1) or host memory (0), and build the internal copies:
- * FP64 with 18 reals per link, FP32 and FP16 with the first two columns
- * only (12 reals, SU(3) reconstruction, Sec. III-A) -- the conversion
+ * FP64 and fixed point with 18 reals per link, FP32 and FP16 with the first
+ * two columns only (12 reals, SU(3) reconstruction, Sec. III-A) -- the conversion
  * [U, F] -> [U^SP, F^SP] of Alg. 1.  Invalidates the clover term.
  * Synchronous with respect to the host buffer (it may be reused on return). */
 int qcd_gauge_load(qcd_ctx *ctx, const void *U, int on_device);
 
 /* Build the clover term F and its site-local inverse F^-1 (Sec. II-B: F_ee,
- * F_oo are block diagonal and "inverted easily") in FP64 from the FP64
- * links, as two 6x6 Hermitian blocks per site in the chiral basis
- * (Sec. III-A), then round them to FP32 and FP16.
+ * F_oo are block diagonal and "inverted easily") from the FP64 links (plaquette
+ * products in fixed point or FP64, see QCD_DF64; the inverse in FP64), as two
+ * 6x6 Hermitian blocks per site in the chiral basis (Sec. III-A), then round
+ * them to FP32 and FP16.
  * Errors: QCD_ESTATE without a gauge field; QCD_ECLOVER_SINGULAR if a block
  * has a (near-)zero pivot. */
 int qcd_clover_build(qcd_ctx *ctx, double kappa, double csw);
@@ -180,7 +188,8 @@ typedef struct {
                                 (Eq. 6) and the reconstruction x_o (Eq. 7)
                                 are FP64 and accumulated in FP64 arithmetic;
                                 the outer D^ applications and the iteration's
-                                own vectors (r, r~, p, q, t, v) are QCD_DF64;
+                                own vectors (r, r~, p, q, t, v) are stored
+                                as QCD_DF64;
                              2: QCD_DF64 for all of the outer level.
                              Outer dot products and norms are summed in FP64
                              and the final true residual is FP64 in every
@@ -309,7 +318,8 @@ int qcd_force(qcd_ctx *ctx, const void *U, const void *x, const void *lam, void 
  * sums whole iterations (launches = iterations, their algorithmic bytes).
  * 0 turns timing off.  QCD_EINVAL for other values. */
 typedef enum {
-    QCD_K_MULT_F64 = 0,  /* stencil kernels (MULT, D^, b^, x_o, D), by precision; */
+    QCD_K_MULT_F64 = 0,  /* stencil kernels (MULT, D^, b^, x_o, D), by the precision of the
+                            operator (fixed-point kernels included); */
     QCD_K_MULT_F32 = 1,  /* FP32: all but the second half of D^, which is QCD_K_DHAT_F32 */
     QCD_K_MULT_F16 = 2,
     QCD_K_BLAS = 3,      /* fused BLAS-1 + reduction kernels (all but the FP32 level's) */
@@ -347,7 +357,8 @@ long qcd_launch_count(const qcd_ctx *ctx);
 int qcd_autotune(qcd_ctx *ctx, const char *cache_path);
 
 /* The tuned configurations: up to max entries (key; variant: 0 the
- * compiler's register budget, 1 capped at 80 registers (128 for QCD_DF64),
+ * compiler's register budget, 1 capped at 80 registers (FP32 / FP16; for
+ * QCD_F64 and QCD_DF64 128, without effect on their fixed-point kernels),
  * 2 the FP32 / FP16 kernel whose hops are software-pipelined (the next
  * hop's neighbour spinor and link loaded before the current hop computes);
  * threads per block along the sites, or
