@@ -114,18 +114,18 @@ struct M3 {
 struct AlgX {
     using M = M3x;
     using T = long long;
-    // the link, or its conjugate transpose
-    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu, bool dg)
+    // the link, or its conjugate transpose, its real parts times sr and its
+    // imaginary parts times si
+    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu, bool dg, int sr, int si)
     {
         const int4 *p = (const int4 *)U.a[par];
-        const int sg = dg ? -1 : 1;
         M r;
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const int4 v = __ldg(p + soa(cb, 36, mu * 9 + (dg ? 3 * j + i : 3 * i + j)));
-                r.m[i][j] = fxc{v.x, v.y, v.z * sg, v.w * sg};
+                r.m[i][j] = fxc{v.x * sr, v.y * sr, v.z * si, v.w * si};
             }
         return r;
     }
@@ -134,13 +134,13 @@ struct AlgX {
         fx_mul_elem<false, false>(A, B, i, j, r, s);
     }
     static __device__ __forceinline__ void set(M &A, int i, int j, T r, T s) { A.m[i][j] = fx_unpack(fx_pack(r, s)); }
-    static __device__ __forceinline__ double value(T t) { return (double)t * (1.0 / (double)(1ll << FX_BITS)); }
+    static constexpr double UNIT = 1.0 / (double)(1ll << FX_BITS);
 };
 
 struct AlgD {
     using M = M3;
     using T = double;
-    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu, bool dg)
+    static __device__ __forceinline__ M load(const GaugePtr &U, int par, int cb, int mu, bool dg, int sr, int si)
     {
         const double2 *p = (const double2 *)U.a[par];
         M r;
@@ -149,7 +149,7 @@ struct AlgD {
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const double2 v = __ldg(p + soa(cb, 36, mu * 9 + (dg ? 3 * j + i : 3 * i + j)));
-                r.m[i][j] = mk(v.x, dg ? -v.y : v.y);
+                r.m[i][j] = mk(sr * v.x, si * v.y);
             }
         return r;
     }
@@ -162,14 +162,14 @@ struct AlgD {
         s = z.i;
     }
     static __device__ __forceinline__ void set(M &A, int i, int j, T r, T s) { A.m[i][j] = mk(r, s); }
-    static __device__ __forceinline__ double value(T t) { return t; }
+    static constexpr double UNIT = 1.0;
 };
 
 // F_munu at site n of parity par (coordinates c): the three real diagonal
 // entries, then (re, im) of the entries (1,0), (2,0), (2,1) below it
 template <class Alg>
 __device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U, int par, const int c[4], int mu, int nu,
-                                               double F[9])
+                                               double ck, double F[9])
 {
     using M = typename Alg::M;
     using T = typename Alg::T;
@@ -201,8 +201,8 @@ __device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U,
                 M P;
                 {
                     // X Y: U_nu(n+dm mu [-nu]) (daggered below) times U_mu of the other end
-                    const M X = Alg::load(U, h ? par : op, at(dm, h ? -1 : 0), nu, h);
-                    const M Y = Alg::load(U, k ? par : op, at(k ? -1 : 0, h ? -1 : 1), mu, !k);
+                    const M X = Alg::load(U, h ? par : op, at(dm, h ? -1 : 0), nu, h, 1, h ? -1 : 1);
+                    const M Y = Alg::load(U, k ? par : op, at(k ? -1 : 0, h ? -1 : 1), mu, !k, 1, k ? 1 : -1);
 #pragma unroll
                     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -212,15 +212,16 @@ __device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U,
                             Alg::set(P, i, j, r, s);
                         }
                 }
-                const M A = Alg::load(U, k ? op : par, at(k ? -1 : 0, 0), mu, k);
+                // with the signs of both brackets: dagger in k, minus in k and in h
+                const M A = Alg::load(U, k ? op : par, at(k ? -1 : 0, 0), mu, k, k ^ h ? -1 : 1, h ? -1 : 1);
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
 #pragma unroll
                     for (int j = 0; j < 3; ++j) {
                         T r, s;
                         Alg::elem(A, P, i, j, r, s);
-                        Rr[i][j] += k ? -r : r;
-                        Ri[i][j] += k ? -s : s;
+                        Rr[i][j] += r;
+                        Ri[i][j] += s;
                     }
             }
 #pragma unroll
@@ -228,29 +229,29 @@ __device__ __forceinline__ void field_strength(const Geom &g, const GaugePtr &U,
 #pragma unroll
                 for (int j = 0; j < 3; ++j) Alg::set(R, i, j, Rr[i][j], Ri[i][j]);
         }
-        const M B = Alg::load(U, h ? op : par, at(0, h ? -1 : 0), nu, !h);
+        const M B = Alg::load(U, h ? op : par, at(0, h ? -1 : 0), nu, !h, 1, h ? 1 : -1);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             T r, s;
             Alg::elem(R, B, i, i, r, s);
-            Fd[i] += h ? -s : s;
+            Fd[i] += s;
 #pragma unroll
             for (int j = 0; j < i; ++j) {
                 T r2, s2;
                 Alg::elem(R, B, i, j, r, s);
                 Alg::elem(R, B, j, i, r2, s2);
-                const T dr = r - r2, di = s + s2;
-                Fr[i + j - 1] += h ? -dr : dr;
-                Fi[i + j - 1] += h ? -di : di;
+                Fr[i + j - 1] += r - r2;
+                Fi[i + j - 1] += s + s2;
             }
         }
     }
-    // (K - K^dag)/(8i)
+    // ck (K - K^dag)/(8i)
+    const double f = 0.125 * Alg::UNIT * ck;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        F[i] = 0.25 * Alg::value(Fd[i]);
-        F[3 + 2 * i] = 0.125 * Alg::value(Fi[i]);
-        F[4 + 2 * i] = -0.125 * Alg::value(Fr[i]);
+        F[i] = 2.0 * f * (double)Fd[i];
+        F[3 + 2 * i] = f * (double)Fi[i];
+        F[4 + 2 * i] = -f * (double)Fr[i];
     }
 }
 
@@ -409,9 +410,10 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
 // now (k_field_strength 2.45 ms, issue-bound at 0.45 of a slot per cycle with
 // twelve warps an SM; k_clover_build 1.4 ms, the inverses on the FP64 pipe).
 // Field strengths: thread = (site, plane), blockIdx.y the plane; planes (0,1)
-// (0,2) (0,3) (1,2) (1,3) (2,3).  FS: [plane][9][Vh_pad] doubles of one parity.
+// (0,2) (0,3) (1,2) (1,3) (2,3).  FS: [plane][9][Vh_pad] doubles of one parity,
+// times csw kappa.
 template <class Alg>
-__global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, int par, double *FS)
+__global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, int par, double ck, double *FS)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
     if (cb >= g.Vh) return;
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, i
     int c[4];
     site_coords(g, par, cb, c);
     double f[9];
-    field_strength<Alg>(g, U, par, c, mu, nu, f);
+    field_strength<Alg>(g, U, par, c, mu, nu, ck, f);
 #pragma unroll
     for (int k = 0; k < 9; ++k) FS[((size_t)w * 9 + k) * g.Vh_pad + cb] = f[k];
 }
@@ -427,20 +429,20 @@ __global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, i
 // The chiral block blockIdx.y (0: A_+, gamma5 = +1; 1: A_-) of every site of
 // a parity, assembled from the field strengths, stored, inverted, stored.
 template <bool FX>
-__global__ void __launch_bounds__(128) k_clover_build(Geom g, const double *__restrict__ FS, double ck, CloverOut F,
+__global__ void __launch_bounds__(128) k_clover_build(Geom g, const double *__restrict__ FS, CloverOut F,
                                                       CloverOut Fi, int *bad)
 {
     const int cb = blockIdx.x * blockDim.x + threadIdx.x, blk = blockIdx.y;
     if (cb >= g.Vh) return;
-    const double se = blk == 0 ? -1.0 : 1.0;  // sign of E_l in B_l -+ E_l
     auto fs = [&](int plane, int k) { return __ldg(FS + ((size_t)plane * 9 + k) * g.Vh_pad + cb); };
     // G_l = B_l -+ E_l: B_1 = F_yz, B_2 = -F_xz, B_3 = F_xy, E = F_xt, F_yt, F_zt
     double G1[9], G2[9], G3[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        G1[k] = ck * (fs(3, k) + se * fs(2, k));
-        G2[k] = ck * (se * fs(4, k) - fs(1, k));
-        G3[k] = ck * (fs(0, k) + se * fs(5, k));
+        const double e1 = fs(2, k), e2 = fs(4, k), e3 = fs(5, k);
+        G1[k] = fs(3, k) + (blk ? e1 : -e1);
+        G2[k] = (blk ? e2 : -e2) - fs(1, k);
+        G3[k] = fs(0, k) + (blk ? e3 : -e3);
     }
     auto ent = [](const double G[9], int i, int j) {  // G_ij of the Hermitian G
         if (i == j) return mk(G[i], 0.0);
@@ -496,11 +498,11 @@ int clover_build(qcd_ctx *c, double kappa, double csw)
         const double ck = csw * kappa;
         const CloverOut F = out(c->C, c->Cx, par), Fi = out(c->Ci, c->Cix, par);
         if (c->fx_links) {
-            k_field_strength<AlgX><<<gs, 128, 0, c->stream>>>(c->g, U, par, FS);
-            k_clover_build<true><<<gc, 128, 0, c->stream>>>(c->g, FS, ck, F, Fi, c->flag_dev);
+            k_field_strength<AlgX><<<gs, 128, 0, c->stream>>>(c->g, U, par, ck, FS);
+            k_clover_build<true><<<gc, 128, 0, c->stream>>>(c->g, FS, F, Fi, c->flag_dev);
         } else {
-            k_field_strength<AlgD><<<gs, 128, 0, c->stream>>>(c->g, U, par, FS);
-            k_clover_build<false><<<gc, 128, 0, c->stream>>>(c->g, FS, ck, F, Fi, c->flag_dev);
+            k_field_strength<AlgD><<<gs, 128, 0, c->stream>>>(c->g, U, par, ck, FS);
+            k_clover_build<false><<<gc, 128, 0, c->stream>>>(c->g, FS, F, Fi, c->flag_dev);
         }
         QCD_CUDA_CHECK(cudaGetLastError());
     }
