@@ -75,12 +75,16 @@ typedef enum {
  * FP32 at about 64x its FP64 rate.  Operator calls with QCD_DF64 take
  * complex128 buffers.
  * The operators of QCD_F64 and QCD_DF64 compute in block fixed point on the
- * integer pipe (57-bit components and an exponent per site; norm-wise at least
- * as accurate as FP64 arithmetic) when every loaded link is zero or has a
- * squared Frobenius norm between 0.5 and 3.001 (SU(3): 3); with another link in
- * the field, QCD_F64 computes in FP64 and QCD_DF64 in pairs of floats.  In
- * fixed point a non-finite component makes every component of the sites it
- * reaches NaN. */
+ * integer pipe (57-bit components and an exponent per site) where every loaded
+ * link is close (1/64) to a multiple of a unitary matrix, of squared Frobenius
+ * norm between 0.5 and 3.001 (SU(3): 3), and has no entry below 2^-32.  Their
+ * errors, measured against the norms of the links and vectors, are no larger than
+ * FP64 arithmetic's (SU(3) fields: 1.9e-16 against 2.2e-16 of a MULT); a component
+ * much smaller than the largest of its site or of a neighbour keeps fewer bits
+ * than FP64 would (57, less the binary digits by which it is smaller).  With any
+ * other link in the field, unit, diagonal and zero links among them, QCD_F64
+ * computes in FP64 and QCD_DF64 in pairs of floats.  In fixed point a non-finite
+ * component makes every component of the sites it reaches NaN. */
 typedef enum { QCD_F64 = 0, QCD_F32 = 1, QCD_F16 = 2, QCD_DF64 = 3 } qcd_prec;
 
 /* Create a context for one lattice on the current CUDA device.

@@ -13,7 +13,9 @@
 // the result is sum ah bh + (mid >> 28) in units of 2^56.  Every step is
 // exact integer arithmetic but for that term and the final rounding, about
 // 2^-57 of the largest component of the site: several times less than the FP64
-// forms lose in their chains of roundings (2^-53 of the running sum per FMA).
+// forms lose in their chains of roundings (2^-53 of the running sum per FMA) --
+// against the size of the site, that is: a component 2^-20 of its site's largest
+// keeps 37 bits where FP64 keeps 53.
 #pragma once
 
 #include "qcd_internal.cuh"
@@ -27,9 +29,20 @@ constexpr int FX_LIMB = 28;
 // With it every product of links below stays in range: |A B| <= 3, |A B C| <=
 // 5.2 entry by entry, so that limbs stay below 2^31 and sums below 2^63.
 constexpr float FX_LINK_FRO2 = 3.001f;
-// So do links of a smaller one but zero: a link's entries are rounded to 2^-55,
-// which for norms down to this is no more than FP64's own rounding of a product.
+// Rounding here is relative to the largest entry of a link (2^-55) and of a site
+// (2^-57), FP64's to each term of a sum.  The two agree where a link turns no
+// vector into one much smaller than itself and mixes the colours, so a field keeps
+// the FP64 forms if it has a link that
+//   has a squared norm below this (uniformly small entries, zero links);
 constexpr float FX_LINK_FRO2_MIN = 0.5f;
+//   is further than this from a multiple of a unitary matrix (the rows' squared
+//   norms and products, against their mean squared norm: diag(1, 1e-12, 1), a
+//   small or a dependent row; its action stays within 5 per cent of the mean);
+constexpr float FX_LINK_UNITARY = 1.f / 64;
+//   or has an entry whose square is below this (2^-32: unit, diagonal and block
+//   diagonal links, whose colours stay apart).  A random SU(3) link has one with
+//   a probability of some 1e-18.
+constexpr float FX_LINK_ENTRY2 = 5.4e-20f;
 
 // a += x y as one instruction (written in C the sums are reassociated into
 // products and 64-bit additions, three instructions each)
@@ -86,24 +99,55 @@ __device__ __forceinline__ long long fx_from_unit(double d, int &bad)
     return b < 0 ? -m : m;
 }
 
+// Whether a link, its entries f rounded to FP32, is one that the fixed-point forms
+// take (the constants above; false for NaN)
+__device__ __forceinline__ bool fx_link_ok(const float2 f[9])
+{
+    float n[3], small = 1.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        n[i] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float e = f[3 * i + j].x * f[3 * i + j].x + f[3 * i + j].y * f[3 * i + j].y;
+            n[i] += e;
+            small = fminf(small, e);
+        }
+    }
+    const float fro = n[0] + n[1] + n[2], tol = FX_LINK_UNITARY * fro;
+    bool ok = fro <= FX_LINK_FRO2 && fro >= FX_LINK_FRO2_MIN && small >= FX_LINK_ENTRY2;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        ok = ok && fabsf(3.f * n[i] - fro) <= tol;
+        const int k = i == 2 ? 0 : i + 1;  // row i times row k
+        float re = 0.f, im = 0.f;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float2 a = f[3 * i + j], b = f[3 * k + j];
+            re += a.x * b.x + a.y * b.y;
+            im += a.y * b.x - a.x * b.y;
+        }
+        ok = ok && 9.f * (re * re + im * im) <= tol * tol;
+    }
+    return ok;
+}
+
 // The link m (row by row) as direction mu of site cb; true if it is out of range
 __device__ __forceinline__ bool fx_store_link(const double2 m[9], int4 *ux, int cb, int mu)
 {
-    float fro = 0.f;
     int bad = 0;
-    bool zero = true;
+    float2 f[9];
+#pragma unroll
     for (int k = 0; k < 9; ++k) {
         ux[soa(cb, 36, mu * 9 + k)] = fx_pack(fx_from_unit(m[k].x, bad), fx_from_unit(m[k].y, bad));
-        bool tiny = false;  // below FP32's normal range (above it is bad): no part of the norm
-        float x = f32_int<false>(m[k].x, tiny);
-        if (tiny) x = 0.f;
+        bool tiny = false;  // below FP32's normal range (above it is bad): too small to count
+        f[k].x = f32_int<false>(m[k].x, tiny);
+        if (tiny) f[k].x = 0.f;
         tiny = false;
-        float y = f32_int<false>(m[k].y, tiny);
-        if (tiny) y = 0.f;
-        fro += x * x + y * y;
-        zero = zero && ((__double_as_longlong(m[k].x) | __double_as_longlong(m[k].y)) << 1) == 0;
+        f[k].y = f32_int<false>(m[k].y, tiny);
+        if (tiny) f[k].y = 0.f;
     }
-    return bad || !(fro <= FX_LINK_FRO2) || (!zero && fro < FX_LINK_FRO2_MIN);
+    return bad || !fx_link_ok(f);
 }
 
 // ---------------------------------------------------------------- 3x3 matrices

@@ -1,6 +1,6 @@
 """The fixed-point forms of the FP64 link algebra against the oracle, where
 they can go wrong: ragged and two-site lattices, exact unit links, and links
-too large for the fixed-point range (the FP64 form takes over)."""
+that the fixed-point forms do not take (the FP64 ones take over)."""
 import numpy as np
 import pytest
 
@@ -190,4 +190,76 @@ def test_entries_below_the_normal_range_of_fp32(tiny):
     for s, k in ((0, 1), (0, 2), (1, 0), (1, 1), (1, 2)):  # the components without the diagonal
         # entries of both blocks, each rounded by half a unit, times 2^120 / 2 each
         assert np.abs(got[:, s, k] - want[:, s, k]).max() <= 2.0 ** (120 - 148) + 1e-5 * np.abs(want[:, s, k]).max()
+    ctx.close()
+
+
+def diagonal_links(dims, d, seed):
+    """Links diag(d) with random phases: colours that do not mix."""
+    V = inputs.volume(dims)
+    ph = np.exp(2j * np.pi * np.random.default_rng(seed).random((V, 4, 3)))
+    U = np.zeros((V, 4, 3, 3), np.complex128)
+    U[..., range(3), range(3)] = np.asarray(d) * ph
+    return U
+
+
+@pytest.mark.parametrize("d", [(1.0, 1e-12, 1.0), (1.0, 0.01, 0.7), (1.0, 1.0, 1.0)])
+@pytest.mark.parametrize("prec", [0, 3])
+def test_colours_that_do_not_mix(d, prec):
+    """H and D^ colour by colour, where a colour is small against the others: in
+    the links, or (phases only) in the vector.  All terms of a component carry the
+    same small factor, so its error is a few roundings of its own size."""
+    dims, t_bc, kappa = (6, 2, 4, 10), -1, 0.12
+    tol = {0: 1e-14, 3: 1e-13}[prec]
+    Vh = inputs.volume(dims) // 2
+    U = diagonal_links(dims, d, 314)
+    v = inputs.gaussian_source(dims, 315)[:Vh]
+    if d[1] == 1.0:
+        v = v * np.array([1.0, 2.0 ** -30, 2.0 ** -70])
+    ctx = make_ctx(dims, U, kappa, 0.0, t_bc)
+    inp = torch.from_numpy(v).cuda()
+    out = torch.zeros_like(inp)
+    ctx.dslash_eo(out, inp, 0, 0, prec)
+    got, want = out.cpu().numpy(), oracle.hop_eo(dims, t_bc, U, 0, v)
+    for i in range(3):
+        assert rel(got[..., i], want[..., i]) < tol, i
+    Fi = oracle.invert_sites(oracle.clover_field(dims, U, kappa, 0.0))
+    ctx.dhat(out, inp, prec)
+    got, want = out.cpu().numpy(), oracle.dhat(dims, t_bc, U, Fi, kappa, v)
+    for i in range(3):
+        assert rel(got[..., i], want[..., i]) < tol, i
+    ctx.close()
+
+
+def test_a_large_neighbour_behind_zero_links():
+    """H where a site 1e25 times larger than the others is cut off by zero links."""
+    dims, t_bc = (6, 2, 4, 10), -1
+    Vh = inputs.volume(dims) // 2
+    U = inputs.random_gauge(dims, 0.3, 316)
+    stride = np.cumprod((1,) + dims[:3])
+    U[0] = 0.0
+    for mu in range(4):
+        U[(dims[mu] - 1) * stride[mu], mu] = 0.0  # the link into site 0
+    v = inputs.gaussian_source(dims, 317)[:Vh]
+    v[0] *= 1e25
+    ctx = make_ctx(dims, U, 0.12, 0.0, t_bc)
+    inp = torch.from_numpy(v).cuda()
+    out = torch.zeros_like(inp)
+    ctx.dslash_eo(out, inp, 1, 0, 0)
+    assert rel(out.cpu().numpy(), oracle.hop_eo(dims, t_bc, U, 1, v)) < 1e-14
+    ctx.close()
+
+
+def test_force_at_links_that_do_not_mix_colours():
+    """The clover part of the gradient (csw makes the hopping part negligible)
+    where it is a product of small link entries only."""
+    dims, kappa, csw, t_bc = (6, 2, 4, 10), 0.12, 1e45, -1
+    U = diagonal_links(dims, (1.0, 1e-12, 1.0), 318)
+    U[..., range(3), range(3)] = np.abs(U[..., range(3), range(3)])  # no plaquette phase: F = 1
+    x, lam = inputs.gaussian_source(dims, 319), inputs.gaussian_source(dims, 320)
+    x[..., [0, 2]] = 0.0
+    lam[..., [0, 2]] = 0.0
+    ctx = make_ctx(dims, U, kappa, csw, t_bc)
+    G = torch.zeros(U.shape, dtype=torch.complex128, device="cuda")
+    ctx.force(torch.from_numpy(U).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(lam).cuda(), G)
+    assert rel(G.cpu().numpy(), oracle.link_grad(dims, t_bc, U, kappa, csw, x, lam)) < TOL
     ctx.close()
