@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const do
 #pragma unroll
         for (int j = 0; j < 3; ++j)
             Z.z[par][soa(cb, 108, zi * 9 + 3 * i + j)] = fx_pack((tr[i][j] << up1) >> DN, (tI[i][j] << up1) >> DN);
-    Z.e[(size_t)(zi * 2 + par) * g.Vh_pad + cb] = E == 0 ? FX_ZERO : E == 0x7ff ? FX_NAN : E - (1023 + 54) + DN - up1;
+    Z.e[(size_t)(zi * 2 + par) * g.Vh_pad + cb] = E == 0x7ff ? FX_NAN : E - (1023 + 54) + DN - up1;
 }
 
 // G_mu(m) of the sites of parity blockIdx.z, direction blockIdx.y

@@ -199,9 +199,9 @@ __device__ __forceinline__ fx2 operator+(fx2 a, fx2 b) { return {a.h + b.h, a.l 
 __device__ __forceinline__ fx2 operator-(fx2 a, fx2 b) { return {a.h - b.h, a.l - b.l}; }
 __device__ __forceinline__ fx2 operator-(fx2 a) { return {-a.h, -a.l}; }
 
-// Unit exponents: the value of t is t 2^e.  A zero site has FX_ZERO; a site
-// with an infinite or NaN component has FX_NAN, and so has every result that
-// reads it.
+// Unit exponents: the value of t is t 2^e.  FX_ZERO is below every one of them (a
+// sum of nothing); a site with an infinite or NaN component has FX_NAN, and so
+// has every result that reads it.
 constexpr int FX_ZERO = -100000, FX_NAN = 100000;
 
 // the limbs of a signed t, the low one unsigned (the partner's low limb is
@@ -210,15 +210,24 @@ __device__ __forceinline__ fx2 fx_split(long long t) { return {(int)(t >> FX_LIM
 
 __device__ __forceinline__ int fx_clamp63(int s) { return s > 63 ? 63 : s; }
 
-// a double's exponent field, and its t in units of 2^(E - 1023 - 56) for a site
+// a double's exponent field (zero and denormals: that of the smallest normal
+// number, whose unit they share), and its t in units of 2^(E - 1023 - 56) for a site
 // whose largest exponent field is E (bits below one unit cut off)
-__device__ __forceinline__ int fx_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
+__device__ __forceinline__ int fx_field(double d)
+{
+    const int ex = (__double2hiint(d) >> 20) & 0x7ff;
+    return ex ? ex : 1;
+}
+// the upper word of its mantissa
+__device__ __forceinline__ unsigned fx_mant(int hi)
+{
+    return ((unsigned)hi & 0xfffffu) | ((hi & 0x7ff00000) ? 0x100000u : 0u);
+}
 __device__ __forceinline__ fx2 fx_limbs(double d, int E)
 {
-    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
-    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-    unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << (FX_VBITS - 53);
-    m >>= fx_clamp63(ex ? E - ex : 63);
+    const int hi = __double2hiint(d);
+    unsigned long long m = (((unsigned long long)fx_mant(hi) << 32) | (unsigned)__double2loint(d)) << (FX_VBITS - 53);
+    m >>= fx_clamp63(E - fx_field(d));
     const int sg = (hi >> 31) | 1;
     const fx2 v = fx_split((long long)m);
     return {v.h * sg, v.l * sg};
@@ -227,23 +236,22 @@ __device__ __forceinline__ fx2 fx_limbs(double d, int E)
 // operands stored with balanced limbs)
 __device__ __forceinline__ long long fx_int(double d, int E)
 {
-    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
-    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-    unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 2;
-    m >>= fx_clamp63(ex ? E - ex : 63);
+    const int hi = __double2hiint(d);
+    unsigned long long m = (((unsigned long long)fx_mant(hi) << 32) | (unsigned)__double2loint(d)) << 2;
+    m >>= fx_clamp63(E - fx_field(d));
     return hi < 0 ? -(long long)m : (long long)m;
 }
 // the same for a float pair: field of the leading float, widened
 __device__ __forceinline__ int fx_field(df d)
 {
     const int ex = (__float_as_int(d.hi) >> 23) & 0xff;
-    return ex == 0xff ? 0x7ff : ex ? ex + 896 : 0;
+    return ex == 0xff ? 0x7ff : (ex ? ex : 1) + 896;
 }
 __device__ __forceinline__ long long fx_float(float f, int E)
 {
     const int b = __float_as_int(f), ex = (b >> 23) & 0xff;
-    const long long m = (long long)((b & 0x7fffff) | 0x800000) << (FX_VBITS - 24);
-    const long long t = m >> fx_clamp63(ex ? E - (ex + 896) : 63);
+    const long long m = (long long)((b & 0x7fffff) | (ex ? 0x800000 : 0)) << (FX_VBITS - 24);
+    const long long t = m >> fx_clamp63(E - ((ex ? ex : 1) + 896));
     return b < 0 ? -t : t;
 }
 __device__ __forceinline__ fx2 fx_limbs(df d, int E) { return fx_split(fx_float(d.hi, E) + fx_float(d.lo, E)); }
@@ -261,7 +269,7 @@ __device__ __forceinline__ int fx_from_spinor(const Spinor<T> &p, Spinor<fx2> &o
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int i = 0; i < 3; ++i) o.s[a][i] = cx<fx2>{fx_limbs(p.s[a][i].r, E), fx_limbs(p.s[a][i].i, E)};
-    return E == 0 ? FX_ZERO : E == 0x7ff ? FX_NAN : E - (1023 + FX_VBITS - 1);
+    return E == 0x7ff ? FX_NAN : E - (1023 + FX_VBITS - 1);
 }
 
 // t 2^e in the arithmetic type T

@@ -93,7 +93,7 @@ __device__ __forceinline__ int fx_from_half(const HalfSp<T> &p, HalfSp<fx2> &o)
         o.u[i] = cx<fx2>{fx_limbs(p.u[i].r, E), fx_limbs(p.u[i].i, E)};
         o.d[i] = cx<fx2>{fx_limbs(p.d[i].r, E), fx_limbs(p.d[i].i, E)};
     }
-    return E == 0 ? FX_ZERO : E == 0x7ff ? FX_NAN : E - (1023 + FX_VBITS - 1);
+    return E == 0x7ff ? FX_NAN : E - (1023 + FX_VBITS - 1);
 }
 
 // v scaled below 2^57; e follows

@@ -263,3 +263,46 @@ def test_force_at_links_that_do_not_mix_colours():
     ctx.force(torch.from_numpy(U).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(lam).cuda(), G)
     assert rel(G.cpu().numpy(), oracle.link_grad(dims, t_bc, U, kappa, csw, x, lam)) < TOL
     ctx.close()
+
+
+@pytest.mark.parametrize("scale", [1e-300, 1e-309, 1e-314])
+def test_vectors_near_and_below_the_normal_range(scale):
+    """The FP64 operators keep FP64's denormal values.  Down there each of the oracle's
+    products (48 a component in H, 24 in F^-1) rounds by half a unit of 2^-1074."""
+    dims, kappa, csw, t_bc = (6, 2, 4, 10), 0.12, 1.0, -1
+    Vh = inputs.volume(dims) // 2
+    U = inputs.random_gauge(dims, 0.3, 321)
+    v = scale * inputs.gaussian_source(dims, 322)[:Vh]
+    ctx = make_ctx(dims, U, kappa, csw, t_bc)
+    F = oracle.clover_field(dims, U, kappa, csw)
+    Fi = oracle.invert_sites(F)
+    inp = torch.from_numpy(v).cuda()
+    out = torch.zeros_like(inp)
+    big = 2.0 ** 900  # (norms of denormals would underflow)
+
+    def close(want):
+        err = np.abs(out.cpu().numpy() - want).max()
+        assert err <= 100 * 2.0 ** -1074 + 1e-14 * np.abs(want * big).max() / big
+
+    ctx.dslash_eo(out, inp, 1, 0, 0)
+    close(oracle.hop_eo(dims, t_bc, U, 1, v))
+    ctx.dhat(out, inp, 0)
+    close(oracle.dhat(dims, t_bc, U, Fi, kappa, v))
+    ctx.clover_apply(out, inp, 0, True, 0)
+    close(oracle.site_apply(oracle.field_to_half(dims, 0, Fi), v))
+    ctx.close()
+
+
+def test_force_of_vectors_whose_products_are_denormal():
+    """x and lambda of 1e-155: Y, Z and the gradient are denormal (some 2^40 units of
+    2^-1074), the products behind one entry (hundreds) each rounding by half a unit."""
+    dims, kappa, csw, t_bc = (6, 2, 4, 10), 0.12, 3.0, -1
+    U = inputs.random_gauge(dims, 0.3, 323)
+    x, lam = 1e-155 * inputs.gaussian_source(dims, 324), 1e-155 * inputs.gaussian_source(dims, 325)
+    ctx = make_ctx(dims, U, kappa, csw, t_bc)
+    G = torch.zeros(U.shape, dtype=torch.complex128, device="cuda")
+    ctx.force(torch.from_numpy(U).cuda(), torch.from_numpy(x).cuda(), torch.from_numpy(lam).cuda(), G)
+    want = oracle.link_grad(dims, t_bc, U, kappa, csw, x, lam)
+    assert np.abs(want).max() > 2.0 ** 35 * 2.0 ** -1074
+    assert np.abs(G.cpu().numpy() - want).max() <= 1000 * 2.0 ** -1074
+    ctx.close()
