@@ -140,6 +140,12 @@ __device__ inline void finalize(int op, SolverState *st)
 // warp scheduler's FP64 lanes busy for 64 cycles, and the FP64 tree of a block and
 // of its grid held each fused-dot kernel for some 2 us (two-level solves at one
 // launch shape: 8^4 2.94 -> 2.58 ms, 12^3x24 4.42 -> 3.97, 24^3x48 17.65 -> 17.27).
+// A pair's 2^-48 is far below the 2^-24 of the warp sums that it adds.  Its range is
+// FP32's, so the warp sums enter times 2^-5 (up to 32 a block; exact down to
+// 2^-121) and a grid's sum beyond 3.4e38 is taken again in FP64: only a warp sum
+// itself can leave the range.  (A check for it in every block instead of the
+// factor, against no care for the range: 16^3x32 solves 3.25 / 3.32 ms; the factor:
+// 3.29 / 3.30.)
 template <class A>
 struct WideOf {
     using type = double;
@@ -158,6 +164,21 @@ __device__ __forceinline__ double wide_pack(double v) { return v; }
 __device__ __forceinline__ double wide_pack(df v)
 {
     return __hiloint2double(__float_as_int(v.hi), __float_as_int(v.lo));
+}
+// a warp sum as a term of the block's; a total back to its own scale, and
+// whether it is finite there
+__device__ __forceinline__ double wide_in(double v) { return v; }
+__device__ __forceinline__ df wide_in(float v) { return df(v * 0x1p-5f); }
+__device__ __forceinline__ bool wide_out(double v, double &sum)
+{
+    sum = v;
+    return true;
+}
+__device__ __forceinline__ bool wide_out(df v, double &sum)
+{
+    const df t(v.hi * 0x1p5f, v.lo * 0x1p5f);
+    sum = (double)t;
+    return isfinite(t.hi);
 }
 template <class W>
 __device__ __forceinline__ W wide_unpack(double d)
@@ -209,7 +230,7 @@ __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bi
     if (lane == 0)
 #pragma unroll
         for (int k = 0; k < N; ++k) sh[wid][k] = v[k];
-    const auto mine = [&](int w, int k) { return W(sh[w][k]); };
+    const auto mine = [&](int w, int k) { return wide_in(sh[w][k]); };
     if (bidx != nblk - 1) {
         // Every block but the last: warps 1.. post their sums and leave at
         // once (bar.arrive does not wait; their output stores proceed), warp
@@ -304,8 +325,15 @@ __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bi
     __syncthreads();
     if (wid == 0) {
         const W t = warps_sum<N, W>(nw, [&](int w, int k) { return wide_unpack<W>(sw[w][k]); });
+        double sum;
+        const bool fin = wide_out(t, sum);
+        if constexpr (std::is_same<W, df>::value)
+            if (__any_sync(0xffffffffu, !fin))  // (rare)
+                sum = 32.0 * warps_sum<N, double>(nblk, [&](int b, int k) {
+                          return (double)wide_unpack<W>(__ldcg(ra.partials + (size_t)b * 4 + k));
+                      });
         SolverState *st = (SolverState *)sst;
-        if ((lane & 7) == 0) st->sum[lane >> 3] = (lane >> 3) < N ? (double)t : 0.0;
+        if ((lane & 7) == 0) st->sum[lane >> 3] = (lane >> 3) < N ? sum : 0.0;
         __syncwarp();
         if (lane == 0) finalize(ra.op, st);
         __syncwarp();

@@ -360,3 +360,33 @@ def test_chunk_timing_counts_whole_iterations(lat8):
     assert 4800 < per_site < 5300, per_site
     with pytest.raises(qcd.QCDError):
         ctx.set_profiling(3)
+
+
+@pytest.mark.parametrize("kappa", [1.4e9, 2.3e9])
+@pytest.mark.parametrize("levels", [2, 3])
+def test_inner_sums_beyond_the_range_of_fp32(kappa, levels):
+    """Inner norms above 3.4e38 whose warp sums are below it: |t|^2 of about 2e39 in
+    blocks of 6e37 (kappa 1.4e9), and of 1.5e40 in blocks of 4.5e38 from warps of
+    1.1e38 (2.3e9).  Free field (D = 1 - kappa H, H = 8 on constants, 6 - 2i gamma_x on
+    the plane wave with p_x = pi/2), a source of both modes on the even sites (so
+    that x_o = kappa H x_e has nothing to cancel)."""
+    from paper_1709_08785_gb300 import qcd
+
+    dims = (8, 8, 8, 16)
+    U = inputs.unit_gauge(dims)
+    V = inputs.volume(dims)
+    c = inputs.gaussian_source((2, 2, 2, 2), 60)[:2]
+    x = np.arange(V) % dims[0]
+    b = even_mask(dims)[:, None, None] * (c[0][None] + (1j ** x)[:, None, None] * c[1][None])
+    ctx = qcd.Context(dims, 1)
+    ctx.gauge_load(torch.from_numpy(U).cuda())
+    ctx.clover_build(kappa, 0.0)
+    bd = torch.from_numpy(b).cuda()
+    xd = torch.zeros_like(bd)
+    info = ctx.solve(bd, xd, tol=1e-12, precision_levels=levels)
+    assert info["status"] == 0 and info["restarts"] == 0, info
+    # the inner solves end by their tolerance (as at kappa 1e6), not at a sum that is no number
+    assert info["outer_iters"] <= 2 and info["dhat_applies"][1] <= 14, info
+    F = oracle.clover_field(dims, U, kappa, 0.0)
+    assert oracle.true_residual(dims, 1, U, F, kappa, b, xd.cpu().numpy()) <= 1e-12
+    ctx.close()
