@@ -384,7 +384,6 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
         // FP64 and DF64 operators read fixed-point fields (fx.cuh)
         if (c->fx_links && (prec == QCD_F64 || prec == QCD_DF64) && kind != 3) {
             B.in.prec = B.tmp.prec = QCD_FX;
-            if (kind <= 1) B.out.prec = QCD_FX;
         }
         rc = canon_to_half(c, B.in.prec, f32io, src, -1, B.in, nr, B.stride);
         if (rc) return rc;
@@ -427,7 +426,7 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
             if (s.canon) continue;
         }
         if (rc) return rc;
-        rc = half_to_canon(c, B.out.prec, f32io, B.out, dst, -1, nr, B.stride);
+        rc = half_to_canon(c, prec, f32io, B.out, dst, -1, nr, B.stride);
         if (rc) return rc;
     }
     return QCD_OK;

@@ -244,8 +244,8 @@ struct StencilCall {
     size_t red_pstride = 0;
     bool rhs_grid = false;
     // operator calls without a reduction, FP32, or FP64 / DF64 in fixed point: the
-    // result goes to canonical half vectors (complex64 / complex128, 16-byte
-    // aligned) canon_stride reals apart instead of out
+    // result goes to canonical half vectors (complex64, 16-byte aligned; complex128)
+    // canon_stride reals apart instead of out
     void *canon = nullptr;
     size_t canon_stride = 0;
 };

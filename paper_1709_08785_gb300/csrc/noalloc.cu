@@ -22,9 +22,9 @@ namespace qcd {
 // library holds this array until the process exits.
 constexpr size_t NOALLOC_SCRATCH_BYTES = 24u << 20;
 
-// behind it the two fixed-point exponents per site that the FP64 and DF64
-// operators' fields carry (or the FP16 norms)
-constexpr size_t NOALLOC_NORM_BYTES = NOALLOC_SCRATCH_BYTES / 48;
+// behind it the fixed-point exponent per site that the FP64 and DF64 operators'
+// input carries: 4 bytes for two vectors' 384
+constexpr size_t NOALLOC_NORM_BYTES = NOALLOC_SCRATCH_BYTES / 96;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + NOALLOC_NORM_BYTES];
 
@@ -101,7 +101,8 @@ extern "C" int qcd_dslash_eo_noalloc(qcd_ctx *c, void *out, const void *in, int 
     // FP64 and DF64 hop in fixed point, as in qcd_dslash_eo
     const bool fx = c->fx_links && (prec == QCD_F64 || prec == QCD_DF64);
     HVec vin, vout;
-    vin.prec = vout.prec = fx ? QCD_FX : prec;
+    vin.prec = fx ? QCD_FX : prec;
+    vout.prec = prec;  // (in fixed point the result goes straight to the caller)
     vin.p = base;
     vout.p = (char *)base + hb;
     if (nb) {
@@ -109,7 +110,6 @@ extern "C" int qcd_dslash_eo_noalloc(qcd_ctx *c, void *out, const void *in, int 
         vout.norm = (float *)((char *)base + 2 * hb + nb);
     } else if (fx) {
         vin.norm = (float *)((char *)base + NOALLOC_SCRATCH_BYTES);
-        vout.norm = vin.norm + c->g.Vh_pad;
     }
     // timing events are created on demand by the profiler: keep it off here
     const bool prof = c->profiling;
@@ -130,7 +130,7 @@ extern "C" int qcd_dslash_eo_noalloc(qcd_ctx *c, void *out, const void *in, int 
         }
         rc = launch_stencil(c, s);
     }
-    if (rc == QCD_OK && !s.canon) rc = half_to_canon(c, vout.prec, f32io, vout, out, -1, 1, 0);
+    if (rc == QCD_OK && !s.canon) rc = half_to_canon(c, prec, f32io, vout, out, -1, 1, 0);
     c->profiling = prof;
     return rc;
 }

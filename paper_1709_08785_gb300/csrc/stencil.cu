@@ -66,7 +66,7 @@ bool is_mrhs(const StencilCall &sc)
 bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst)
 {
     const bool fx = c->fx_links && (s.prec == QCD_F64 || s.prec == QCD_DF64);
-    return (fx || s.prec == QCD_F32) && s.red == R_NONE && (uintptr_t)dst % 16 == 0 &&
+    return (fx || (s.prec == QCD_F32 && (uintptr_t)dst % 16 == 0)) && s.red == R_NONE &&
            (s.mode == M_HOP || s.mode == M_MULT || s.mode == M_DHAT || s.mode == M_FULL);
 }
 

@@ -85,12 +85,21 @@ __device__ __forceinline__ void fx_body(const StencilArgs &A)
     if constexpr (MODE == M_RECON) return;
     if (!live) return;
     if constexpr (OUT == TO_CANON) {
-        // 16 bytes a lane; the six stores of a warp cover its 16 sites' 3 KB
-        double2 *o = (double2 *)((double *)A.canon + r * A.canon_stride) + (size_t)cb * 12;
+        // 16 bytes a lane; the six stores of a warp cover its 16 sites' 3 KB.  A
+        // caller's vector off the 16-byte boundary takes the same numbers in halves.
+        double *o = (double *)A.canon + r * A.canon_stride + (size_t)cb * 24;
+        const bool whole = (size_t)A.canon % 16 == 0;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
             const cx<T> z = j < 3 ? v.u[j] : v.d[j - 3];
-            o[fx_comp(a, j / 3, j % 3)] = make_double2(to_d(z.r), to_d(z.i));
+            const double2 d = make_double2(to_d(z.r), to_d(z.i));
+            double *to = o + 2 * fx_comp(a, j / 3, j % 3);
+            if (whole) {
+                *(double2 *)to = d;
+            } else {
+                to[0] = d.x;
+                to[1] = d.y;
+            }
         }
     } else {
         store_half<P>(vec(A.out), cb, a, v);
