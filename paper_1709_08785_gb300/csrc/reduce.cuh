@@ -143,9 +143,9 @@ __device__ inline void finalize(int op, SolverState *st)
 // A pair's 2^-48 is far below the 2^-24 of the warp sums that it adds.  Its range is
 // FP32's, so the warp sums enter times 2^-5 (up to 32 a block; exact down to
 // 2^-121) and a grid's sum beyond 3.4e38 is taken again in FP64: only a warp sum
-// itself can leave the range.  (A check for it in every block instead of the
-// factor, against no care for the range: 16^3x32 solves 3.25 / 3.32 ms; the factor:
-// 3.29 / 3.30.)
+// itself can leave the range.  (Three-level solves at 4^4 and 8^4 with no care for
+// the range 2.62 / 2.23 ms, so 2.63 / 2.21, with the FP64 sum inlined 2.66 / 2.25, with a
+// check in every block instead of the factor 2% more at 16^3x32.)
 template <class A>
 struct WideOf {
     using type = double;
@@ -201,6 +201,21 @@ __device__ __forceinline__ W warps_sum(int nw, const Src &src)
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) t = t + wide_shfl(t, off);
     return t;
+}
+
+// The grid's sums from the float-pair partials in FP64, lanes 8 k .. 8 k + 7 sum k
+// (a function of its own and rolled: inlined, it slowed the path beside it)
+template <int N>
+__device__ __noinline__ double pairs_sum_slow(const double *partials, int nblk)
+{
+    const int lane = threadIdx.x + threadIdx.y * blockDim.x & 31, k = lane >> 3;
+    double t = 0.0;
+    if (k < N)
+#pragma unroll 1
+        for (int b = lane & 7; b < nblk; b += 8) t += (double)wide_unpack<df>(__ldcg(partials + (size_t)b * 4 + k));
+#pragma unroll 1
+    for (int off = 4; off > 0; off >>= 1) t += wide_shfl(t, off);
+    return 32.0 * t;
 }
 
 // Reduce N values over the grid; blocks may be 1-D or 2-D.  The per-thread
@@ -329,9 +344,7 @@ __device__ __forceinline__ void grid_reduce_ex(A v[N], const RedArgs &ra, int bi
         const bool fin = wide_out(t, sum);
         if constexpr (std::is_same<W, df>::value)
             if (__any_sync(0xffffffffu, !fin))  // (rare)
-                sum = 32.0 * warps_sum<N, double>(nblk, [&](int b, int k) {
-                          return (double)wide_unpack<W>(__ldcg(ra.partials + (size_t)b * 4 + k));
-                      });
+                sum = pairs_sum_slow<N>(ra.partials, nblk);
         SolverState *st = (SolverState *)sst;
         if ((lane & 7) == 0) st->sum[lane >> 3] = (lane >> 3) < N ? sum : 0.0;
         __syncwarp();
