@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const do
     const double *y0 = Y + (size_t)plane * 9 * st + (size_t)par * g.Vh_pad + cb;
     const double *y1 = Y + (size_t)plane * 9 * st + (size_t)(1 - par) * g.Vh_pad + up;
     double a[9], b[9];
-    int E = 0;
+    int E = FX_FIELD_MIN<double>;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         a[k] = __ldg(y0 + k * st);

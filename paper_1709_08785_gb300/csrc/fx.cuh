@@ -210,57 +210,54 @@ __device__ __forceinline__ fx2 fx_split(long long t) { return {(int)(t >> FX_LIM
 
 __device__ __forceinline__ int fx_clamp63(int s) { return s > 63 ? 63 : s; }
 
-// a double's exponent field (zero and denormals: that of the smallest normal
-// number, whose unit they share), and its t in units of 2^(E - 1023 - 56) for a site
-// whose largest exponent field is E (bits below one unit cut off)
-__device__ __forceinline__ int fx_field(double d)
+// a double's exponent field, and its t in units of 2^(E - 1023 - 56) for a site
+// whose largest exponent field is E >= 1 (bits below one unit cut off).  Field 0
+// (zero and denormals) has field 1's unit and no leading one.
+__device__ __forceinline__ int fx_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
+template <int UP>  // the mantissa's 53 bits up by UP
+__device__ __forceinline__ unsigned long long fx_mant(double d, int E)
 {
-    const int ex = (__double2hiint(d) >> 20) & 0x7ff;
-    return ex ? ex : 1;
-}
-// the upper word of its mantissa
-__device__ __forceinline__ unsigned fx_mant(int hi)
-{
-    return ((unsigned)hi & 0xfffffu) | ((hi & 0x7ff00000) ? 0x100000u : 0u);
+    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff, one = min(ex, 1);
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | ((unsigned)one << 20);
+    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << UP;
+    return m >> fx_clamp63(E - 1 - ex + one);
 }
 __device__ __forceinline__ fx2 fx_limbs(double d, int E)
 {
-    const int hi = __double2hiint(d);
-    unsigned long long m = (((unsigned long long)fx_mant(hi) << 32) | (unsigned)__double2loint(d)) << (FX_VBITS - 53);
-    m >>= fx_clamp63(E - fx_field(d));
-    const int sg = (hi >> 31) | 1;
-    const fx2 v = fx_split((long long)m);
+    const int sg = (__double2hiint(d) >> 31) | 1;
+    const fx2 v = fx_split((long long)fx_mant<FX_VBITS - 53>(d, E));
     return {v.h * sg, v.l * sg};
 }
 // the same as one signed integer in units of 2^(E - 1023 - 54), |t| < 2^55 (for
 // operands stored with balanced limbs)
 __device__ __forceinline__ long long fx_int(double d, int E)
 {
-    const int hi = __double2hiint(d);
-    unsigned long long m = (((unsigned long long)fx_mant(hi) << 32) | (unsigned)__double2loint(d)) << 2;
-    m >>= fx_clamp63(E - fx_field(d));
-    return hi < 0 ? -(long long)m : (long long)m;
+    const long long m = (long long)fx_mant<2>(d, E);
+    return __double2hiint(d) < 0 ? -m : m;
 }
 // the same for a float pair: field of the leading float, widened
 __device__ __forceinline__ int fx_field(df d)
 {
     const int ex = (__float_as_int(d.hi) >> 23) & 0xff;
-    return ex == 0xff ? 0x7ff : (ex ? ex : 1) + 896;
+    return ex == 0xff ? 0x7ff : ex + 896;
 }
-__device__ __forceinline__ long long fx_float(float f, int E)
+__device__ __forceinline__ long long fx_float(float f, int E)  // E >= 897
 {
-    const int b = __float_as_int(f), ex = (b >> 23) & 0xff;
-    const long long m = (long long)((b & 0x7fffff) | (ex ? 0x800000 : 0)) << (FX_VBITS - 24);
-    const long long t = m >> fx_clamp63(E - ((ex ? ex : 1) + 896));
+    const int b = __float_as_int(f), ex = (b >> 23) & 0xff, one = min(ex, 1);
+    const long long m = (long long)((b & 0x7fffff) | one << 23) << (FX_VBITS - 24);
+    const long long t = m >> fx_clamp63(E - 897 - ex + one);
     return b < 0 ? -t : t;
 }
 __device__ __forceinline__ fx2 fx_limbs(df d, int E) { return fx_split(fx_float(d.hi, E) + fx_float(d.lo, E)); }
+// the least E of an arithmetic type
+template <class T>
+constexpr int FX_FIELD_MIN = std::is_same<T, df>::value ? 897 : 1;
 
 // a spinor in FP64 or DF64 arithmetic as limbs; returns its unit exponent
 template <class T>
 __device__ __forceinline__ int fx_from_spinor(const Spinor<T> &p, Spinor<fx2> &o)
 {
-    int E = 0;
+    int E = FX_FIELD_MIN<T>;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll

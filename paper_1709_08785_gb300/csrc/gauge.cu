@@ -364,7 +364,7 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
 #pragma unroll
     for (int q = 0; q < 18; ++q) p64[soa(cb, 36, blk * 18 + q)] = make_double2(r[2 * q], r[2 * q + 1]);
     if constexpr (FX) {
-        int E = 1;
+        int E = FX_FIELD_MIN<double>;
 #pragma unroll
         for (int k = 0; k < 36; ++k) E = max(E, fx_field(r[k]));
 #pragma unroll

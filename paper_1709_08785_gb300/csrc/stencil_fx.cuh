@@ -81,7 +81,7 @@ __device__ __forceinline__ void store_half(const SpinorPtr &v, int cb, int a, co
 template <class T>
 __device__ __forceinline__ int fx_from_half(const HalfSp<T> &p, HalfSp<fx2> &o)
 {
-    int E = 0;
+    int E = FX_FIELD_MIN<T>;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         E = max(E, max(fx_field(p.u[i].r), fx_field(p.u[i].i)));
