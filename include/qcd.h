@@ -355,17 +355,20 @@ long qcd_launch_count(const qcd_ctx *ctx);
  * fused reduction and right-hand-side count): every candidate is timed on scratch
  * buffers, with L2 evicted, and the fastest kept for this context.  If
  * cache_path is not NULL the choices are read from and added to that JSON
- * file, keyed by device name, lattice extents and configuration, so a later
- * context tunes nothing it finds there.  Needs qcd_clover_build.
+ * file, keyed by device name, lattice extents and configuration (QCD_F64 and
+ * QCD_DF64 in fixed point apart from the same in FP64 and float pairs: a
+ * context that changes between such fields is tuned for each), so a later
+ * context tunes nothing it finds there, unless an entry's shape is one that
+ * the kernel does not have.  Needs qcd_clover_build.
  * Synchronous. */
 int qcd_autotune(qcd_ctx *ctx, const char *cache_path);
 
 /* The tuned configurations: up to max entries (key; variant: 0 the
  * compiler's register budget, 1 capped at 80 registers (FP32 / FP16; for
- * QCD_F64 and QCD_DF64 128, without effect on their fixed-point kernels),
+ * QCD_DF64 128, without effect on the fixed-point kernels),
  * 2 the FP32 / FP16 kernel whose hops are software-pipelined (the next
  * hop's neighbour spinor and link loaded before the current hop computes);
- * threads per block along the sites, or
+ * threads per block along the sites (in fixed point two a site), or
  * right-hand sides per block for the multi-RHS kernel; microseconds per
  * launch); returns the number of entries held. Any output pointer may be
  * NULL. */

@@ -250,7 +250,10 @@ struct StencilCall {
     size_t canon_stride = 0;
 };
 int launch_stencil(qcd_ctx *c, const StencilCall &s);
-unsigned tune_key(const StencilCall &s);
+// precision, mode, reduction, dagger and right-hand sides of a launch, and whether
+// its FP64 or DF64 kernel is the fixed-point one
+constexpr unsigned TUNE_KEY_FX = 1u << 13;
+unsigned tune_key(const qcd_ctx *c, const StencilCall &s);
 // F32 hopping / MULT on several right-hand sides: the shared-memory staged kernel
 bool is_mrhs(const StencilCall &s);
 bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst);  // whether launch_stencil takes s.canon = dst

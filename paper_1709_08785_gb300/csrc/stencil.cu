@@ -37,11 +37,13 @@ static void site_bytes(int prec, double &spinor, double &link, double &clover)
     else { spinor = 52; link = 24; clover = 144; }
 }
 
-unsigned tune_key(const StencilCall &sc)
+static bool runs_fx(const qcd_ctx *c, int prec) { return c->fx_links && (prec == QCD_F64 || prec == QCD_DF64); }
+
+unsigned tune_key(const qcd_ctx *c, const StencilCall &sc)
 {
     const unsigned nr = sc.nrhs < 1 ? 1 : (sc.nrhs > 31 ? 31 : sc.nrhs);
     return (unsigned)sc.prec | ((unsigned)sc.mode << 2) | ((unsigned)sc.red << 5) | ((unsigned)(sc.dagger != 0) << 7) |
-           (nr << 8);
+           (nr << 8) | (runs_fx(c, sc.prec) ? TUNE_KEY_FX : 0u);
 }
 
 double stencil_bytes(const qcd_ctx *c, const StencilCall &sc)
@@ -65,8 +67,7 @@ bool is_mrhs(const StencilCall &sc)
 
 bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst)
 {
-    const bool fx = c->fx_links && (s.prec == QCD_F64 || s.prec == QCD_DF64);
-    return (fx || (s.prec == QCD_F32 && (uintptr_t)dst % 16 == 0)) && s.red == R_NONE &&
+    return (runs_fx(c, s.prec) || (s.prec == QCD_F32 && (uintptr_t)dst % 16 == 0)) && s.red == R_NONE &&
            (s.mode == M_HOP || s.mode == M_MULT || s.mode == M_DHAT || s.mode == M_FULL);
 }
 
@@ -88,7 +89,7 @@ static void default_shape(const qcd_ctx *c, const StencilCall &sc, int &variant,
     if (nrhs > 1) bx = is_mrhs(sc) ? nrhs : nrhs <= 4 ? 64 : 32;
     // fixed point (two threads a site, 168 registers): blocks of 128 threads, three
     // an SM; 256 threads fit once (MULT at 24^3x48 175 / 223 us)
-    if (c->fx_links && (sc.prec == QCD_F64 || sc.prec == QCD_DF64)) {
+    if (runs_fx(c, sc.prec)) {
         bx = nrhs > 1 ? 32 : 64;
         // down to one warp a block while SMs would stay without one
         while (nrhs == 1 && bx > 16 && (int)nblocks(c->g.Vh, bx) < c->num_sms) bx >>= 1;
@@ -104,7 +105,7 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     A.g = c->g;
     const int p = sc.prec;
     // FP64 and DF64 in fixed point where the links allow it
-    A.fx = c->fx_links && (p == QCD_F64 || p == QCD_DF64);
+    A.fx = runs_fx(c, p);
     const int pf = A.fx ? QCD_DF64 : p;  // the precision slot of the fields
     for (int par = 0; par < 2; ++par) {
         A.U.a[par] = pf == QCD_F64 ? c->U64[par] : pf == QCD_F32 ? c->U32[par] : pf == QCD_DF64 ? c->UX[par] : c->U16a[par];
@@ -170,7 +171,7 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
         one.rhs_grid = false;
         int v, b;
         default_shape(c, one, v, b);
-        auto it = c->tune.find(tune_key(one));
+        auto it = c->tune.find(tune_key(c, one));
         if (it != c->tune.end()) {
             v = it->second.variant;
             b = it->second.bx;
@@ -192,14 +193,13 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
         variant = sc.force_variant;
         bx = sc.force_bx;
     } else {
-        auto it = c->tune.find(tune_key(sc));
+        auto it = c->tune.find(tune_key(c, sc));
         if (it != c->tune.end()) {
             variant = it->second.variant;
-            bx = it->second.bx;
+            bx = it->second.bx / (A.fx ? 2 : 1);  // threads a block
         }
     }
     const int cap = A.fx ? 192 : 384;  // sites times right-hand sides of a block (fixed point: two threads each)
-    if (A.fx && bx > 64) bx = 64;  // a tuning cache may hold shapes of other kernels
     if (!is_mrhs(sc) && bx * nrhs > cap) {
         // more right-hand sides than a block of the generic kernels holds:
         // launch them in groups (no reduction spans the groups)

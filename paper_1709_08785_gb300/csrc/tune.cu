@@ -1,13 +1,13 @@
 // Autotuner for the stencil kernels: for each launch configuration the
-// solvers use (precision, mode, fused reduction, dagger, right-hand sides) it
-// times every candidate -- register budget (compiler's / capped at 80 for FP32
-// and FP16; the fixed-point kernels of FP64 and DF64 have one, and 32 or 64
-// sites per block) x threads per block along the sites, or for the
+// solvers use (precision, in fixed point or not, mode, fused reduction, dagger,
+// right-hand sides) it times every candidate -- register budget (compiler's / capped at 80 for FP32
+// and FP16; the fixed-point kernels of FP64 and DF64 have one, and 32, 64 or 128
+// threads per block, two a site) x threads per block along the sites, or for the
 // multi-RHS kernel x right-hand sides per block (the RHS tile) -- on scratch
 // buffers with L2 evicted before each launch, keeps the fastest, and stores
 // the choice in a JSON cache keyed by device name, lattice and configuration.
-// Launches that have no tuned entry use the default (compiler's budget, 128
-// sites per block, all right-hand sides in one block).
+// Launches that have no tuned entry use default_shape (stencil.cu), which is among
+// the candidates.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -64,7 +64,26 @@ std::string cache_prefix(qcd_ctx *c)
 
 // The cache is a JSON object with one entry per line:
 //   "<device>|<Lx>x<Ly>x<Lz>x<Lt>|<key>": [variant, bx, microseconds],
+// with "fx|" before the key of a fixed-point kernel (its own bit of it left out)
 using Cache = std::map<std::string, qcd_ctx::TuneEntry>;
+
+std::string cache_key(const std::string &prefix, unsigned key)
+{
+    return prefix + (key & TUNE_KEY_FX ? "fx|" : "") + std::to_string(key & ~TUNE_KEY_FX);
+}
+
+// Whether a kernel of configuration s has the shape of a cached entry; another (a
+// file written by hand) is timed again.  The kernels exchange values within whole
+// warps and hold 384 threads at most, 256 with pipelined hops, 128 in fixed point.
+bool shape_ok(const qcd_ctx *c, const StencilCall &s, const qcd_ctx::TuneEntry &e)
+{
+    if (e.variant < 0 || e.variant > 2) return false;
+    if (is_mrhs(s)) return e.bx >= 1 && e.bx <= s.nrhs;
+    const bool fx = tune_key(c, s) & TUNE_KEY_FX;
+    const int most = fx ? 128 : e.variant == 2 ? 256 : 384;
+    return e.bx >= 32 && e.bx % 32 == 0 && e.bx <= most / s.nrhs &&
+           (int)nblocks(c->g.Vh, fx ? e.bx / 2 : e.bx) <= c->partial_blocks;
+}
 
 Cache read_cache(const char *path)
 {
@@ -190,14 +209,15 @@ int tune_one(qcd_ctx *c, StencilCall s, qcd_ctx::TuneEntry *out)
     const int nv = mr ? 2 : pipe ? 3 : (low || (s.prec == QCD_DF64 && !c->fx_links)) ? 2 : 1;
     // sites per block; for the multi-RHS kernel the right-hand sides per block
     // (all, a half, a third, a quarter)
-    // (the fixed-point FP64 and DF64 kernels run two threads a site: smaller blocks)
-    const bool fx = c->fx_links && (s.prec == QCD_F64 || s.prec == QCD_DF64);
-    const int bxs1[] = {64, fx ? 32 : 128, 256}, bxsn[] = {32, 64};
+    // (the fixed-point FP64 and DF64 kernels run two threads a site: smaller
+    // blocks, down to the one warp of the default shape on small lattices)
+    const bool fx = in.prec == QCD_FX;
+    const int bxs1[] = {64, fx ? 32 : 128, fx ? 16 : 256}, bxsn[] = {32, 64};
     int bxst[4], nt = 0;
     for (int d : {1, 2, 3, 4})
         if (s.nrhs % d == 0) bxst[nt++] = s.nrhs / d;
     const int *bxs = mr ? bxst : s.nrhs > 1 ? bxsn : bxs1;
-    const int nbx = mr ? nt : s.nrhs > 1 || fx ? 2 : 3;
+    const int nbx = mr ? nt : s.nrhs > 1 ? 2 : 3;
     qcd_ctx::TuneEntry best{0, 128, 1e30};
     // QCD_TUNE_LOG set in the environment: every candidate's time on stderr
     static const bool log = std::getenv("QCD_TUNE_LOG") != nullptr;
@@ -212,8 +232,8 @@ int tune_one(qcd_ctx *c, StencilCall s, qcd_ctx::TuneEntry *out)
             if ((rc = time_candidate(c, s, &us))) return rc;
             if (log)
                 std::fprintf(stderr, "tune prec %d mode %d red %d nrhs %d: variant %d bx %d %.2f us\n", s.prec, s.mode,
-                             s.red, s.nrhs, v, bx, us);
-            if (us < best.us) best = qcd_ctx::TuneEntry{v, bx, us};
+                             s.red, s.nrhs, v, fx ? 2 * bx : bx, us);
+            if (us < best.us) best = qcd_ctx::TuneEntry{v, fx ? 2 * bx : bx, us};
         }
     *out = best;
     return QCD_OK;
@@ -260,10 +280,10 @@ int autotune(qcd_ctx *c, const char *cache_path)
         s.out_par = 0;
         s.a = 1.0;
         s.cc = -c->kappa * c->kappa;
-        const unsigned key = tune_key(s);
-        const std::string ck = prefix + std::to_string(key);
+        const unsigned key = tune_key(c, s);
+        const std::string ck = cache_key(prefix, key);
         auto hit = cache.find(ck);
-        if (hit != cache.end()) {
+        if (hit != cache.end() && shape_ok(c, s, hit->second)) {
             c->tune[key] = hit->second;
             continue;
         }
@@ -284,7 +304,7 @@ int tune_entries(qcd_ctx *c, int max, unsigned *keys, int *variant, int *bx, dou
     int n = 0;
     for (const auto &kv : c->tune) {
         if (n < max) {
-            if (keys) keys[n] = kv.first;
+            if (keys) keys[n] = kv.first & ~TUNE_KEY_FX;
             if (variant) variant[n] = kv.second.variant;
             if (bx) bx[n] = kv.second.bx;
             if (us) us[n] = kv.second.us;

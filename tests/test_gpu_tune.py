@@ -271,3 +271,89 @@ def test_multi_rhs_resident_loop_bit_exact(tmp_path, variant, tile):
                 got = many[0].reshape(Vh, 4, 3)[cbs].astype(np.complex128)
                 assert np.linalg.norm((got - want).ravel()) / np.linalg.norm(want.ravel()) < 2e-6
     ctx.close()
+
+
+def test_cache_entries_belong_to_one_kind_of_links(tmp_path):
+    """FP64 and DF64 launch shapes are tuned apart for links that run in fixed
+    point and for links that do not (1.3 SU(3)): a cache filled with the ones is not
+    read for the others, and a second context finds both."""
+    from paper_1709_08785_gb300 import qcd
+
+    dims = (4, 4, 4, 8)
+    cache = str(tmp_path / "tune.json")
+    U = inputs.random_gauge(dims, 0.25, 120)
+
+    def tune(*scales):
+        ctx = qcd.Context(dims, -1)
+        for s in scales:
+            ctx.gauge_load(torch.from_numpy(s * U).cuda())
+            ctx.clover_build(0.12 / s, 1.0 / s ** 3)
+            ctx.autotune(cache)
+        e = ctx.tune_info()
+        ctx.close()
+        return e
+
+    n = len(tune(1.0))
+    first = json.load(open(cache))
+    wide = sum((int(k.rsplit("|", 1)[1]) & 3) in (0, 3) for k in first)
+    assert len(first) == n and wide > 0
+    tune(1.3)
+    both = json.load(open(cache))
+    assert len(both) == n + wide and all(both[k] == first[k] for k in first)
+    assert len(tune(1.0, 1.3)) == n + wide  # one context that held both fields keeps both
+    assert json.load(open(cache)) == both
+
+
+def test_shapes_that_no_kernel_has_are_timed_again(tmp_path):
+    """A cache written by hand: block sizes that are no whole warps, negative or
+    too large are not used."""
+    from paper_1709_08785_gb300 import qcd
+
+    dims, kappa, csw = (6, 2, 4, 10), 0.124, 1.6
+    cache = str(tmp_path / "tune.json")
+    U = inputs.random_gauge(dims, 0.25, 121)
+
+    def context():
+        ctx = qcd.Context(dims, -1)
+        ctx.gauge_load(torch.from_numpy(U).cuda())
+        ctx.clover_build(kappa, csw)
+        ctx.autotune(cache)
+        return ctx
+
+    context().close()
+    data = json.load(open(cache))
+    for i, k in enumerate(data):
+        data[k] = [data[k][0], (20, -64, 0, 1 << 20, 100, 33)[i % 6], 1.0]
+    with open(cache, "w") as f:
+        f.write("{\n" + ",\n".join('  "%s": [%d, %d, %.3f]' % (k, *e) for k, e in data.items()) + "\n}\n")
+    ctx = context()
+    for e in ctx.tune_info():
+        assert e["threads"] in (1, 2, 3, 4, 6, 12) + (32, 64, 128, 256), e
+    Vh = inputs.volume(dims) // 2
+    v = inputs.gaussian_source(dims, 122)[:Vh]
+    Fi = oracle.invert_sites(oracle.clover_field(dims, U, kappa, csw))
+    want = oracle.dhat(dims, -1, U, Fi, kappa, v)
+    for prec, tol, dt in ((0, 1e-13, torch.complex128), (1, 2e-6, torch.complex64)):
+        out = torch.zeros(v.shape, dtype=dt, device="cuda")
+        ctx.dhat(out, torch.from_numpy(v).to(dt).cuda(), prec)
+        assert np.linalg.norm(out.cpu().numpy() - want) / np.linalg.norm(want) < tol
+    ctx.close()
+
+
+def test_small_lattices_can_keep_the_default_shape(tmp_path):
+    """The fixed-point kernels' candidates reach down to one warp a block, which is
+    the default where larger blocks leave SMs idle (the log lists what was timed)."""
+    import os
+    import subprocess
+    import sys
+
+    code = ("import torch; from paper_1709_08785_gb300 import inputs, qcd\n"
+            "c = qcd.Context((4, 4, 4, 4), -1)\n"
+            "c.gauge_load(torch.from_numpy(inputs.random_gauge((4, 4, 4, 4), 0.25, 123)).cuda())\n"
+            "c.clover_build(0.12, 1.0); c.autotune()\n")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
+                       env=dict(os.environ, QCD_TUNE_LOG="1"), check=True,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    for prec in (0, 3):
+        lines = [ln for ln in r.stderr.splitlines() if ln.startswith("tune prec %d " % prec)]
+        assert {int(ln.split("bx ")[1].split()[0]) for ln in lines} == {32, 64, 128}, lines
