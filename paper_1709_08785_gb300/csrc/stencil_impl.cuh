@@ -142,6 +142,15 @@ __device__ __forceinline__ bool stencil_site(const StencilArgs &A, int cb, int r
     return true;
 }
 
+// The FP32 results of a block's whole warps (blockDim.x is a multiple of 32) to the
+// caller's canonical vector of right-hand side r
+__device__ __forceinline__ void canon_from_block(const StencilArgs &A, int r, int cb, const Spinor<float> &acc)
+{
+    extern __shared__ float4 sm_canon[];
+    const int w = (threadIdx.x + threadIdx.y * blockDim.x) >> 5;
+    canon_store(A.g, (float *)A.canon + r * A.canon_stride, -1, cb, acc, sm_canon + w * SB * (canon_words<float> + 1));
+}
+
 template <int P, int MODE, int RED, bool DAG, bool CANON = false>
 __device__ __forceinline__ void stencil_body(const StencilArgs &A)
 {
@@ -171,11 +180,8 @@ __device__ __forceinline__ void stencil_body(const StencilArgs &A)
     // the output after the partial: the release that publishes the block's
     // partial does not wait for these stores (the next kernel, not the
     // finishing block, reads them)
-    if constexpr (CANON) {  // whole warps: blockDim.x is a multiple of 32
-        extern __shared__ float4 sm_canon[];
-        using TC = float;
-        const int w = (threadIdx.x + threadIdx.y * blockDim.x) >> 5;
-        canon_store(A.g, (TC *)A.canon + r * A.canon_stride, -1, cb, acc, sm_canon + w * SB * (canon_words<TC> + 1));
+    if constexpr (CANON) {
+        canon_from_block(A, r, cb, acc);
         return;
     }
     if (pending) Prec<P>::store(rhs_ptr(A.out, r, A.rhs_stride, A.norm_stride), cb, acc);
@@ -200,7 +206,7 @@ __global__ void __maxnreg__(80) stencil_kernel_r80(StencilArgs A)
 // The pipelined variant (FP32 / FP16, one right-hand side): the hops of
 // hopping_pipe, the clover term from global memory; the compiler's register
 // budget (the prefetched raw data of one hop lives beside the current one)
-template <int P, int MODE, int RED, bool DAG>
+template <int P, int MODE, int RED, bool DAG, bool CANON = false>
 __device__ __forceinline__ void stencil_body_pipe(const StencilArgs &A)
 {
     pdl_enter();
@@ -219,6 +225,10 @@ __device__ __forceinline__ void stencil_body_pipe(const StencilArgs &A)
             A, cb, 0, red, acc, [&](Spinor<float> &a) { hopping_pipe<P, DAG>(A.g, A.U, A.in, A.out_par, cb, a); },
             [&](Spinor<float> &x) { clover_any<P>(A.C, A.out_par, cb, x); }, [](Spinor<float> &) {});
     if constexpr (RED != R_NONE) grid_reduce<RED == R_OMEGA ? 3 : RED == R_DOT_AUX ? 2 : 1>(red, A.red);
+    if constexpr (CANON) {
+        canon_from_block(A, 0, cb, acc);
+        return;
+    }
     if (pending) Prec<P>::store(A.out, cb, acc);
 }
 
@@ -319,6 +329,13 @@ __global__ void __maxnreg__(80) stencil_kernel_canon_r80(StencilArgs A)
     stencil_body<P, MODE, R_NONE, DAG, true>(A);
 }
 
+// (tuned shapes with pipelined hops: MULT call at 24^3x48 72.2 -> 68.9 us)
+template <int P, int MODE, bool DAG>
+__global__ void __launch_bounds__(256) stencil_kernel_canon_pipe(StencilArgs A)
+{
+    if constexpr (P == QCD_F32) stencil_body_pipe<P, MODE, R_NONE, DAG, true>(A);
+}
+
 // ---- host launcher -------------------------------------------------------
 template <int P, int MODE, int RED, bool DAG>
 static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s, int variant)
@@ -327,6 +344,12 @@ static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s
                   (MODE == M_HOP || MODE == M_MULT || MODE == M_DHAT || MODE == M_FULL)) {
         if (A.canon) {
             const size_t sm = (size_t)block.x * block.y * 7 * 16;  // canon_store's words
+            if constexpr (MODE == M_MULT) {  // (the tuner has no entry for the others)
+                if (variant == 2 && block.y == 1 && block.x <= 256) {
+                    launch_pdl(stencil_kernel_canon_pipe<P, MODE, DAG>, grid, block, sm, s, A);
+                    return;
+                }
+            }
             if (variant == 1) launch_pdl(stencil_kernel_canon_r80<P, MODE, DAG>, grid, block, sm, s, A);
             else launch_pdl(stencil_kernel_canon<P, MODE, DAG>, grid, block, sm, s, A);
             return;

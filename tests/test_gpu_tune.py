@@ -357,3 +357,48 @@ def test_small_lattices_can_keep_the_default_shape(tmp_path):
     for prec in (0, 3):
         lines = [ln for ln in r.stderr.splitlines() if ln.startswith("tune prec %d " % prec)]
         assert {int(ln.split("bx ")[1].split()[0]) for ln in lines} == {32, 64, 128}, lines
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("threads", [64, 256])
+def test_tuned_variants_of_an_operator_call(tmp_path, variant, threads):
+    """The FP32 MULT call runs the tuned variant: on an aligned result (written by
+    the kernel) and on one 8 bytes off (through the internal layout) the same bits,
+    plain and daggered, and the oracle's values."""
+    import ctypes
+
+    from paper_1709_08785_gb300 import qcd
+
+    dims, kappa, csw = (6, 2, 4, 10), 0.124, 1.6
+    U = inputs.random_gauge(dims, 0.25, 124)
+    cache = str(tmp_path / "tune.json")
+    for _ in range(2):
+        ctx = qcd.Context(dims, -1)
+        ctx.gauge_load(torch.from_numpy(U).cuda())
+        ctx.clover_build(kappa, csw)
+        ctx.autotune(cache)
+        data = json.load(open(cache))
+        for k in data:
+            key = int(k.rsplit("|", 1)[1])
+            if (key & 3, (key >> 2) & 7, (key >> 5) & 3, key >> 8) == (1, 1, 0, 1):
+                data[k] = [variant, threads, 1.0]
+        with open(cache, "w") as f:
+            f.write("{\n" + ",\n".join('  "%s": [%d, %d, %.3f]' % (k, *e) for k, e in data.items()) + "\n}\n")
+    assert [(e["variant"], e["threads"]) for e in ctx.tune_info()
+            if (e["prec"], e["mode"], e["red"], e["nrhs"]) == (1, 1, 0, 1)] == [(variant, threads)]
+    Vh = inputs.volume(dims) // 2
+    v = inputs.gaussian_source(dims, 125)[:Vh]
+    inp = torch.from_numpy(v).to(torch.complex64).cuda()
+    Fi = oracle.invert_sites(oracle.clover_field(dims, U, kappa, csw))
+    for dag in (0, 1):
+        out = torch.zeros_like(inp)
+        ctx.mult_eo(out, inp, 1, dag, 1, 1)
+        off = torch.zeros(out.numel() + 1, dtype=out.dtype, device="cuda")[1:]
+        assert off.data_ptr() % 16 == 8
+        assert ctx.lib.qcd_mult_eo(ctx._h, ctypes.c_void_p(off.data_ptr()), ctypes.c_void_p(inp.data_ptr()), 1, dag, 1, 1) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(off.view_as(out), out)
+        want = oracle.site_apply(oracle.field_to_half(dims, 1, Fi), oracle.hop_eo(dims, -1, U, 1, v, bool(dag)))
+        got = out.cpu().numpy()
+        assert np.linalg.norm(got - want) / np.linalg.norm(want) < 2e-6
+    ctx.close()
