@@ -166,6 +166,7 @@ struct qcd_ctx {
     // force: the per-site insertion matrices; adjoint solve: gamma5 g
     void *force_buf = nullptr;
     size_t force_bytes = 0;
+    bool force_fp64 = false;  // no room for the fixed-point form
     void *adj_buf = nullptr;
 
     // autotuned launch configurations of the stencil kernels, by tune_key

@@ -593,8 +593,10 @@ int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_can
     const size_t vp = (size_t)c->g.Vh_pad;
     const size_t yx = 54 * 2 * vp * sizeof(double), zx = 2 * vp * 108 * 16, ex = 24 * vp * sizeof(int);
     const size_t y64 = (size_t)c->g.V * 6 * 9 * 16, fx = yx + zx + ex + 2 * vp * 36 * 16;
-    const size_t ybytes = c->fx_links && fx > y64 ? fx : y64;
-    if (c->force_bytes < ybytes) {
+    // Where the device has no room for the fixed-point form's 2784 bytes a site, the
+    // context keeps the FP64 form with its 864.
+    auto hold = [&](size_t bytes) -> int {
+        if (c->force_bytes >= bytes) return QCD_OK;
         if (c->force_buf) {
             cudaStreamSynchronize(c->stream);
             cudaFree(c->force_buf);
@@ -603,12 +605,20 @@ int force(qcd_ctx *c, const void *x, const void *lam, void *G, const void *U_can
             c->force_buf = nullptr;
             c->force_bytes = 0;
         }
-        int rc = dev_alloc(c, &c->force_buf, ybytes);
-        if (rc) return rc;
-        c->force_bytes = ybytes;
+        const int rc = dev_alloc(c, &c->force_buf, bytes);
+        if (rc == QCD_OK) c->force_bytes = bytes;
+        return rc;
+    };
+    int rc = QCD_OK;
+    bool use_fx = c->fx_links && !c->force_fp64;
+    if (use_fx && (rc = hold(fx > y64 ? fx : y64)) == QCD_ENOMEM) {
+        c->force_fp64 = true;
+        use_fx = false;
     }
+    if (!use_fx) rc = hold(y64);
+    if (rc) return rc;
     int *wide = nullptr;
-    if (c->fx_links) {
+    if (use_fx) {
         wide = c->flag_dev + 1;
         QCD_CUDA_CHECK(cudaMemsetAsync(wide, 0, sizeof(int), c->stream));
         double *Y = (double *)c->force_buf;

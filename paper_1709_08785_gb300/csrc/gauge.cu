@@ -405,36 +405,42 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
         }
 }
 
+// Field strengths of the sites [first, end) of one parity, times csw kappa:
+// [plane][9][stride] doubles
+struct FsBuf {
+    double *p;
+    int first, end;
+    size_t stride;
+};
+
 // Both kernels replace one that walked the planes twice per site in FP64 with
 // its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 3.85 ms
 // now (k_field_strength 2.45 ms, issue-bound at 0.45 of a slot per cycle with
 // twelve warps an SM; k_clover_build 1.4 ms, the inverses on the FP64 pipe).
 // Field strengths: thread = (site, plane), blockIdx.y the plane; planes (0,1)
-// (0,2) (0,3) (1,2) (1,3) (2,3).  FS: [plane][9][Vh_pad] doubles of one parity,
-// times csw kappa.
+// (0,2) (0,3) (1,2) (1,3) (2,3).
 template <class Alg>
-__global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, int par, double ck, double *FS)
+__global__ void __launch_bounds__(128, 3) k_field_strength(Geom g, GaugePtr U, int par, double ck, FsBuf FS)
 {
-    const int cb = blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
-    if (cb >= g.Vh) return;
+    const int cb = FS.first + blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
+    if (cb >= FS.end) return;
     const int mu = w < 3 ? 0 : w < 5 ? 1 : 2, nu = w < 3 ? w + 1 : w < 5 ? w - 1 : 3;
     int c[4];
     site_coords(g, par, cb, c);
     double f[9];
     field_strength<Alg>(g, U, par, c, mu, nu, ck, f);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) FS[((size_t)w * 9 + k) * g.Vh_pad + cb] = f[k];
+    for (int k = 0; k < 9; ++k) FS.p[((size_t)w * 9 + k) * FS.stride + (cb - FS.first)] = f[k];
 }
 
-// The chiral block blockIdx.y (0: A_+, gamma5 = +1; 1: A_-) of every site of
-// a parity, assembled from the field strengths, stored, inverted, stored.
+// The chiral block blockIdx.y (0: A_+, gamma5 = +1; 1: A_-) of every one of these
+// sites, assembled from the field strengths, stored, inverted, stored.
 template <bool FX>
-__global__ void __launch_bounds__(128) k_clover_build(Geom g, const double *__restrict__ FS, CloverOut F,
-                                                      CloverOut Fi, int *bad)
+__global__ void __launch_bounds__(128) k_clover_build(FsBuf FS, CloverOut F, CloverOut Fi, int *bad)
 {
-    const int cb = blockIdx.x * blockDim.x + threadIdx.x, blk = blockIdx.y;
-    if (cb >= g.Vh) return;
-    auto fs = [&](int plane, int k) { return __ldg(FS + ((size_t)plane * 9 + k) * g.Vh_pad + cb); };
+    const int cb = FS.first + blockIdx.x * blockDim.x + threadIdx.x, blk = blockIdx.y;
+    if (cb >= FS.end) return;
+    auto fs = [&](int plane, int k) { return __ldg(FS.p + ((size_t)plane * 9 + k) * FS.stride + (cb - FS.first)); };
     // G_l = B_l -+ E_l: B_1 = F_yz, B_2 = -F_xz, B_3 = F_xy, E = F_xt, F_yt, F_zt
     double G1[9], G2[9], G3[9];
 #pragma unroll
@@ -488,24 +494,33 @@ int clover_build(qcd_ctx *c, double kappa, double csw)
     };
     // the field strengths of one parity at a time
     // (the buffer at least as large as the operator calls need it, so that the
-    // first of them does not free it, wait and allocate again)
-    const size_t fs = (size_t)c->g.Vh_pad * 54 * sizeof(double), ops = (size_t)c->g.V * 12 * 16 * 2;
+    // first of them does not free it, wait and allocate again; where the device has
+    // no room for that, of a part of the sites at a time)
+    constexpr size_t SITE = 54 * sizeof(double);
+    int n = c->g.Vh_pad;
+    const size_t fs = n * SITE, ops = (size_t)c->g.V * 12 * 16 * 2;
     int rc = ensure_staging(c, fs > ops ? fs : ops);
-    if (rc) return rc;
-    double *FS = (double *)c->staging;
-    for (int par = 0; par < 2; ++par) {
-        const dim3 gs(nblocks(c->g.Vh, 128), 6), gc(nblocks(c->g.Vh, 128), 2);
-        const double ck = csw * kappa;
-        const CloverOut F = out(c->C, c->Cx, par), Fi = out(c->Ci, c->Cix, par);
-        if (c->fx_links) {
-            k_field_strength<AlgX><<<gs, 128, 0, c->stream>>>(c->g, U, par, ck, FS);
-            k_clover_build<true><<<gc, 128, 0, c->stream>>>(c->g, FS, F, Fi, c->flag_dev);
-        } else {
-            k_field_strength<AlgD><<<gs, 128, 0, c->stream>>>(c->g, U, par, ck, FS);
-            k_clover_build<false><<<gc, 128, 0, c->stream>>>(c->g, FS, F, Fi, c->flag_dev);
-        }
-        QCD_CUDA_CHECK(cudaGetLastError());
+    while (rc == QCD_ENOMEM && n > 128) {
+        n = (n / 2 + 127) / 128 * 128;
+        rc = ensure_staging(c, n * SITE);
     }
+    if (rc) return rc;
+    for (int par = 0; par < 2; ++par)
+        for (int first = 0; first < c->g.Vh; first += n) {
+            const FsBuf FS{(double *)c->staging, first, first + n < c->g.Vh ? first + n : c->g.Vh, (size_t)n};
+            const unsigned nb = nblocks(FS.end - first, 128);
+            const dim3 gs(nb, 6), gc(nb, 2);
+            const double ck = csw * kappa;
+            const CloverOut F = out(c->C, c->Cx, par), Fi = out(c->Ci, c->Cix, par);
+            if (c->fx_links) {
+                k_field_strength<AlgX><<<gs, 128, 0, c->stream>>>(c->g, U, par, ck, FS);
+                k_clover_build<true><<<gc, 128, 0, c->stream>>>(FS, F, Fi, c->flag_dev);
+            } else {
+                k_field_strength<AlgD><<<gs, 128, 0, c->stream>>>(c->g, U, par, ck, FS);
+                k_clover_build<false><<<gc, 128, 0, c->stream>>>(FS, F, Fi, c->flag_dev);
+            }
+            QCD_CUDA_CHECK(cudaGetLastError());
+        }
     int bad = 0;
     QCD_CUDA_CHECK(cudaMemcpyAsync(&bad, c->flag_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     QCD_CUDA_CHECK(cudaStreamSynchronize(c->stream));
