@@ -428,7 +428,7 @@ int canon_to_half(qcd_ctx *c, int prec, int src_is_f32, const void *src, int ful
 {
     ProfScope prof(c, QCD_K_OTHER, 0.0);
     if (src_is_f32) {
-        PREC_SWITCH_FX(prec, (launch_to_half<P, float>(c, (const float *)src, dst, full, nrhs, rhs_stride)); break);
+        PREC_SWITCH(prec, (launch_to_half<P, float>(c, (const float *)src, dst, full, nrhs, rhs_stride)); break);
     } else {
         PREC_SWITCH_FX(prec, (launch_to_half<P, double>(c, (const double *)src, dst, full, nrhs, rhs_stride)); break);
     }
@@ -440,9 +440,9 @@ int half_to_canon(qcd_ctx *c, int prec, int dst_is_f32, HVec src, void *dst, int
 {
     ProfScope prof(c, QCD_K_OTHER, 0.0);
     if (dst_is_f32) {
-        PREC_SWITCH_FX(prec, (launch_to_canon<P, float>(c, src, (float *)dst, full, nrhs, rhs_stride)); break);
+        PREC_SWITCH(prec, (launch_to_canon<P, float>(c, src, (float *)dst, full, nrhs, rhs_stride)); break);
     } else {
-        PREC_SWITCH_FX(prec, (launch_to_canon<P, double>(c, src, (double *)dst, full, nrhs, rhs_stride)); break);
+        PREC_SWITCH(prec, (launch_to_canon<P, double>(c, src, (double *)dst, full, nrhs, rhs_stride)); break);
     }
     QCD_CUDA_CHECK(cudaGetLastError());
     return QCD_OK;

@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const do
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) fx_mul_elem<false, false>(Um, M, i, j, tr[i][j], tI[i][j]);
+        for (int j = 0; j < 3; ++j) fx_mul_elem(Um, M, i, j, tr[i][j], tI[i][j]);
     full(a, M);
     unsigned mh = 0, ml = 0;
 #pragma unroll
@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const do
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             long long r, s;
-            fx_mul_elem<false, false>(M, Um, i, j, r, s);
+            fx_mul_elem(M, Um, i, j, r, s);
             tr[i][j] += r;
             tI[i][j] += s;
             const long long t[2] = {tr[i][j], tI[i][j]};
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(128, 3) k_force_link_x(Geom g, GaugePtr U, For
 #pragma unroll
                     for (int j = 0; j < 3; ++j) {
                         long long r, s;
-                        fx_mul_elem<false, false>(Q, T, i, j, r, s);
+                        fx_mul_elem(Q, T, i, j, r, s);
                         B.m[i][j] = fx_unpack(fx_pack(r, s));
                     }
             }
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(128, 3) k_force_link_x(Geom g, GaugePtr U, For
 #pragma unroll
                 for (int j = 0; j < 3; ++j) {
                     long long r, s;
-                    fx_mul_elem<false, false>(Pm, B, i, j, r, s);
+                    fx_mul_elem(Pm, B, i, j, r, s);
                     r >>= sb;
                     s >>= sb;
                     tr[i][j] = (tr[i][j] >> sa) + (neg ? -r : r);

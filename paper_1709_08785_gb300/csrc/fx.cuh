@@ -156,34 +156,28 @@ struct M3x {
     fxc m[3][3];
 };
 
-// C = op(A) op(B), op = dagger where DA / DB is set, times sgn (+-1); in the
-// operands' scale: t_C = t_A t_B 2^-55.  For entries up to 1 every
+// (A B)_ij in the operands' scale: t_C = t_A t_B 2^-55.  For entries up to 1 every
 // accumulator stays below 2^62 (three complex products, limbs up to 2^29.6
 // after one product of three terms).
-template <bool DA, bool DB>
 __device__ __forceinline__ void fx_mul_elem(const M3x &A, const M3x &B, int i, int j, long long &tr, long long &ti)
 {
     // mid sums start at half a unit of their final shift
     long long mr = 1ll << 26, mi = 1ll << 26, hr = 0, hi = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const fxc a = DA ? A.m[k][i] : A.m[i][k];
-        const fxc b = DB ? B.m[j][k] : B.m[k][j];
-        // (ar + i sa ai)(br + i sb bi)
-        const int aih = DA ? -a.ih : a.ih, ail = DA ? -a.il : a.il;
-        const int bih = DB ? -b.ih : b.ih, bil = DB ? -b.il : b.il;
+        const fxc a = A.m[i][k], b = B.m[k][j];
         fx_mac(mr, a.rh, b.rl);
         fx_mac(mr, a.rl, b.rh);
-        fx_mac(mr, -aih, bil);
-        fx_mac(mr, -ail, bih);
-        fx_mac(mi, a.rh, bil);
-        fx_mac(mi, a.rl, bih);
-        fx_mac(mi, aih, b.rl);
-        fx_mac(mi, ail, b.rh);
+        fx_mac(mr, -a.ih, b.il);
+        fx_mac(mr, -a.il, b.ih);
+        fx_mac(mi, a.rh, b.il);
+        fx_mac(mi, a.rl, b.ih);
+        fx_mac(mi, a.ih, b.rl);
+        fx_mac(mi, a.il, b.rh);
         fx_mac(hr, a.rh, b.rh);
-        fx_mac(hr, -aih, bih);
-        fx_mac(hi, a.rh, bih);
-        fx_mac(hi, aih, b.rh);
+        fx_mac(hr, -a.ih, b.ih);
+        fx_mac(hi, a.rh, b.ih);
+        fx_mac(hi, a.ih, b.rh);
     }
     tr = (hr << 1) + (mr >> 27);
     ti = (hi << 1) + (mi >> 27);
@@ -191,7 +185,7 @@ __device__ __forceinline__ void fx_mul_elem(const M3x &A, const M3x &B, int i, i
 
 // ---------------------------------------------------------------- spinors
 // A real as limbs, with the additions the spin projection needs (limb by limb:
-// the sum of two numbers below 2^55 has limbs below 2^28 and 2^29)
+// the sum of two numbers below 2^57 has limbs up to 2^30 and below 2^29)
 struct fx2 {
     int h, l;
 };
@@ -269,98 +263,9 @@ __device__ __forceinline__ int fx_from_spinor(const Spinor<T> &p, Spinor<fx2> &o
     return E == 0x7ff ? FX_NAN : E - (1023 + FX_VBITS - 1);
 }
 
-// t 2^e in the arithmetic type T
 __device__ __forceinline__ double fx_pow2(int e)  // 2^e; the caller keeps e in the normal range
 {
     return __longlong_as_double((long long)(1023 + e) << 52);
-}
-__device__ __forceinline__ void fx_normalise(const Spinor<long long> &v, int &e, Spinor<long long> &o);
-template <class T>
-__device__ __forceinline__ void fx_to_spinor(const Spinor<long long> &v, int e, Spinor<T> &o)
-{
-    if constexpr (std::is_same<T, df>::value) {
-        // float pairs without the FP64 pipe: the site scaled to 57 bits, the top
-        // 24 exactly and the next 31 rounded to a float
-        Spinor<long long> t;
-        int en = e;
-        fx_normalise(v, en, t);
-        const int es = en + FX_VBITS - 24;
-        if (es > -100 && es < 100) {
-            const float s = __int_as_float((127 + es) << 23), s31 = 4.656612873077392578125e-10f * s;  // 2^-31 s
-            auto conv = [&](long long x) {
-                const float hi = (float)(int)(x >> (FX_VBITS - 24)) * s;
-                const float lo = (float)((int)(x >> (FX_VBITS - 55)) & 0x7fffffff) * s31;
-                return fast_two_sum(hi, lo);
-            };
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) o.s[a][i] = mk(conv(t.s[a][i].r), conv(t.s[a][i].i));
-            return;
-        }
-    }
-    if (e >= FX_NAN / 2) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) o.s[a][i] = mk(T(__longlong_as_double(0x7ff8000000000000ll)), T(__longlong_as_double(0x7ff8000000000000ll)));
-        return;
-    }
-    // below the normal range (sites under 2^-900) in two steps
-    const double s1 = fx_pow2(e < -1000 ? -1000 : e);
-    const double s2 = e >= -1000 ? 1.0 : e < -2000 ? 0.0 : fx_pow2(e + 1000);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            double r = (double)v.s[a][i].r * s1, m = (double)v.s[a][i].i * s1;
-            if (e < -1000) {
-                r *= s2;
-                m *= s2;
-            }
-            o.s[a][i] = mk(T(r), T(m));
-        }
-}
-
-// v scaled below 2^57; e follows
-__device__ __forceinline__ void fx_normalise(const Spinor<long long> &v, int &e, Spinor<long long> &o)
-{
-    unsigned mh = 0, ml = 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const long long c[2] = {v.s[a][i].r, v.s[a][i].i};
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const unsigned h = (unsigned)((unsigned long long)c[k] >> 32), s = (unsigned)((int)h >> 31);
-                mh |= h ^ s;
-                ml |= (unsigned)c[k] ^ s;
-            }
-        }
-    // lz >= 1 leading zeros of the largest magnitude (up to 63 for all zero)
-    const int lz = mh ? __clz(mh) : 32 + min(__clz(ml), 31);
-    const int up = lz - 1;  // the largest to 2^62 or more, then six bits down: below 2^57
-    constexpr int DN = 63 - FX_VBITS;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            o.s[a][i].r = (v.s[a][i].r << up) >> DN;
-            o.s[a][i].i = (v.s[a][i].i << up) >> DN;
-        }
-    if (e > FX_ZERO / 2 && e < FX_NAN / 2) e += DN - up;
-}
-
-// the same, split into limbs
-__device__ __forceinline__ void fx_normalise(const Spinor<long long> &v, int &e, Spinor<fx2> &o)
-{
-    Spinor<long long> t;
-    fx_normalise(v, e, t);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) o.s[a][i] = cx<fx2>{fx_split(t.s[a][i].r), fx_split(t.s[a][i].i)};
 }
 
 // ---------------------------------------------------------------- fields
@@ -379,21 +284,10 @@ __device__ __forceinline__ void fx_store(const SpinorPtr &v, int cb, const Spino
     ((int *)v.norm)[cb] = e;
 }
 
-template <>
+template <>  // written by conversions only; the operators load it themselves (stencil_fx.cuh)
 struct Prec<QCD_FX> {
     using T = double;
     static constexpr int SP_NC = 12;
-    static __device__ __forceinline__ void load(const SpinorPtr &v, int cb, Spinor<T> &s)
-    {
-        const int4 *p = (const int4 *)v.p;
-        Spinor<long long> t;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const int4 q = __ldg(p + soa(cb, 12, k));
-            t.s[k / 3][k % 3] = mk(((long long)q.x << FX_LIMB) + q.y, ((long long)q.z << FX_LIMB) + q.w);
-        }
-        fx_to_spinor(t, __ldg((const int *)v.norm + cb), s);
-    }
     static __device__ __forceinline__ void store(const SpinorPtr &v, int cb, const Spinor<T> &s)
     {
         Spinor<fx2> o;

@@ -131,7 +131,7 @@ struct AlgX {
     }
     static __device__ __forceinline__ void elem(const M &A, const M &B, int i, int j, T &r, T &s)
     {
-        fx_mul_elem<false, false>(A, B, i, j, r, s);
+        fx_mul_elem(A, B, i, j, r, s);
     }
     static __device__ __forceinline__ void set(M &A, int i, int j, T r, T s) { A.m[i][j] = fx_unpack(fx_pack(r, s)); }
     static constexpr double UNIT = 1.0 / (double)(1ll << FX_BITS);

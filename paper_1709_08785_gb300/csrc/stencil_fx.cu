@@ -147,7 +147,7 @@ int dispatch_fx_p(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 b
 }  // namespace
 
 // block.x: two threads a site.  The hopping term and MULT are the same in FP64
-// and DF64; without a canonical target they give fixed-point fields.
+// and DF64: to canonical vectors, or MULT (the first half of D^) to a fixed-point field.
 int dispatch_fx(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s)
 {
 #define QCD_OUT(MODE, DAG, OUT) launch_pdl(fx_kernel<QCD_F64, MODE, R_NONE, DAG, OUT>, grid, block, 0, s, A)
@@ -162,11 +162,11 @@ int dispatch_fx(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 blo
             if (sc.mode == M_MULT) QCD_DIR(M_MULT, TO_CANON);
             QCD_DIR(M_HOP, TO_CANON);
         }
-        if (sc.out.prec == QCD_FX) {
-            if (sc.mode == M_MULT) QCD_DIR(M_MULT, TO_FX);
-            QCD_DIR(M_HOP, TO_FX);
+        if (sc.mode == M_MULT && !sc.dagger && sc.out.prec == QCD_FX) {
+            QCD_OUT(M_MULT, false, TO_FX);
+            return QCD_OK;
         }
-        set_error_message("the FP64 and DF64 hopping terms give fixed-point fields");
+        set_error_message("the FP64 and DF64 hopping terms give canonical vectors, MULT fixed-point fields too");
         return QCD_EINVAL;
     }
     if (sc.dagger) {
