@@ -210,14 +210,15 @@ int tune_one(qcd_ctx *c, StencilCall s, qcd_ctx::TuneEntry *out)
     // sites per block; for the multi-RHS kernel the right-hand sides per block
     // (all, a half, a third, a quarter)
     // (the fixed-point FP64 and DF64 kernels run two threads a site: smaller
-    // blocks, down to the one warp of the default shape on small lattices)
+    // blocks, and on small lattices the one warp of the default shape)
     const bool fx = in.prec == QCD_FX;
+    const bool tiny = fx && (int)nblocks(c->g.Vh, 32) < c->num_sms;
     const int bxs1[] = {64, fx ? 32 : 128, fx ? 16 : 256}, bxsn[] = {32, 64};
     int bxst[4], nt = 0;
     for (int d : {1, 2, 3, 4})
         if (s.nrhs % d == 0) bxst[nt++] = s.nrhs / d;
     const int *bxs = mr ? bxst : s.nrhs > 1 ? bxsn : bxs1;
-    const int nbx = mr ? nt : s.nrhs > 1 ? 2 : 3;
+    const int nbx = mr ? nt : s.nrhs > 1 || (fx && !tiny) ? 2 : 3;
     qcd_ctx::TuneEntry best{0, 128, 1e30};
     // QCD_TUNE_LOG set in the environment: every candidate's time on stderr
     static const bool log = std::getenv("QCD_TUNE_LOG") != nullptr;
