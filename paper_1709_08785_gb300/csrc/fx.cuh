@@ -83,8 +83,8 @@ __device__ __forceinline__ float f32_int(double d, bool &slow)
     return __uint_as_float((zero ? 0u : u) | (hi & 0x80000000u));
 }
 
-// rint-free conversion of a double with |d| <= 1: t = d 2^55 (bits below one
-// unit cut off: 2^-55 absolute, an eighth of a unit in the last place of 1).
+// rint-free conversion of a double with |d| <= 1: t = d 2^55, rounded to nearest
+// (2^-56 absolute, a sixteenth of a unit in the last place of 1).
 // Larger, infinite or NaN values set *bad (links of SU(3) have none).
 __device__ __forceinline__ long long fx_from_unit(double d, int &bad)
 {
@@ -95,7 +95,8 @@ __device__ __forceinline__ long long fx_from_unit(double d, int &bad)
     if (ex == 0) return 0;  // zero and denormals
     long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;  // 2^52 <= m < 2^53
     const int sh = 1023 - ex;                                    // |d| = m 2^(-52 - sh)
-    m = sh >= 0 ? (m << 3) >> (sh > 63 ? 63 : sh) : m << 3;
+    const int s = sh > 63 ? 63 : sh;
+    m = sh > 0 ? ((m << 3) + (1ll << (s - 1))) >> s : m << 3;
     return b < 0 ? -m : m;
 }
 
@@ -208,25 +209,26 @@ __device__ __forceinline__ int fx_clamp63(int s) { return s > 63 ? 63 : s; }
 // whose largest exponent field is E >= 1 (bits below one unit cut off).  Field 0
 // (zero and denormals) has field 1's unit and no leading one.
 __device__ __forceinline__ int fx_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
-template <int UP>  // the mantissa's 53 bits up by UP
+template <int UP, bool ROUND>  // the mantissa's 53 bits up by UP; rounded or cut
 __device__ __forceinline__ unsigned long long fx_mant(double d, int E)
 {
     const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff, one = min(ex, 1);
     const unsigned mh = ((unsigned)hi & 0xfffffu) | ((unsigned)one << 20);
     const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << UP;
-    return m >> fx_clamp63(E - 1 - ex + one);
+    const int s = fx_clamp63(E - 1 - ex + one);
+    return (ROUND ? m + ((1ull << s) >> 1) : m) >> s;
 }
 __device__ __forceinline__ fx2 fx_limbs(double d, int E)
 {
     const int sg = (__double2hiint(d) >> 31) | 1;
-    const fx2 v = fx_split((long long)fx_mant<FX_VBITS - 53>(d, E));
+    const fx2 v = fx_split((long long)fx_mant<FX_VBITS - 53, false>(d, E));
     return {v.h * sg, v.l * sg};
 }
-// the same as one signed integer in units of 2^(E - 1023 - 54), |t| < 2^55 (for
-// operands stored with balanced limbs)
+// the same as one signed integer in units of 2^(E - 1023 - 54), rounded to nearest,
+// |t| <= 2^55 (for operands stored with balanced limbs)
 __device__ __forceinline__ long long fx_int(double d, int E)
 {
-    const long long m = (long long)fx_mant<2>(d, E);
+    const long long m = (long long)fx_mant<2, true>(d, E);
     return __double2hiint(d) < 0 ? -m : m;
 }
 // the same for a float pair: field of the leading float, widened
