@@ -396,6 +396,7 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
             s.rhs_stride = B.stride;
             s.norm_stride = (size_t)c->g.Vh_pad;
             s.dagger = dagger;
+            s.after_pack = true;
             if (kind == 2 || kind == 4) {  // D^ = 1 - kappa^2 H~_eo H~_oe, or S_ee = F_ee D^
                 s.mode = M_MULT;
                 s.out_par = 1;
@@ -403,6 +404,7 @@ int op_half(qcd_ctx *c, void *out, const void *in, int prec, int nrhs, int kind,
                 s.in = B.in;
                 rc = launch_stencil(c, s);
                 if (rc) return rc;
+                s.after_pack = false;
                 s.mode = kind == 4 ? M_FULL : M_DHAT;
                 s.out_par = 0;
                 s.out = B.out;

@@ -13,14 +13,14 @@ namespace qcd {
 
 // Launch with programmatic stream serialization: the kernel (which starts
 // with pdl_enter) may become resident before its predecessor in the stream
-// has finished, and waits on the device for it.
+// has finished, and waits on the device for it.  overlap = false: a plain launch.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                              Args &&...args)
+inline cudaError_t launch_pdl_if(bool overlap, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t s, Args &&...args)
 {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = overlap;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -29,6 +29,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              Args &&...args)
+{
+    return launch_pdl_if(true, kernel, grid, block, smem, s, std::forward<Args>(args)...);
 }
 
 // An internal half-lattice vector in the site-blocked layout.
@@ -249,6 +255,7 @@ struct StencilCall {
     // canon_stride reals apart instead of out
     void *canon = nullptr;
     size_t canon_stride = 0;
+    bool after_pack = false;  // the launch before it is canon_to_half's
 };
 int launch_stencil(qcd_ctx *c, const StencilCall &s);
 // precision, mode, reduction, dagger and right-hand sides of a launch, and whether

@@ -71,12 +71,15 @@ bool canon_out(const qcd_ctx *c, const StencilCall &s, const void *dst)
            (s.mode == M_HOP || s.mode == M_MULT || s.mode == M_DHAT || s.mode == M_FULL);
 }
 
+// the threads that five blocks of 128 an SM hold
+static long one_wave(const qcd_ctx *c) { return 640L * c->num_sms; }
+
 // The launch shape where the tuner has no entry: sites per block (for the
 // multi-RHS kernel the right-hand sides per block) and register budget.
-// FP32 and FP16 with more threads than one wave at the compiler's budget holds
-// (five blocks of 128 an SM): the 80-register kernels, six such blocks.  Solves
-// with every such launch at one shape, budget / 80 registers: 20^3x40 10.43 / 9.98
-// ms, 24^3x48 18.55 / 17.65, FP16 inner level at 40^3x80 104.8 / 96.6.  Below, the
+// FP32 and FP16 with more threads than one wave at the compiler's budget holds: the
+// 80-register kernels, six such blocks.  Solves with every such launch at one shape,
+// budget / 80 registers: 20^3x40 10.43 / 9.98 ms, 24^3x48 18.55 / 17.65, FP16 inner
+// level at 40^3x80 104.8 / 96.6.  Below, the
 // SMs are not full and spills only lengthen the chain: 16^3x32 5.74 / 5.91 ms,
 // 12^3x24 4.42 / 4.54.  Where dot products are fused, 256 sites per block (half
 // the partials of 128) once that leaves most SMs a block: 128 / 256 sites 12^3x24
@@ -95,7 +98,7 @@ static void default_shape(const qcd_ctx *c, const StencilCall &sc, int &variant,
         while (nrhs == 1 && bx > 16 && (int)nblocks(c->g.Vh, bx) < c->num_sms) bx >>= 1;
     }
     const bool low = sc.prec == QCD_F32 || sc.prec == QCD_F16;
-    if (low && !is_mrhs(sc) && (long)c->g.Vh * nrhs > 640L * c->num_sms) variant = 1;
+    if (low && !is_mrhs(sc) && (long)c->g.Vh * nrhs > one_wave(c)) variant = 1;
     if (low && sc.red != R_NONE && c->g.Vh >= 128 * c->num_sms) bx = 256;
 }
 
@@ -149,6 +152,17 @@ int launch_stencil(qcd_ctx *c, const StencilCall &sc)
     A.done = sc.done;
     A.canon = sc.canon;
     A.canon_stride = sc.canon_stride;
+    // A large FP32 or FP16 stencil does not start beside the blocks of the pack before
+    // it: there it took half as long again, and the D^ half behind it too (probably
+    // because an SM that is never empty keeps the split of L1 and shared memory that
+    // the pack's 14 KB a block asked for).  Overlapped / apart, FP32 D^ call: 24^3x48
+    // 144.7 / 106.3 us, 18^3x36 52.4 / 39.0, 16^3x32 35.8 / 30.0 but its MULT call 17.0 / 20.4,
+    // 12^3x24 19.3 / 22.6: from one wave on.  FP16: 24^3x48 87.6 / 81.9, 18^3x36 33.5 / 35.1,
+    // two right-hand sides 40.1 / 42.3 at 16^3x32, 82.3 / 76.1 at 20^3x40: from two waves
+    // of six blocks an SM on.  (FP64 MULT call 24^3x48 228.7 / 230.1.)
+    const long threads = (long)c->g.Vh * A.nrhs;
+    A.apart = sc.after_pack &&
+              ((p == QCD_F32 && threads > one_wave(c)) || (p == QCD_F16 && threads > 2L * 768 * c->num_sms));
     A.done_stride = sc.done_stride;
     A.red_pstride = sc.red_pstride;
     A.skip = nullptr;

@@ -715,6 +715,7 @@ struct StencilArgs {
     size_t red_pstride;   // and its reduction's partials start red.partials + r red_pstride
     void *canon;          // operator calls: the result in canonical half vectors, canon_stride
     size_t canon_stride;  // reals apart, in place of out
+    int apart;            // (host) launched without overlap with its predecessor
 };
 
 // a host-supplied scalar in the kernel's arithmetic type (float: the

@@ -346,34 +346,34 @@ static void launch_t(const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s
             const size_t sm = (size_t)block.x * block.y * 7 * 16;  // canon_store's words
             if constexpr (MODE == M_MULT) {  // (the tuner has no entry for the others)
                 if (variant == 2 && block.y == 1 && block.x <= 256) {
-                    launch_pdl(stencil_kernel_canon_pipe<P, MODE, DAG>, grid, block, sm, s, A);
+                    launch_pdl_if(!A.apart, stencil_kernel_canon_pipe<P, MODE, DAG>, grid, block, sm, s, A);
                     return;
                 }
             }
-            if (variant == 1) launch_pdl(stencil_kernel_canon_r80<P, MODE, DAG>, grid, block, sm, s, A);
-            else launch_pdl(stencil_kernel_canon<P, MODE, DAG>, grid, block, sm, s, A);
+            if (variant == 1) launch_pdl_if(!A.apart, stencil_kernel_canon_r80<P, MODE, DAG>, grid, block, sm, s, A);
+            else launch_pdl_if(!A.apart, stencil_kernel_canon<P, MODE, DAG>, grid, block, sm, s, A);
             return;
         }
     }
     if constexpr (P == QCD_F32 || P == QCD_F16) {
         if (variant == 1) {
-            launch_pdl(stencil_kernel_r80<P, MODE, RED, DAG>, grid, block, 0, s, A);
+            launch_pdl_if(!A.apart, stencil_kernel_r80<P, MODE, RED, DAG>, grid, block, 0, s, A);
             return;
         }
         if constexpr (MODE == M_MULT || MODE == M_DHAT || MODE == M_FULL) {
             if (variant == 2 && block.y == 1 && block.x <= 256) {
-                launch_pdl(stencil_kernel_pipe<P, MODE, RED, DAG>, grid, block, 0, s, A);
+                launch_pdl_if(!A.apart, stencil_kernel_pipe<P, MODE, RED, DAG>, grid, block, 0, s, A);
                 return;
             }
         }
     }
     if constexpr (P == QCD_DF64) {
         if (variant == 1) {
-            launch_pdl(stencil_kernel_r128<P, MODE, RED, DAG>, grid, block, 0, s, A);
+            launch_pdl_if(!A.apart, stencil_kernel_r128<P, MODE, RED, DAG>, grid, block, 0, s, A);
             return;
         }
     }
-    launch_pdl(stencil_kernel<P, MODE, RED, DAG>, grid, block, 0, s, A);
+    launch_pdl_if(!A.apart, stencil_kernel<P, MODE, RED, DAG>, grid, block, 0, s, A);
 }
 
 template <int P>
