@@ -267,8 +267,8 @@ __global__ void k_force_link(Geom g, const double2 *__restrict__ U, const double
 // q = m - nu, + for mu < nu: 8 products a plane instead of 18, and 24 a site for
 // Z.  The hopping part keeps FP64 and uses the projector's rank: with h the
 // two projected spin rows, sum_s ((1-g)lambda)_s conj(x_s) = sum_a h_a(lambda)
-// conj(h_a(x)).  16^3x32: 8.4 ms before, 1.25 ms now (the caller's links
-// into fixed point 0.03, Y 0.19, Z 0.18, links 0.84, issue-bound at half a slot
+// conj(h_a(x)).  16^3x32: 8.4 ms before, 1.27 ms now (the caller's links
+// into fixed point 0.03, Y 0.19, Z 0.20, links 0.84, issue-bound at half a slot
 // per cycle).
 
 // (sigma_p v)_a = ph v[perm]: ph as a power of i (the tables above)

@@ -6,8 +6,8 @@
 // built from three IMAD.WIDE is ten times cheaper than one FP64 FMA.  A
 // number is a signed integer t times a power of two shared by a whole site
 // (spinors, |t| < 2^57; clover blocks, 2^55) or by the field (links, whose
-// entries are at most 1 = 2^55), kept as two limbs, t = h 2^28 + l.  A sum of products keeps two 64-bit
-// accumulators:
+// entries are at most 1 = 2^55), kept as two limbs, t = h 2^28 + l.  A sum of
+// products keeps two 64-bit accumulators:
 //     sum a b = 2^56 sum ah bh + 2^28 sum (ah bl + al bh) + (sum al bl),
 // the last term (below 1/4 unit of the result per product) is dropped, and
 // the result is sum ah bh + (mid >> 28) in units of 2^56.  Every step is
@@ -66,7 +66,8 @@ __device__ __forceinline__ int4 fx_pack(long long r, long long i) { return make_
 // FP64 -> FP32 on the integer pipe: a conversion instruction keeps the two FP64
 // lanes as long as an FMA, and the kernels that build the links and the clover
 // blocks in four precisions waited on those (24^3x48, links 0.28 -> 0.23 ms,
-// clover blocks 0.81 -> 0.70 ms a parity).
+// clover blocks 0.81 -> 0.70 ms a parity; with the links' check and rounding 0.21
+// and 0.73).
 // Rounded to nearest even as (float)d; odd = true: cut off, the last bit set if
 // anything was lost, so that rounding the result to IEEE half equals rounding d.
 // Only for zero and FP32's normal range: *slow is set for anything else.
@@ -92,11 +93,10 @@ __device__ __forceinline__ long long fx_from_unit(double d, int &bad)
     const int hi = (int)(b >> 32);
     const int ex = (hi >> 20) & 0x7ff;
     bad |= (b & 0x7fffffffffffffffll) > __double_as_longlong(1.0 + 1e-9);
-    if (ex == 0) return 0;  // zero and denormals
+    if (ex == 0) return 0;  // zero and denormals (far below a unit)
     long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;  // 2^52 <= m < 2^53
     const int sh = 1023 - ex;                                    // |d| = m 2^(-52 - sh)
-    const int s = sh > 63 ? 63 : sh;
-    m = sh > 0 ? ((m << 3) + (1ll << (s - 1))) >> s : m << 3;
+    m = (((m << 4) >> (sh < 0 ? 0 : sh > 63 ? 63 : sh)) + 1) >> 1;
     return b < 0 ? -m : m;
 }
 
@@ -214,9 +214,9 @@ __device__ __forceinline__ unsigned long long fx_mant(double d, int E)
 {
     const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff, one = min(ex, 1);
     const unsigned mh = ((unsigned)hi & 0xfffffu) | ((unsigned)one << 20);
-    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << UP;
-    const int s = fx_clamp63(E - 1 - ex + one);
-    return (ROUND ? m + ((1ull << s) >> 1) : m) >> s;
+    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << (UP + ROUND);
+    const unsigned long long t = m >> fx_clamp63(E - 1 - ex + one);
+    return ROUND ? (t + 1) >> 1 : t;
 }
 __device__ __forceinline__ fx2 fx_limbs(double d, int E)
 {

@@ -102,7 +102,7 @@ int gauge_convert(qcd_ctx *c, const void *U_dev)
 //   P2  = U_nu(n+mu-nu)^dag U_mu(n-nu)^dag,   P2' = U_nu(n-mu-nu)^dag U_mu(n-mu-nu)
 // (twelve products leaf by leaf).  One loop runs over the four P, daggers taken
 // while loading, so that the code stays within the instruction cache (unrolled,
-// the warps waited on fetches: 1.65 ms a parity at 24^3x48 against 1.22).  The
+// the warps waited on fetches: 1.65 ms a parity at 24^3x48 against 1.22, now 1.16).  The
 // products run in an algebra: AlgX, the fixed-point form of fx.cuh on the
 // integer pipe, whose accumulators hold every product of links with a Frobenius
 // norm up to sqrt(3) (each of SU(3) has exactly that); AlgD, FP64, for fields
@@ -263,7 +263,8 @@ struct Herm6 {
 __device__ __forceinline__ constexpr int tri(int i, int j) { return i * (i - 1) / 2 + j; }
 
 // A -> A^-1 by A = L D L^dag (no pivoting; the clover blocks are close to the
-// identity), all in registers: L, then M = L^-1 over it, then M^dag D^-1 M.
+// identity), in place: L, then M = L^-1 over it, then M^dag D^-1 M.  (The kernel
+// has a frame of 288 bytes in local memory, the 36 reals of a block, without spills.)
 // Returns false on a (near-)zero pivot.
 __device__ __forceinline__ bool herm_inverse6(Herm6 &A)
 {
@@ -414,9 +415,9 @@ struct FsBuf {
 };
 
 // Both kernels replace one that walked the planes twice per site in FP64 with
-// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 3.85 ms
-// now (k_field_strength 2.45 ms, issue-bound at 0.45 of a slot per cycle with
-// twelve warps an SM; k_clover_build 1.4 ms, the inverses on the FP64 pipe).
+// its matrices in local memory: 24^3x48, both parities, 23.5 ms before, 3.8 ms
+// now (k_field_strength 2.3 ms, issue-bound at 0.45 of a slot per cycle with
+// twelve warps an SM; k_clover_build 1.5 ms, the inverses on the FP64 pipe).
 // Field strengths: thread = (site, plane), blockIdx.y the plane; planes (0,1)
 // (0,2) (0,3) (1,2) (1,3) (2,3).
 template <class Alg>
