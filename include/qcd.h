@@ -110,7 +110,8 @@ int qcd_gauge_load(qcd_ctx *ctx, const void *U, int on_device);
  * F_oo are block diagonal and "inverted easily") from the FP64 links (plaquette
  * products in fixed point or FP64, see QCD_DF64; the inverse in FP64), as two
  * 6x6 Hermitian blocks per site in the chiral basis (Sec. III-A), then round
- * them to FP32 and FP16.
+ * them to FP32 and FP16.  The context then holds a buffer of 384 bytes a site (the
+ * operator calls' and host-pointer calls'; less where the device has no room).
  * Errors: QCD_ESTATE without a gauge field; QCD_ECLOVER_SINGULAR if a block
  * has a (near-)zero pivot. */
 int qcd_clover_build(qcd_ctx *ctx, double kappa, double csw);
@@ -196,8 +197,13 @@ typedef struct {
                                 as QCD_DF64;
                              2: QCD_DF64 for all of the outer level.
                              Outer dot products and norms are summed in FP64
-                             and the final true residual is FP64 in every
-                             mode; QCD_EINVAL outside 0..2 */
+                             and the final true residual is taken by the
+                             QCD_F64 operators in every mode: in FP64, or in
+                             fixed point (see QCD_DF64), whose links and
+                             clover blocks differ from the FP64 ones by their
+                             rounding, which moves b - D x by less than
+                             4e-16 |x| (kappa up to 1/8, entries of F below
+                             2); QCD_EINVAL outside 0..2 */
     int eo_hermitian;     /* even_odd = 1: 0 (default) iterates on
                              D^_ee = 1 - kappa^2 F_ee^-1 H_eo F_oo^-1 H_oe
                              (Eq. 8); 1 on the gamma5-hermitian Schur
@@ -255,7 +261,7 @@ int qcd_solve(qcd_ctx *ctx, const void *b, void *x, double tol, const qcd_solve_
  * opts: precision_levels 2, even_odd 1, use_x0 0, outer_df64 0 or 1,
  * eo_hermitian 0 (anything else: QCD_EINVAL); 1 <= nrhs <= 16.  The
  * context keeps a workspace of about 16 FP64 and 7 FP32 half vectors per
- * right-hand side until it is destroyed.  Kernel timing (qcd_set_profiling)
+ * right-hand side, and two in fixed point, until it is destroyed.  Kernel timing (qcd_set_profiling)
  * does not bracket the lockstep second halves of D^.  Returns QCD_OK when
  * every right-hand side converged, else the first failing status (each
  * entry of infos has its own). */
@@ -309,7 +315,11 @@ int qcd_solve_adjoint(qcd_ctx *ctx, const void *g, void *lam, double tol, const 
  * link) and the clover term (the plaquette leaves with the spin-traced
  * insertion Tr_spin[sigma_munu x lam^dag] at each corner) contribute.
  * U: the device gauge field in canonical layout (the one loaded); x, lam:
- * device complex128 [V][4][3]; G: device complex128 [V][4][3][3]. FP64. */
+ * device complex128 [V][4][3]; G: device complex128 [V][4][3][3].  The hopping
+ * part in FP64, the clover part in fixed point where the links allow it (see
+ * QCD_DF64), else in FP64.  The context keeps a workspace of 2784 bytes a site
+ * until it is destroyed (864 where the device has no room for that, or the
+ * loaded links none in fixed point: then all in FP64). */
 int qcd_force(qcd_ctx *ctx, const void *U, const void *x, const void *lam, void *G);
 
 /* Kernel timing.  qcd_set_profiling(ctx, 1): each launch of the operator
