@@ -7,8 +7,8 @@ namespace qcd {
 namespace {
 
 // where the result goes: out in P, out as a fixed-point field, or the caller's
-// canonical complex128 vectors
-enum { TO_P = 0, TO_FX = 1, TO_CANON = 2 };
+// canonical complex128 vectors, on a 16-byte boundary or off it
+enum { TO_P = 0, TO_FX = 1, TO_CANON = 2, TO_CANON8 = 3 };
 
 template <int P, int MODE, int RED, bool DAG, int OUT>
 __device__ __forceinline__ void fx_body(const StencilArgs &A)
@@ -84,21 +84,19 @@ __device__ __forceinline__ void fx_body(const StencilArgs &A)
     if constexpr (RED != R_NONE) grid_reduce<RED == R_OMEGA ? 3 : RED == R_DOT_AUX ? 2 : 1>(red, A.red);
     if constexpr (MODE == M_RECON) return;
     if (!live) return;
-    if constexpr (OUT == TO_CANON) {
-        // 16 bytes a lane; the six stores of a warp cover its 16 sites' 3 KB.  A
-        // caller's vector off the 16-byte boundary takes the same numbers in halves.
+    if constexpr (OUT == TO_CANON || OUT == TO_CANON8) {
+        // 16 bytes a lane; the six stores of a warp cover its 16 sites' 3 KB (off the
+        // 16-byte boundary the same numbers in halves)
         double *o = (double *)A.canon + r * A.canon_stride + (size_t)cb * 24;
-        const bool whole = (size_t)A.canon % 16 == 0;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
             const cx<T> z = j < 3 ? v.u[j] : v.d[j - 3];
-            const double2 d = make_double2(to_d(z.r), to_d(z.i));
             double *to = o + 2 * fx_comp(a, j / 3, j % 3);
-            if (whole) {
-                *(double2 *)to = d;
+            if constexpr (OUT == TO_CANON) {
+                *(double2 *)to = make_double2(to_d(z.r), to_d(z.i));
             } else {
-                to[0] = d.x;
-                to[1] = d.y;
+                to[0] = to_d(z.r);
+                to[1] = to_d(z.i);
             }
         }
     } else {
@@ -151,16 +149,18 @@ int dispatch_fx_p(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 b
 int dispatch_fx(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 block, cudaStream_t s)
 {
 #define QCD_OUT(MODE, DAG, OUT) launch_pdl(fx_kernel<QCD_F64, MODE, R_NONE, DAG, OUT>, grid, block, 0, s, A)
-#define QCD_DIR(MODE, OUT)                        \
-    do {                                          \
-        if (sc.dagger) QCD_OUT(MODE, true, OUT);  \
-        else QCD_OUT(MODE, false, OUT);           \
-        return QCD_OK;                            \
+#define QCD_CANON(MODE, DAG)                                    \
+    do {                                                        \
+        if ((size_t)A.canon % 16) QCD_OUT(MODE, DAG, TO_CANON8); \
+        else QCD_OUT(MODE, DAG, TO_CANON);                      \
+        return QCD_OK;                                          \
     } while (0)
     if (sc.red == R_NONE && (sc.mode == M_HOP || sc.mode == M_MULT)) {
         if (A.canon) {
-            if (sc.mode == M_MULT) QCD_DIR(M_MULT, TO_CANON);
-            QCD_DIR(M_HOP, TO_CANON);
+            if (sc.mode == M_MULT && sc.dagger) QCD_CANON(M_MULT, true);
+            if (sc.mode == M_MULT) QCD_CANON(M_MULT, false);
+            if (sc.dagger) QCD_CANON(M_HOP, true);
+            QCD_CANON(M_HOP, false);
         }
         if (sc.mode == M_MULT && !sc.dagger && sc.out.prec == QCD_FX) {
             QCD_OUT(M_MULT, false, TO_FX);
@@ -173,15 +173,9 @@ int dispatch_fx(const StencilCall &sc, const StencilArgs &A, dim3 grid, dim3 blo
         set_error_message("dagger is only available for the hopping and MULT kernels");
         return QCD_EINVAL;
     }
-    if (A.canon && sc.mode == M_DHAT) {
-        QCD_OUT(M_DHAT, false, TO_CANON);
-        return QCD_OK;
-    }
-    if (A.canon && sc.mode == M_FULL) {
-        QCD_OUT(M_FULL, false, TO_CANON);
-        return QCD_OK;
-    }
-#undef QCD_DIR
+    if (A.canon && sc.mode == M_DHAT) QCD_CANON(M_DHAT, false);
+    if (A.canon && sc.mode == M_FULL) QCD_CANON(M_FULL, false);
+#undef QCD_CANON
 #undef QCD_OUT
     return sc.prec == QCD_DF64 ? dispatch_fx_p<QCD_DF64>(sc, A, grid, block, s)
                                : dispatch_fx_p<QCD_F64>(sc, A, grid, block, s);
