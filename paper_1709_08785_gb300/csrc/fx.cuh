@@ -207,7 +207,9 @@ __device__ __forceinline__ int fx_clamp63(int s) { return s > 63 ? 63 : s; }
 
 // a double's exponent field, and its t in units of 2^(E - 1023 - 56) for a site
 // whose largest exponent field is E >= 1 (bits below one unit cut off).  Field 0
-// (zero and denormals) has field 1's unit and no leading one.
+// (zero and denormals) has field 1's unit and no leading one.  (S_ee calls in FP64 at
+// 16^3x32, with denormals cut to zero / so / with a test a site and a scaling where it
+// matters: 111.4 / 113.7 / 117.5 us; hopping term 42.5 / 42.5 / 45.1.)
 __device__ __forceinline__ int fx_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
 template <int UP, bool ROUND>  // the mantissa's 53 bits up by UP; rounded or cut
 __device__ __forceinline__ unsigned long long fx_mant(double d, int E)
