@@ -18,7 +18,7 @@ namespace qcd {
 // Grid-stride driver: each thread applies op to its sites, reduces NRED
 // doubles over the grid and runs the finaliser.
 template <int NRED, class Op>
-__global__ void __launch_bounds__(256) blas_kernel(int n, Op op, RedArgs red, const int *done, int *skip)
+__device__ __forceinline__ void blas_body(int n, const Op &op, const RedArgs &red, const int *done, int *skip)
 {
     pdl_enter();
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
@@ -31,6 +31,25 @@ __global__ void __launch_bounds__(256) blas_kernel(int n, Op op, RedArgs red, co
     A acc[4] = {A(0), A(0), A(0), A(0)};
     for (int cb = blockIdx.x * blockDim.x + threadIdx.x; cb < n; cb += gridDim.x * blockDim.x) op(cb, acc);
     if constexpr (NRED > 0) grid_reduce<NRED>(acc, red);
+}
+template <int NRED, class Op>
+__global__ void __launch_bounds__(256) blas_kernel(int n, Op op, RedArgs red, const int *done, int *skip)
+{
+    blas_body<NRED>(n, op, red, done, skip);
+}
+// An operation of at most 104 registers (Op104).  How many of a kernel's blocks start
+// beside its predecessor's decides how evenly the small grids of the next kernels
+// spread over the SMs: the conversion to fixed point at the compiler's 105 registers
+// (112 held) instead of 102 (104) slowed the plain FP64 solve at 12x10x10x16 from 9.1
+// to 10.5 ms (and 12^3x16 took 12.3 instead of 13.1).
+template <class Op>
+struct Op104 {
+    static constexpr bool value = false;
+};
+template <int NRED, class Op>
+__global__ void __maxnreg__(104) blas_kernel_r104(int n, Op op, RedArgs red, const int *done, int *skip)
+{
+    blas_body<NRED>(n, op, red, done, skip);
 }
 
 // Blocks of blas_kernel<NRED, Op> resident on one SM (256 threads each),
@@ -71,7 +90,10 @@ static int run(qcd_ctx *c, int nsites, const Op &op, int fin, SolverState *st, c
     ra.st = st;
     ra.op = fin;
     ProfScope prof(c, cls, bytes);
-    launch_pdl(blas_kernel<NRED, Op>, dim3(blocks), dim3(threads), 0, c->stream, nsites, op, ra, done, prof.flag);
+    if constexpr (Op104<Op>::value)
+        launch_pdl(blas_kernel_r104<NRED, Op>, dim3(blocks), dim3(threads), 0, c->stream, nsites, op, ra, done, prof.flag);
+    else
+        launch_pdl(blas_kernel<NRED, Op>, dim3(blocks), dim3(threads), 0, c->stream, nsites, op, ra, done, prof.flag);
     QCD_CUDA_CHECK(cudaGetLastError());
     return QCD_OK;
 }
@@ -505,6 +527,10 @@ struct OpToFx {
         const int e = fx_from_spinor(S, o);
         fx_store(dst, cb, o, e);
     }
+};
+template <int P>
+struct Op104<OpToFx<P>> {
+    static constexpr bool value = true;
 };
 
 int convert_half(qcd_ctx *c, HVec src, HVec dst, const int *done)
