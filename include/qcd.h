@@ -202,7 +202,7 @@ typedef struct {
                              fixed point (see QCD_DF64), whose links and
                              clover blocks differ from the FP64 ones by their
                              rounding, which moves b - D x by less than
-                             4e-16 |x| (kappa up to 1/8, entries of F below
+                             6e-16 |x| (kappa up to 1/8, entries of F below
                              2); QCD_EINVAL outside 0..2 */
     int eo_hermitian;     /* even_odd = 1: 0 (default) iterates on
                              D^_ee = 1 - kappa^2 F_ee^-1 H_eo F_oo^-1 H_oe

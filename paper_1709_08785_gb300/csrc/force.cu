@@ -412,12 +412,12 @@ __global__ void __launch_bounds__(128, 3) k_force_Z(Geom g, GaugePtr U, const do
     auto full = [&](const double v[9], M3x &m) {
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const int4 d = fx_pack(0, fx_int(v[i], E));
+            const int4 d = fx_pack(0, fx_int<true>(v[i], E));
             m.m[i][i] = fx_unpack(d);
 #pragma unroll
             for (int j = 0; j < i; ++j) {
                 const int k = 3 + 2 * (i + j - 1);
-                const int4 o = fx_pack(fx_int(v[k], E), fx_int(v[k + 1], E));
+                const int4 o = fx_pack(fx_int<true>(v[k], E), fx_int<true>(v[k + 1], E));
                 m.m[i][j] = fx_unpack(o);
                 m.m[j][i] = fxc{-o.x, -o.y, o.z, o.w};
             }

@@ -226,11 +226,12 @@ __device__ __forceinline__ fx2 fx_limbs(double d, int E)
     const fx2 v = fx_split((long long)fx_mant<FX_VBITS - 53, false>(d, E));
     return {v.h * sg, v.l * sg};
 }
-// the same as one signed integer in units of 2^(E - 1023 - 54), rounded to nearest,
-// |t| <= 2^55 (for operands stored with balanced limbs)
+// the same as one signed integer in units of 2^(E - 1023 - 54), rounded to nearest or
+// cut, |t| <= 2^55 (for operands stored with balanced limbs)
+template <bool ROUND>
 __device__ __forceinline__ long long fx_int(double d, int E)
 {
-    const long long m = (long long)fx_mant<2, true>(d, E);
+    const long long m = (long long)fx_mant<2, ROUND>(d, E);
     return __double2hiint(d) < 0 ? -m : m;
 }
 // the same for a float pair: field of the leading float, widened

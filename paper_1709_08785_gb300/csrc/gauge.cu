@@ -370,7 +370,8 @@ __device__ __forceinline__ void store_block(const Herm6 &A, int blk, int cb, con
         for (int k = 0; k < 36; ++k) E = max(E, fx_field(r[k]));
 #pragma unroll
         for (int q = 0; q < 18; ++q)
-            ((int4 *)O.x)[soa(cb, 36, blk * 18 + q)] = fx_pack(fx_int(r[2 * q], E), fx_int(r[2 * q + 1], E));
+            // (cut: rounded, the blocks of an 8^4 build took 5 us of 121 longer)
+            ((int4 *)O.x)[soa(cb, 36, blk * 18 + q)] = fx_pack(fx_int<false>(r[2 * q], E), fx_int<false>(r[2 * q + 1], E));
         O.e[2 * cb + blk] = E - (1023 + 54);
     } else {
 #pragma unroll
