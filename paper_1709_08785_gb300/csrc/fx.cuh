@@ -66,8 +66,8 @@ __device__ __forceinline__ int4 fx_pack(long long r, long long i) { return make_
 // FP64 -> FP32 on the integer pipe: a conversion instruction keeps the two FP64
 // lanes as long as an FMA, and the kernels that build the links and the clover
 // blocks in four precisions waited on those (24^3x48, links 0.28 -> 0.23 ms,
-// clover blocks 0.81 -> 0.70 ms a parity; with the links' check and rounding 0.21
-// and 0.73).
+// clover blocks 0.81 -> 0.70 ms a parity; with the links' check and rounding
+// and denormals kept 0.21 and 0.73).
 // Rounded to nearest even as (float)d; odd = true: cut off, the last bit set if
 // anything was lost, so that rounding the result to IEEE half equals rounding d.
 // Only for zero and FP32's normal range: *slow is set for anything else.
